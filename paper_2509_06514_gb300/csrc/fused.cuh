@@ -144,58 +144,89 @@ __device__ __forceinline__ void ks_next(Key4& k, uint32_t rc, uint32_t L) {
 
 // ---- keyed PRF: PRF_p(x) = AES-128 with key p over enc(x) = (x, 0, ..., 0) ----
 
-// Round 1 of both encryptions. State after round 0 is p (x = 0) or p ^ 1 (x = 1): they
-// differ only in byte 0 of column 0, which only output column 0 of round 1 reads.
-__device__ __forceinline__ void keyed_round1(const Blk p, uint32_t L, const Key4& k, Blk& a, Blk& b) {
-    const uint32_t c0 = T<1>(tix(p.y, L, 1)) ^ T<2>(tix(p.z, L, 2)) ^ T<3>(tix(p.w, L, 3)) ^ k.a;
-    a.x = c0 ^ T<0>(tix(p.x, L, 0));
-    b.x = c0 ^ T<0>(tix(p.x ^ 1u, L, 0));
-    a.y = T<0>(tix(p.y, L, 0)) ^ T<1>(tix(p.z, L, 1)) ^ T<2>(tix(p.w, L, 2)) ^ T<3>(tix(p.x, L, 3)) ^ k.b;
-    a.z = T<0>(tix(p.z, L, 0)) ^ T<1>(tix(p.w, L, 1)) ^ T<2>(tix(p.x, L, 2)) ^ T<3>(tix(p.y, L, 3)) ^ k.c;
-    a.w = T<0>(tix(p.w, L, 0)) ^ T<1>(tix(p.x, L, 1)) ^ T<2>(tix(p.y, L, 2)) ^ T<3>(tix(p.z, L, 3)) ^ k.d;
-    b.y = a.y;
-    b.z = a.z;
-    b.w = a.w;
+// SubWord(RotWord(w)) from the four T-table entries of w's bytes (t_b = T<b> of byte b): each entry
+// holds S[byte] twice.
+__device__ __forceinline__ uint32_t sub_rot_of(uint32_t t0, uint32_t t1, uint32_t t2, uint32_t t3) {
+    return __byte_perm(__byte_perm(t1, t2, 0x0042u), __byte_perm(t3, t0, 0x0050u), 0x5410u);
 }
 
-// Both children of parent seed p: PRF_p(0) ^ ca and PRF_p(1) ^ cb (the correction words
-// are folded into the last AddRoundKey).
-__device__ __forceinline__ void keyed_pair(const Blk p, uint32_t L, const Blk ca, const Blk cb, Blk& a, Blk& b) {
-    Key4 k{p.x, p.y, p.z, p.w};
-    ks_next(k, 0x01u, L);
-    keyed_round1(p, L, k, a, b);
-#pragma unroll 2
-    for (int r = 2; r <= 9; ++r) {
-        ks_next(k, c_rcon[r], L);
-        a = aes_round(a, L, k.a, k.b, k.c, k.d);
-        b = aes_round(b, L, k.a, k.b, k.c, k.d);
-    }
-    ks_next(k, 0x36u, L);
-    a = aes_final(a, L, k.a ^ ca.x, k.b ^ ca.y, k.c ^ ca.z, k.d ^ ca.w);
-    b = aes_final(b, L, k.a ^ cb.x, k.b ^ cb.y, k.c ^ cb.z, k.d ^ cb.w);
-}
-
-// lsb of both PRF outputs: rounds 1-8 in full, then only what byte 0 of the output needs:
-// column 0 of round 9 and byte 0 of round 10 (whose round-key byte 0 is
-// rk9.w0.b0 ^ S[rk9.w3.b1] ^ 0x36).
-__device__ __forceinline__ uint32_t keyed_leaf_bits(const Blk p, uint32_t L) {
-    Key4 k{p.x, p.y, p.z, p.w};
-    Blk a, b;
-    ks_next(k, 0x01u, L);
-    keyed_round1(p, L, k, a, b);
+// Rounds 1 and 2 of both encryptions and round keys 1 and 2 (k holds the seed before and round key
+// 2 after). The state after round 0 is p (x = 0) or p ^ 1 (x = 1): the two differ in byte 0 of
+// column 0, which only column 0 of round 1 reads (17 lookups for both, not 32), and after round 1 in
+// column 0, of which each column of round 2 reads one byte (20 lookups, not 32). The first key
+// schedule step substitutes p.w, whose four bytes round 1 has looked up. Against two separate
+// rounds 2 and a separate first key step, 16 of 345 lookups of a node pair and of 288 of a leaf
+// pair less.
+__device__ __forceinline__ void keyed_rounds12(const Blk p, uint32_t L, Key4& k, Blk& a, Blk& b) {
+    const uint32_t w0 = T<0>(tix(p.w, L, 0)), w1 = T<1>(tix(p.w, L, 1)), w2 = T<2>(tix(p.w, L, 2)),
+                   w3 = T<3>(tix(p.w, L, 3));
+    k.a ^= sub_rot_of(w0, w1, w2, w3) ^ 0x01u;
+    k.b ^= k.a;
+    k.c ^= k.b;
+    k.d ^= k.c;
+    const uint32_t c0 = T<1>(tix(p.y, L, 1)) ^ T<2>(tix(p.z, L, 2)) ^ w3 ^ k.a;
+    const uint32_t ax = c0 ^ T<0>(tix(p.x, L, 0));
+    const uint32_t bx = c0 ^ T<0>(tix(p.x ^ 1u, L, 0));
+    const uint32_t y = T<0>(tix(p.y, L, 0)) ^ T<1>(tix(p.z, L, 1)) ^ w2 ^ T<3>(tix(p.x, L, 3)) ^ k.b;
+    const uint32_t z = T<0>(tix(p.z, L, 0)) ^ w1 ^ T<2>(tix(p.x, L, 2)) ^ T<3>(tix(p.y, L, 3)) ^ k.c;
+    const uint32_t w = w0 ^ T<1>(tix(p.x, L, 1)) ^ T<2>(tix(p.y, L, 2)) ^ T<3>(tix(p.z, L, 3)) ^ k.d;
     ks_next(k, 0x02u, L);
-    a = aes_round(a, L, k.a, k.b, k.c, k.d);
-    b = aes_round(b, L, k.a, k.b, k.c, k.d);
+    const uint32_t sx = T<1>(tix(y, L, 1)) ^ T<2>(tix(z, L, 2)) ^ T<3>(tix(w, L, 3)) ^ k.a;
+    a.x = sx ^ T<0>(tix(ax, L, 0));
+    b.x = sx ^ T<0>(tix(bx, L, 0));
+    const uint32_t sy = T<0>(tix(y, L, 0)) ^ T<1>(tix(z, L, 1)) ^ T<2>(tix(w, L, 2)) ^ k.b;
+    a.y = sy ^ T<3>(tix(ax, L, 3));
+    b.y = sy ^ T<3>(tix(bx, L, 3));
+    const uint32_t sz = T<0>(tix(z, L, 0)) ^ T<1>(tix(w, L, 1)) ^ T<3>(tix(y, L, 3)) ^ k.c;
+    a.z = sz ^ T<2>(tix(ax, L, 2));
+    b.z = sz ^ T<2>(tix(bx, L, 2));
+    const uint32_t sw = T<0>(tix(w, L, 0)) ^ T<2>(tix(y, L, 2)) ^ T<3>(tix(z, L, 3)) ^ k.d;
+    a.w = sw ^ T<1>(tix(ax, L, 1));
+    b.w = sw ^ T<1>(tix(bx, L, 1));
+}
+
+// Rounds 1-8 of both encryptions (k: round key 8 after). Node pairs and leaf pairs share them, and a
+// subtree walk runs both through one copy of this code: the walk's instructions decide how well the
+// instruction caches feed the warps.
+__device__ __forceinline__ void keyed_rounds18(const Blk p, uint32_t L, Key4& k, Blk& a, Blk& b) {
+    k = {p.x, p.y, p.z, p.w};
+    keyed_rounds12(p, L, k, a, b);
 #pragma unroll 2
     for (int r = 3; r <= 8; ++r) {
         ks_next(k, c_rcon[r], L);
         a = aes_round(a, L, k.a, k.b, k.c, k.d);
         b = aes_round(b, L, k.a, k.b, k.c, k.d);
     }
+}
+
+// Rounds 9 and 10 of a node pair: PRF_p(0) ^ ca and PRF_p(1) ^ cb (the correction words are folded
+// into the last AddRoundKey).
+__device__ __forceinline__ void keyed_pair_tail(uint32_t L, Key4 k, const Blk ca, const Blk cb, Blk& a, Blk& b) {
     ks_next(k, 0x1bu, L);
-    const uint32_t a9 = aes_round_col0(a, L, k.a);
-    const uint32_t b9 = aes_round_col0(b, L, k.a);
-    const uint32_t kbit = (k.a ^ sbox0_lsb(k.d >> 8, L)) & 1u;  // lsb(0x36) = 0
+    a = aes_round(a, L, k.a, k.b, k.c, k.d);
+    b = aes_round(b, L, k.a, k.b, k.c, k.d);
+    ks_next(k, 0x36u, L);
+    a = aes_final(a, L, k.a ^ ca.x, k.b ^ ca.y, k.c ^ ca.z, k.d ^ ca.w);
+    b = aes_final(b, L, k.a ^ cb.x, k.b ^ cb.y, k.c ^ cb.z, k.d ^ cb.w);
+}
+
+// Both children of parent seed p.
+__device__ __forceinline__ void keyed_pair(const Blk p, uint32_t L, const Blk ca, const Blk cb, Blk& a, Blk& b) {
+    Key4 k;
+    keyed_rounds18(p, L, k, a, b);
+    keyed_pair_tail(L, k, ca, cb, a, b);
+}
+
+// lsb of both PRF outputs after round 8: only what byte 0 of the output needs, byte 0 of column 0 of
+// round 9 and of round 10, whose round-key bytes take three of the last two key steps' eight
+// substitutions (rk9.w0 bytes 0 and 1; rk10.w0.b0 = rk9.w0.b0 ^ S[rk9.w3.b1] ^ 0x36).
+__device__ __forceinline__ uint32_t keyed_leaf_bits_tail(uint32_t L, const Key4& k, const Blk a, const Blk b) {
+    // bytes 0 and 1 of rk9.w0 (S[rk8.w3.b1] in byte 0 of T<2>, S[rk8.w3.b2] in byte 1 of T<3>)
+    const uint32_t k9 = k.a ^ __byte_perm(T<2>(tix(k.d, L, 1)), T<3>(tix(k.d, L, 2)), 0x0050u) ^ 0x1bu;
+    const uint32_t a9 = aes_round_col0(a, L, k9);
+    const uint32_t b9 = aes_round_col0(b, L, k9);
+    const uint32_t d9 = k.d ^ k.c ^ k.b ^ k9;  // byte 1: rk9.w3.b1
+    const uint32_t kbit = (k9 ^ T<2>(tix(d9, L, 1))) & 1u;  // lsb(0x36) = 0
     return ((sbox0_lsb(a9, L) ^ kbit) & 1u) | (((sbox0_lsb(b9, L) ^ kbit) & 1u) << 1);
 }
 
@@ -213,14 +244,14 @@ __device__ __forceinline__ Blk keyed_one(const Blk p, uint32_t x, uint32_t L) {
 }
 
 // Word 0 (output bytes 0..3) of both PRF outputs: rounds 1-9 in full, then only column 0
-// of round 10 (the additive answer's shares are the leaves' low 32 bits).
+// of round 10 (the additive answer's shares are the leaves' low 32 bits). The loop is rolled:
+// unrolled by two the additive walk measured 3.7 % slower.
 __device__ __forceinline__ void keyed_leaf_words(const Blk p, uint32_t L, uint32_t& wa, uint32_t& wb) {
     Key4 k{p.x, p.y, p.z, p.w};
     Blk a, b;
-    ks_next(k, 0x01u, L);
-    keyed_round1(p, L, k, a, b);
+    keyed_rounds12(p, L, k, a, b);
 #pragma unroll 1
-    for (int r = 2; r <= 9; ++r) {
+    for (int r = 3; r <= 9; ++r) {
         ks_next(k, c_rcon[r], L);
         a = aes_round(a, L, k.a, k.b, k.c, k.d);
         b = aes_round(b, L, k.a, k.b, k.c, k.d);
@@ -234,28 +265,34 @@ __device__ __forceinline__ void keyed_leaf_words(const Blk p, uint32_t L, uint32
 
 // ---- MMO PRF: PRF_p(x) = AES_{K_x}(p) ^ p with fixed round keys rk[x][44] ----
 
-__device__ __forceinline__ void mmo_pair(const Blk p, uint32_t L, const uint32_t (&rk)[2][44], const Blk ca,
-                                         const Blk cb, Blk& a, Blk& b) {
+// Rounds 1-8 under both keys.
+__device__ __forceinline__ void mmo_rounds18(const Blk p, uint32_t L, const uint32_t (&rk)[2][44], Blk& a, Blk& b) {
     a = {p.x ^ rk[0][0], p.y ^ rk[0][1], p.z ^ rk[0][2], p.w ^ rk[0][3]};
     b = {p.x ^ rk[1][0], p.y ^ rk[1][1], p.z ^ rk[1][2], p.w ^ rk[1][3]};
-#pragma unroll 1
-    for (int r = 1; r <= 9; ++r) {
+#pragma unroll 2
+    for (int r = 1; r <= 8; ++r) {
         a = aes_round(a, L, rk[0][4 * r], rk[0][4 * r + 1], rk[0][4 * r + 2], rk[0][4 * r + 3]);
         b = aes_round(b, L, rk[1][4 * r], rk[1][4 * r + 1], rk[1][4 * r + 2], rk[1][4 * r + 3]);
     }
+}
+
+__device__ __forceinline__ void mmo_pair_tail(const Blk p, uint32_t L, const uint32_t (&rk)[2][44], const Blk ca,
+                                              const Blk cb, Blk& a, Blk& b) {
+    a = aes_round(a, L, rk[0][36], rk[0][37], rk[0][38], rk[0][39]);
+    b = aes_round(b, L, rk[1][36], rk[1][37], rk[1][38], rk[1][39]);
     const Blk pa = bxor(p, ca), pb = bxor(p, cb);
     a = aes_final(a, L, rk[0][40] ^ pa.x, rk[0][41] ^ pa.y, rk[0][42] ^ pa.z, rk[0][43] ^ pa.w);
     b = aes_final(b, L, rk[1][40] ^ pb.x, rk[1][41] ^ pb.y, rk[1][42] ^ pb.z, rk[1][43] ^ pb.w);
 }
 
-__device__ __forceinline__ uint32_t mmo_leaf_bits(const Blk p, uint32_t L, const uint32_t (&rk)[2][44]) {
-    Blk a = {p.x ^ rk[0][0], p.y ^ rk[0][1], p.z ^ rk[0][2], p.w ^ rk[0][3]};
-    Blk b = {p.x ^ rk[1][0], p.y ^ rk[1][1], p.z ^ rk[1][2], p.w ^ rk[1][3]};
-#pragma unroll 1
-    for (int r = 1; r <= 8; ++r) {
-        a = aes_round(a, L, rk[0][4 * r], rk[0][4 * r + 1], rk[0][4 * r + 2], rk[0][4 * r + 3]);
-        b = aes_round(b, L, rk[1][4 * r], rk[1][4 * r + 1], rk[1][4 * r + 2], rk[1][4 * r + 3]);
-    }
+__device__ __forceinline__ void mmo_pair(const Blk p, uint32_t L, const uint32_t (&rk)[2][44], const Blk ca,
+                                         const Blk cb, Blk& a, Blk& b) {
+    mmo_rounds18(p, L, rk, a, b);
+    mmo_pair_tail(p, L, rk, ca, cb, a, b);
+}
+
+__device__ __forceinline__ uint32_t mmo_leaf_bits_tail(const Blk p, uint32_t L, const uint32_t (&rk)[2][44], const Blk a,
+                                                       const Blk b) {
     const uint32_t a9 = aes_round_col0(a, L, rk[0][36]);
     const uint32_t b9 = aes_round_col0(b, L, rk[1][36]);
     const uint32_t ba = (sbox0_lsb(a9, L) ^ rk[0][40] ^ p.x) & 1u;
@@ -263,15 +300,10 @@ __device__ __forceinline__ uint32_t mmo_leaf_bits(const Blk p, uint32_t L, const
     return ba | (bb << 1);
 }
 
-__device__ __forceinline__ void mmo_leaf_words(const Blk p, uint32_t L, const uint32_t (&rk)[2][44], uint32_t& wa,
-                                               uint32_t& wb) {
-    Blk a = {p.x ^ rk[0][0], p.y ^ rk[0][1], p.z ^ rk[0][2], p.w ^ rk[0][3]};
-    Blk b = {p.x ^ rk[1][0], p.y ^ rk[1][1], p.z ^ rk[1][2], p.w ^ rk[1][3]};
-#pragma unroll 1
-    for (int r = 1; r <= 9; ++r) {
-        a = aes_round(a, L, rk[0][4 * r], rk[0][4 * r + 1], rk[0][4 * r + 2], rk[0][4 * r + 3]);
-        b = aes_round(b, L, rk[1][4 * r], rk[1][4 * r + 1], rk[1][4 * r + 2], rk[1][4 * r + 3]);
-    }
+__device__ __forceinline__ void mmo_leaf_words_tail(const Blk p, uint32_t L, const uint32_t (&rk)[2][44], Blk a, Blk b,
+                                                    uint32_t& wa, uint32_t& wb) {
+    a = aes_round(a, L, rk[0][36], rk[0][37], rk[0][38], rk[0][39]);
+    b = aes_round(b, L, rk[1][36], rk[1][37], rk[1][38], rk[1][39]);
     wa = (T<2>(tix(a.x, L, 0)) & 0xffu) ^ (T<3>(tix(a.y, L, 1)) & 0xff00u) ^ (T<0>(tix(a.z, L, 2)) & 0xff0000u) ^
          (T<1>(tix(a.w, L, 3)) & 0xff000000u) ^ rk[0][40] ^ p.x;
     wb = (T<2>(tix(b.x, L, 0)) & 0xffu) ^ (T<3>(tix(b.y, L, 1)) & 0xff00u) ^ (T<0>(tix(b.z, L, 2)) & 0xff0000u) ^
@@ -516,8 +548,14 @@ __device__ __forceinline__ void lane_eval(const FusedParams& P, const uint8_t* k
     const uint32_t npairs = 1u << (sq - 1);
     for (;;) {
         const uint32_t t = node.x & 1u;
+        Key4 k;
+        Blk a, b;
+        if (PRF == 0)
+            keyed_rounds18(node, L, k, a, b);
+        else
+            mmo_rounds18(node, L, P.mmo_rk, a, b);
         if (depth == m - 1) {
-            uint32_t b2 = PRF == 0 ? keyed_leaf_bits(node, L) : mmo_leaf_bits(node, L, P.mmo_rk);
+            uint32_t b2 = PRF == 0 ? keyed_leaf_bits_tail(L, k, a, b) : mmo_leaf_bits_tail(node, L, P.mmo_rk, a, b);
             b2 ^= cw_lsb(kq, m, t, 0, m) | (cw_lsb(kq, m, t, 1, m) << 1);
             acc |= b2 << ((2 * p) & 31);
             ++p;
@@ -532,11 +570,10 @@ __device__ __forceinline__ void lane_eval(const FusedParams& P, const uint8_t* k
         } else {
             const Blk c0 = cw_load(kq, m, t, 0, depth + 1);
             const Blk c1 = cw_load(kq, m, t, 1, depth + 1);
-            Blk a, b;
             if (PRF == 0)
-                keyed_pair(node, L, c0, c1, a, b);
+                keyed_pair_tail(L, k, c0, c1, a, b);
             else
-                mmo_pair(node, L, P.mmo_rk, c0, c1, a, b);
+                mmo_pair_tail(node, L, P.mmo_rk, c0, c1, a, b);
             ++depth;
             if (IMPIR_IN_BOUNDS(depth - D < kMaxLaneBits, kSiteStack, depth - D)) stk[depth - D] = b;
             node = a;
@@ -565,13 +602,18 @@ __device__ __forceinline__ void add_walk_chunk(const FusedParams& P, const uint8
     uint32_t depth = w.depth, p = w.p;
     const uint32_t npairs = 1u << (sq - 1), end = p + ch / 2;
     for (;;) {
+        // node and leaf pairs each by their own copy of the rounds: with one copy for both (as in
+        // lane_eval) this walk, whose state fills the registers, measured 11 % slower
         const uint32_t t = node.x & 1u;
+        Blk a, b;
         if (depth == m - 1) {
             uint32_t wa, wb;
-            if (PRF == 0)
+            if (PRF == 0) {
                 keyed_leaf_words(node, L, wa, wb);
-            else
-                mmo_leaf_words(node, L, P.mmo_rk, wa, wb);
+            } else {
+                mmo_rounds18(node, L, P.mmo_rk, a, b);
+                mmo_leaf_words_tail(node, L, P.mmo_rk, a, b, wa, wb);
+            }
             wa ^= cw_load(kq, m, t, 0, m).x;
             wb ^= cw_load(kq, m, t, 1, m).x;
             const uint32_t r = lane * ch + ((2 * p) & (ch - 1));
@@ -587,7 +629,6 @@ __device__ __forceinline__ void add_walk_chunk(const FusedParams& P, const uint8
         } else {
             const Blk c0 = cw_load(kq, m, t, 0, depth + 1);
             const Blk c1 = cw_load(kq, m, t, 1, depth + 1);
-            Blk a, b;
             if (PRF == 0)
                 keyed_pair(node, L, c0, c1, a, b);
             else
