@@ -20,7 +20,7 @@ LIB = os.path.join(HERE, "libimpir.so")
 BUILD_BOUNDS = os.path.join(HERE, "_build_bounds")
 LIB_BOUNDS = os.path.join(HERE, "libimpir_bounds.so")
 ARCH = ["-gencode", "arch=compute_103a,code=sm_103a"]
-UNITS = ["fused_q1.cu", "fused_q2.cu", "fused_q4.cu", "fused_q8.cu", "fused_q16.cu", "fused_add.cu", "setup.cu", "noalloc.cu", "aes_bench.cu", "combine.cu", "host_aes.cpp", "impir_host.cpp",
+UNITS = ["fused_q1.cu", "fused_q2.cu", "fused_q4.cu", "fused_q8.cu", "fused_q16.cu", "fused_add.cu", "fused_tc.cu", "setup.cu", "noalloc.cu", "aes_bench.cu", "combine.cu", "host_aes.cpp", "impir_host.cpp",
          "serve.cpp"]
 
 

@@ -55,7 +55,7 @@ __global__ void __launch_bounds__(512, 1) aes_bench_kernel(const __grid_constant
         if (PRF == 0)
             keyed_pair(p, L, zero, zero, a, b);
         else
-            mmo_pair(p, L, P.mmo_rk, zero, zero, a, b);
+            mmo_pair(p, L, c_mmo.rk, zero, zero, a, b);
         p = bxor(a, b);
     }
     out[g] = make_uint4(p.x, p.y, p.z, p.w);
@@ -263,8 +263,6 @@ extern "C" impir_status impir_aes_calibrate(int prf, uint32_t iters, uint32_t n_
     uint32_t te0[256];
     host_aes_te0(te0);
     FusedParams fp{};
-    host_aes_expand(reinterpret_cast<const uint8_t*>(IMPIR_MMO_KEY0), fp.mmo_rk[0]);
-    host_aes_expand(reinterpret_cast<const uint8_t*>(IMPIR_MMO_KEY1), fp.mmo_rk[1]);
     uint32_t* d_te0 = nullptr;
     uint4 *d_seeds = nullptr, *d_out = nullptr;
     cudaEvent_t e0 = nullptr, e1 = nullptr;

@@ -263,6 +263,49 @@ __device__ __forceinline__ void keyed_leaf_words(const Blk p, uint32_t L, uint32
          (T<1>(tix(b.w, L, 3)) & 0xff000000u) ^ k10;
 }
 
+// Round keys of the fixed-key PRF, computed at compile time.
+struct MmoKeys {
+    uint32_t rk[2][44];
+};
+
+constexpr MmoKeys mmo_keys() {
+    // FIPS-197 key expansion with the S-box computed from its definition
+    uint8_t box[256] = {};
+    uint8_t p = 1, q = 1;  // q = 1 / p throughout
+    do {
+        p = uint8_t(p ^ (p << 1) ^ (p & 0x80 ? 0x1b : 0));  // p *= 3
+        q = uint8_t(q ^ (q << 1));                          // q /= 3
+        q = uint8_t(q ^ (q << 2));
+        q = uint8_t(q ^ (q << 4));
+        if (q & 0x80) q = uint8_t(q ^ 0x09);
+        uint32_t x = 0;
+        for (int r = 0; r < 5; ++r) x ^= (uint32_t(q) << r | uint32_t(q) >> (8 - r));
+        box[p] = uint8_t(x ^ 0x63);
+    } while (p != 1);
+    box[0] = 0x63;
+    const char* keys[2] = {IMPIR_MMO_KEY0, IMPIR_MMO_KEY1};
+    MmoKeys m{};
+    for (int k = 0; k < 2; ++k) {
+        uint32_t rc = 1;
+        for (int i = 0; i < 4; ++i)
+            for (int b = 0; b < 4; ++b) m.rk[k][i] |= uint32_t(uint8_t(keys[k][4 * i + b])) << (8 * b);
+        for (int i = 4; i < 44; ++i) {
+            uint32_t t = m.rk[k][i - 1];
+            if (i % 4 == 0) {
+                t = t >> 8 | t << 24;
+                t = uint32_t(box[t & 0xff]) | uint32_t(box[t >> 8 & 0xff]) << 8 | uint32_t(box[t >> 16 & 0xff]) << 16 |
+                    uint32_t(box[t >> 24]) << 24;
+                t ^= rc;
+                rc = rc << 1 ^ (rc & 0x80 ? 0x11b : 0);
+            }
+            m.rk[k][i] = m.rk[k][i - 4] ^ t;
+        }
+    }
+    return m;
+}
+
+static __constant__ MmoKeys c_mmo = mmo_keys();
+
 // ---- MMO PRF: PRF_p(x) = AES_{K_x}(p) ^ p with fixed round keys rk[x][44] ----
 
 // Rounds 1-8 under both keys.
@@ -521,24 +564,25 @@ __device__ __forceinline__ void scan_chunk_add(const FusedParams& P, uint64_t ti
 // The walk starts from `start`, the node at depth d0 on the lane's path (the root with d0 = 0,
 // or the warp-tile root the warp computed once for this query).
 template <int PRF>
-__device__ __forceinline__ Blk walk_down(const FusedParams& P, const uint8_t* kq, uint32_t m, uint32_t D, uint64_t sub,
+__device__ __forceinline__ Blk walk_down(const uint8_t* kq, uint32_t m, uint32_t D, uint64_t sub,
                                          uint32_t L, const Blk start, uint32_t d0) {
     Blk node = start;
+#pragma unroll 1
     for (uint32_t d = d0 + 1; d <= D; ++d) {
         const uint32_t x = uint32_t(sub >> (D - d)) & 1u;
         const uint32_t t = node.x & 1u;
         const Blk c = cw_load(kq, m, t, x, d);
-        const Blk f = PRF == 0 ? keyed_one(node, x, L) : mmo_one(node, x, L, P.mmo_rk);
+        const Blk f = PRF == 0 ? keyed_one(node, x, L) : mmo_one(node, x, L, c_mmo.rk);
         node = bxor(f, c);
     }
     return node;
 }
 
 template <int PRF>
-__device__ __forceinline__ void lane_eval(const FusedParams& P, const uint8_t* kq, uint32_t m, uint32_t D,
+__device__ __forceinline__ void lane_eval(const uint8_t* kq, uint32_t m, uint32_t D,
                                           uint64_t sub, uint32_t sq, uint32_t* bits, uint32_t lane, uint32_t L,
                                           const Blk start, uint32_t d0) {
-    Blk node = walk_down<PRF>(P, kq, m, D, sub, L, start, d0);
+    Blk node = walk_down<PRF>(kq, m, D, sub, L, start, d0);
     if (sq == 0) {
         if (slice_ok(&bits[lane >> 5], 4)) atomicOr(&bits[lane >> 5], (node.x & 1u) << (lane & 31));
         return;
@@ -553,9 +597,9 @@ __device__ __forceinline__ void lane_eval(const FusedParams& P, const uint8_t* k
         if (PRF == 0)
             keyed_rounds18(node, L, k, a, b);
         else
-            mmo_rounds18(node, L, P.mmo_rk, a, b);
+            mmo_rounds18(node, L, c_mmo.rk, a, b);
         if (depth == m - 1) {
-            uint32_t b2 = PRF == 0 ? keyed_leaf_bits_tail(L, k, a, b) : mmo_leaf_bits_tail(node, L, P.mmo_rk, a, b);
+            uint32_t b2 = PRF == 0 ? keyed_leaf_bits_tail(L, k, a, b) : mmo_leaf_bits_tail(node, L, c_mmo.rk, a, b);
             b2 ^= cw_lsb(kq, m, t, 0, m) | (cw_lsb(kq, m, t, 1, m) << 1);
             acc |= b2 << ((2 * p) & 31);
             ++p;
@@ -573,7 +617,7 @@ __device__ __forceinline__ void lane_eval(const FusedParams& P, const uint8_t* k
             if (PRF == 0)
                 keyed_pair_tail(L, k, c0, c1, a, b);
             else
-                mmo_pair_tail(node, L, P.mmo_rk, c0, c1, a, b);
+                mmo_pair_tail(node, L, c_mmo.rk, c0, c1, a, b);
             ++depth;
             if (IMPIR_IN_BOUNDS(depth - D < kMaxLaneBits, kSiteStack, depth - D)) stk[depth - D] = b;
             node = a;
@@ -611,8 +655,8 @@ __device__ __forceinline__ void add_walk_chunk(const FusedParams& P, const uint8
             if (PRF == 0) {
                 keyed_leaf_words(node, L, wa, wb);
             } else {
-                mmo_rounds18(node, L, P.mmo_rk, a, b);
-                mmo_leaf_words_tail(node, L, P.mmo_rk, a, b, wa, wb);
+                mmo_rounds18(node, L, c_mmo.rk, a, b);
+                mmo_leaf_words_tail(node, L, c_mmo.rk, a, b, wa, wb);
             }
             wa ^= cw_load(kq, m, t, 0, m).x;
             wb ^= cw_load(kq, m, t, 1, m).x;
@@ -632,7 +676,7 @@ __device__ __forceinline__ void add_walk_chunk(const FusedParams& P, const uint8
             if (PRF == 0)
                 keyed_pair(node, L, c0, c1, a, b);
             else
-                mmo_pair(node, L, P.mmo_rk, c0, c1, a, b);
+                mmo_pair(node, L, c_mmo.rk, c0, c1, a, b);
             ++depth;
             if (IMPIR_IN_BOUNDS(depth - D < kMaxLaneBits, kSiteStack, depth - D)) w.stk[depth - D] = b;
             node = a;
@@ -665,8 +709,8 @@ __device__ __forceinline__ void unit_add(const FusedParams& P, const GroupDesc& 
             const uint8_t* kq = query_key(P, query_at(P, qidx, q));
             const Blk start{__shfl_sync(0xffffffffu, top.x, q), __shfl_sync(0xffffffffu, top.y, q),
                             __shfl_sync(0xffffffffu, top.z, q), __shfl_sync(0xffffffffu, top.w, q)};
-            w[q].node = kq[1] == 0 ? walk_down<0>(P, kq, m, D, sub, L, start, Dt)
-                                   : walk_down<1>(P, kq, m, D, sub, L, start, Dt);
+            w[q].node = kq[1] == 0 ? walk_down<0>(kq, m, D, sub, L, start, Dt)
+                                   : walk_down<1>(kq, m, D, sub, L, start, Dt);
             w[q].depth = D;
             w[q].p = 0;
             neg[q] = kq[3] ? 0xffffffffu : 0u;  // party 1 negates its shares (mod 2^32)
@@ -926,6 +970,8 @@ __global__ void __launch_bounds__((NK == 1 && QC <= 8) ? 640 : 512, 1)
     const uint32_t tid = threadIdx.x, nthr = blockDim.x;
     const uint32_t lane = tid & 31, warp = tid >> 5;
 
+    WsHeader* hdr = reinterpret_cast<WsHeader*>(P.ws);
+    if (hdr->n_units == 0) return;  // every tile was the tensor-core kernel's (or no key was well formed)
     // Replicated T-tables (see the layout note at the top of this file).
     for (uint32_t i = tid; i < 256 * 32; i += nthr) {
         const uint32_t x = i >> 5, l = i & 31;
@@ -937,7 +983,6 @@ __global__ void __launch_bounds__((NK == 1 && QC <= 8) ? 640 : 512, 1)
         rb[l] = __funnelshift_l(t0, t0, 16);
         rb[32 + l] = __funnelshift_l(t0, t0, 24);
     }
-    WsHeader* hdr = reinterpret_cast<WsHeader*>(P.ws);
 #ifdef IMPIR_BOUNDS
     if (tid == 0) {
         s_bctx.rec = P.bounds;
@@ -953,8 +998,9 @@ __global__ void __launch_bounds__((NK == 1 && QC <= 8) ? 640 : 512, 1)
 #endif
     SegDesc* segs = reinterpret_cast<SegDesc*>(g_smem + kTableBytes);
     uint32_t n_segs = hdr->n_segs;
-    if (!IMPIR_IN_BOUNDS(n_segs <= kMaxSegments, kSiteSchedule, n_segs)) n_segs = kMaxSegments;
-    const SegDesc* gsegs = reinterpret_cast<const SegDesc*>(P.ws + P.lay.off_segs);
+    const uint32_t first_seg = hdr->first_seg;
+    if (!IMPIR_IN_BOUNDS(first_seg + n_segs <= kMaxSegments, kSiteSchedule, n_segs)) n_segs = 0;
+    const SegDesc* gsegs = reinterpret_cast<const SegDesc*>(P.ws + P.lay.off_segs) + first_seg;
     for (uint32_t i = tid; i < n_segs; i += nthr) segs[i] = gsegs[i];
     __syncthreads();
 
@@ -1012,9 +1058,10 @@ __global__ void __launch_bounds__((NK == 1 && QC <= 8) ? 640 : 512, 1)
         if (lane < gd.count) {
             const uint8_t* kq = query_key(P, query_at(P, qidx, lane));
             top = cw_load(kq, m, 0, 0, 0);  // R(0,0) = C_0[0][0], Eq. (2)
+#pragma unroll 1
             for (uint32_t d = 1; d <= Dt; ++d) {
                 const uint32_t x = uint32_t(tile >> (Dt - d)) & 1u;
-                const Blk f = kq[1] == 0 ? keyed_one(top, x, L) : mmo_one(top, x, L, P.mmo_rk);
+                const Blk f = kq[1] == 0 ? keyed_one(top, x, L) : mmo_one(top, x, L, c_mmo.rk);
                 top = bxor(f, cw_load(kq, m, top.x & 1u, x, d));
             }
         }
@@ -1029,10 +1076,12 @@ __global__ void __launch_bounds__((NK == 1 && QC <= 8) ? 640 : 512, 1)
             if (lane < gd.count && slice_ok(nodes + lane * slot, 16))
                 *reinterpret_cast<uint4*>(nodes + lane * slot) = make_uint4(top.x, top.y, top.z, top.w);
             __syncwarp();
+#pragma unroll 1
             for (uint32_t k = 0; k < 4; ++k) {  // level k -> k + 1 below the warp-tile root
                 const uint32_t per = 1u << k, items = gd.count * per;
                 // parents in descending index order: children 2i, 2i+1 overwrite only parents
                 // already read (in this chunk, before any write) or expanded (earlier chunks)
+#pragma unroll 1
                 for (uint32_t f0 = 0; f0 < items; f0 += 32) {
                     const uint32_t f = f0 + lane;
                     const bool act = f < items;
@@ -1050,7 +1099,7 @@ __global__ void __launch_bounds__((NK == 1 && QC <= 8) ? 640 : 512, 1)
                         if (kq[1] == 0)
                             keyed_pair(par, L, c0, c1, a, b);
                         else
-                            mmo_pair(par, L, P.mmo_rk, c0, c1, a, b);
+                            mmo_pair(par, L, c_mmo.rk, c0, c1, a, b);
                         if (slice_ok(nodes + q * slot + (2 * i) * 16, 32)) {
                             *reinterpret_cast<uint4*>(nodes + q * slot + (2 * i) * 16) = make_uint4(a.x, a.y, a.z, a.w);
                             *reinterpret_cast<uint4*>(nodes + q * slot + (2 * i + 1) * 16) = make_uint4(b.x, b.y, b.z, b.w);
@@ -1059,6 +1108,7 @@ __global__ void __launch_bounds__((NK == 1 && QC <= 8) ? 640 : 512, 1)
                     __syncwarp();
                 }
             }
+#pragma unroll 1
             for (uint32_t qi = 0; qi < gd.count; ++qi) {
                 const uint8_t* kq = query_key(P, query_at(P, qidx, qi));
                 const uint32_t prf = kq[1];
@@ -1073,12 +1123,13 @@ __global__ void __launch_bounds__((NK == 1 && QC <= 8) ? 640 : 512, 1)
                 const Blk start{pv.x, pv.y, pv.z, pv.w};
                 if (lane_on) {
                     if (prf == 0)
-                        lane_eval<0>(P, kq, m, D, sub, sq, bits + qi * P.bits_words, lane, L, start, D - 1);
+                        lane_eval<0>(kq, m, D, sub, sq, bits + qi * P.bits_words, lane, L, start, D - 1);
                     else
-                        lane_eval<1>(P, kq, m, D, sub, sq, bits + qi * P.bits_words, lane, L, start, D - 1);
+                        lane_eval<1>(kq, m, D, sub, sq, bits + qi * P.bits_words, lane, L, start, D - 1);
                 }
             }
         } else {
+#pragma unroll 1
             for (uint32_t qi = 0; qi < gd.count; ++qi) {
                 const uint8_t* kq = query_key(P, query_at(P, qidx, qi));
                 const uint32_t prf = kq[1];
@@ -1086,9 +1137,9 @@ __global__ void __launch_bounds__((NK == 1 && QC <= 8) ? 640 : 512, 1)
                                 __shfl_sync(0xffffffffu, top.z, qi), __shfl_sync(0xffffffffu, top.w, qi)};
                 if (lane_on) {
                     if (prf == 0)
-                        lane_eval<0>(P, kq, m, D, sub, sq, bits + qi * P.bits_words, lane, L, start, Dt);
+                        lane_eval<0>(kq, m, D, sub, sq, bits + qi * P.bits_words, lane, L, start, Dt);
                     else
-                        lane_eval<1>(P, kq, m, D, sub, sq, bits + qi * P.bits_words, lane, L, start, Dt);
+                        lane_eval<1>(kq, m, D, sub, sq, bits + qi * P.bits_words, lane, L, start, Dt);
                 }
             }
         }

@@ -61,7 +61,6 @@ struct DeviceState {
     int device = -1;
     int sms = 0;
     uint32_t* d_te0 = nullptr;
-    uint32_t mmo_rk[2][44];
 };
 
 DeviceState& device_state() {
@@ -74,8 +73,6 @@ DeviceState& device_state() {
         host_aes_te0(te0);
         if (e == cudaSuccess) e = cudaMalloc(&st.d_te0, sizeof te0);
         if (e == cudaSuccess) e = cudaMemcpy(st.d_te0, te0, sizeof te0, cudaMemcpyHostToDevice);
-        host_aes_expand(reinterpret_cast<const uint8_t*>(IMPIR_MMO_KEY0), st.mmo_rk[0]);
-        host_aes_expand(reinterpret_cast<const uint8_t*>(IMPIR_MMO_KEY1), st.mmo_rk[1]);
         if (e != cudaSuccess) {
             st.err = cudaGetErrorString(e);
             return;
@@ -100,6 +97,7 @@ struct Db {
     bool owned = false;
     bool live = false;
     bool cfg_set = false;
+    bool cfg_tuned = false;  // cfg came from the autotuner: the tensor-core kernel may still take a batch
     impir_config cfg{};
     uint64_t version = 0;  // bumped by every bulk update
     uint64_t row_lo = 0;   // a row shard: global index of its first row
@@ -271,11 +269,11 @@ size_t smem_add(const impir_config& c) {
 // build's index checks use it)
 impir_status launch_batch(const DeviceState& dev, const Db& db, const impir_config& cfg, const uint8_t* d_keys,
                           const uint32_t* d_off, uint32_t n, uint8_t* d_out, uint8_t* d_ws, cudaStream_t st,
-                          int mode = 0, size_t keys_bytes = 0) {
+                          int mode = 0, size_t keys_bytes = 0, bool tc_allowed = false) {
     const WsLayout lay = ws_layout(n, db.stride);
     // a row shard covers the warp tiles of its rows (shard bounds are whole tiles) of a
     // database of n_total records; its device rows start at global row row_lo
-    const uint64_t T = 32ull << cfg.lane_bits;
+    const XorShape shape = xor_shape(cfg, mode == 0 && tc_allowed, db.n, db.stride / 16, n, dev.sms);
     const bool shard = db.row_lo != 0 || db.n_total != db.n;
     SetupParams sp{};
     sp.keys = d_keys;
@@ -285,10 +283,9 @@ impir_status launch_batch(const DeviceState& dev, const Db& db, const impir_conf
     sp.n_records = db.n_total;
     sp.n_queries = n;
     sp.words = db.stride / 16;
-    sp.lane_bits = cfg.lane_bits;
-    sp.qpw = cfg.queries_per_warp;
-    sp.tile_lo = shard ? db.row_lo / T : 0;
-    sp.tile_hi = shard ? (db.row_lo + db.n + T - 1) / T : 0;
+    apply_shape(shape, dev.sms, &sp);
+    sp.rec_lo = shard ? db.row_lo : 0;
+    sp.rec_hi = shard ? db.row_lo + db.n : 0;
     sp.bounds = bounds_record();
     sp.keys_bytes = keys_bytes;
     CK(launch_setup(sp, st), "setup kernel launch");
@@ -303,15 +300,10 @@ impir_status launch_batch(const DeviceState& dev, const Db& db, const impir_conf
     fp.n_records = db.n_total;
     fp.n_queries = n;
     fp.words = db.stride / 16;
-    fp.lane_bits = cfg.lane_bits;
-    fp.bits_words = mode == 0 ? 1u << cfg.lane_bits : add_share_words(cfg);
     fp.rec_lo = db.row_lo;
-    std::memcpy(fp.mmo_rk, dev.mmo_rk, sizeof fp.mmo_rk);
-    const size_t smem = mode == 0 ? smem_for(cfg) : smem_add(cfg);
     fp.bounds = sp.bounds;
     fp.db_words = bounds_db_words(db.n * (db.stride / 16), db.stride / 16);
     fp.keys_bytes = keys_bytes;
-    fp.smem_bytes = uint32_t(smem);
     const bool timed = timing_on();
     cudaEvent_t ev0 = nullptr, ev1 = nullptr;
     if (timed) {
@@ -319,14 +311,17 @@ impir_status launch_batch(const DeviceState& dev, const Db& db, const impir_conf
         CK(cudaEventCreate(&ev1), "event create");
         CK(cudaEventRecord(ev0, st), "event record");
     }
-    if (mode == 0)
-        CK(launch_fused(cfg.queries_per_warp, nk_xor(fp.words, cfg.queries_per_warp), dim3(dev.sms),
-                        dim3(cfg.warps_per_cta * 32), smem, st, fp),
-           "fused kernel launch");
-    else
+    if (mode == 0) {
+        CK(launch_xor(shape, dev.sms, st, fp), "fused kernel launch");
+    } else {
+        const size_t smem = smem_add(cfg);
+        fp.lane_bits = cfg.lane_bits;
+        fp.bits_words = add_share_words(cfg);
+        fp.smem_bytes = uint32_t(smem);
         CK(launch_fused_add(cfg.queries_per_warp, nk_need(fp.words), dim3(dev.sms), dim3(cfg.warps_per_cta * 32), smem,
                             st, fp),
            "fused kernel launch (additive)");
+    }
     if (timed) {
         CK(cudaEventRecord(ev1, st), "event record");
         std::lock_guard<std::mutex> lk(g_timing.mu);
@@ -334,10 +329,10 @@ impir_status launch_batch(const DeviceState& dev, const Db& db, const impir_conf
         g_timing.fused += 1;
     }
     if (!d_out) {  // the caller reads the answers from the accumulators itself
-        count_launches(2);
+        count_launches(shape.tc ? 3 : 2);
         return IMPIR_OK;
     }
-    count_launches(3);
+    count_launches(shape.tc ? 4 : 3);
 
     FinalizeParams zp{};
     zp.ws = d_ws;
@@ -370,6 +365,8 @@ impir_status answer_async_impl(const Db& db, const impir_config* cfg_in, const u
         cfg = add_config(cfg, db.stride / 16);
     }
     if (impir_status s = check_config(cfg, db.stride / 16, mode)) return s;
+    // a shape that the caller set is launched as it is
+    const bool tc_allowed = !cfg_in && (!db.cfg_set || db.cfg_tuned);
     if (cfg.queries_per_launch == 1) {
         if (direct_out) return fail(IMPIR_EINVAL, "direct answers need one launch for the batch");
         if (ws_bytes < ws_layout(1, db.stride).total) return fail(IMPIR_ENOMEM, "workspace too small");
@@ -383,7 +380,7 @@ impir_status answer_async_impl(const Db& db, const impir_config* cfg_in, const u
         return fail(IMPIR_ENOMEM, "workspace of %zu bytes is smaller than the %zu needed", ws_bytes,
                     ws_layout(n, db.stride).total);
     return launch_batch(*dev, db, cfg, d_keys, d_off, n, direct_out ? nullptr : d_out, static_cast<uint8_t*>(d_ws), st,
-                        mode, keys_bytes);
+                        mode, keys_bytes, tc_allowed);
 }
 
 // ---- synchronous path context: cached device and pinned buffers ----
@@ -663,6 +660,7 @@ impir_status impir_workspace_status(const void* d_ws, uint32_t* n_bad, uint32_t*
     CK(cudaMemcpy(&h, d_ws, sizeof h, cudaMemcpyDeviceToHost), "workspace status copy");
     if (n_bad) *n_bad = h.n_bad;
     if (first_bad) *first_bad = h.first_bad;
+    if (h.timed_out) return fail(IMPIR_ECUDA, "a wait inside the kernel ran out: the answers are not valid");
     return IMPIR_OK;
 }
 
@@ -686,7 +684,8 @@ static impir_status answer_sync(int32_t h, const uint8_t* keys, uint32_t n, uint
     const WsLayout lay = ws_layout(cfg.queries_per_launch == 1 ? 1 : n, db.stride);
     const size_t out_bytes = size_t(n) * db.bytes;
     const size_t koff = (total + 15) & ~size_t(15), up = koff + size_t(n) * 4;
-    const size_t stage = std::max(up, out_bytes);
+    const size_t hdr_at = (out_bytes + 15) & ~size_t(15);  // the workspace header comes back behind the answers
+    const size_t stage = std::max(up, hdr_at + sizeof(WsHeader));
     if (impir_status s = grow(&g_sync.d_keys, &g_sync.c_keys, up)) return s;
     if (impir_status s = grow(&g_sync.d_ws, &g_sync.c_ws, lay.total)) return s;
     if (!direct)
@@ -697,13 +696,18 @@ static impir_status answer_sync(int32_t h, const uint8_t* keys, uint32_t n, uint
     cudaStream_t st = g_sync.stream;
     uint8_t* d_keys = static_cast<uint8_t*>(g_sync.d_keys);
     CK(cudaMemcpyAsync(d_keys, g_sync.h_stage, up, cudaMemcpyHostToDevice, st), "key upload");
-    if (impir_status s = answer_async_impl(db, &cfg, d_keys, reinterpret_cast<const uint32_t*>(d_keys + koff), n,
+    if (impir_status s = answer_async_impl(db, nullptr, d_keys, reinterpret_cast<const uint32_t*>(d_keys + koff), n,
                                            static_cast<uint8_t*>(g_sync.d_out), g_sync.d_ws, g_sync.c_ws, st, mode,
                                            direct, total))
         return s;
     const void* src = direct ? static_cast<const void*>(static_cast<uint8_t*>(g_sync.d_ws) + lay.off_acc) : g_sync.d_out;
     CK(cudaMemcpyAsync(g_sync.h_stage, src, out_bytes, cudaMemcpyDeviceToHost, st), "answer download");
+    const bool waits = mode == 0 && n >= tc_min_queries(db.stride / 16);  // batches the tensor-core kernel may have taken
+    if (waits)
+        CK(cudaMemcpyAsync(g_sync.h_stage + hdr_at, g_sync.d_ws, sizeof(WsHeader), cudaMemcpyDeviceToHost, st), "status download");
     CK(cudaStreamSynchronize(st), "answer");
+    if (waits && reinterpret_cast<const WsHeader*>(g_sync.h_stage + hdr_at)->timed_out)
+        return fail(IMPIR_ECUDA, "a wait inside the kernel ran out");
     std::memcpy(out, g_sync.h_stage, out_bytes);
     return bounds_verdict();
 }
@@ -744,15 +748,18 @@ impir_status impir_get_config_add32(int32_t h, uint32_t n_queries, impir_config*
     return IMPIR_OK;
 }
 
-impir_status impir_set_config(int32_t h, const impir_config* cfg) {
+static impir_status set_config(int32_t h, const impir_config* cfg, bool tuned) {
     if (!cfg) return fail(IMPIR_EINVAL, "NULL argument");
     std::lock_guard<std::mutex> lk(g_db_mu);
     if (h < 1 || size_t(h) > g_dbs.size() || !g_dbs[h - 1].live) return fail(IMPIR_EINVAL, "unknown database handle %d", h);
     if (impir_status s = check_config(*cfg, g_dbs[h - 1].stride / 16)) return s;
     g_dbs[h - 1].cfg = *cfg;
     g_dbs[h - 1].cfg_set = true;
+    g_dbs[h - 1].cfg_tuned = tuned;
     return IMPIR_OK;
 }
+
+impir_status impir_set_config(int32_t h, const impir_config* cfg) { return set_config(h, cfg, false); }
 
 impir_status impir_autotune(int32_t h, const uint8_t* d_keys, const uint32_t* d_off, uint32_t n, uint8_t* d_out,
                             void* d_ws, size_t ws_bytes, void* stream, impir_config* best) {
@@ -767,7 +774,7 @@ impir_status impir_autotune(int32_t h, const uint8_t* d_keys, const uint32_t* d_
         auto it = g_tune.find(key);
         if (it != g_tune.end()) {
             if (best) *best = it->second;
-            return impir_set_config(h, &it->second);
+            return set_config(h, &it->second, true);
         }
     }
     const impir_config base = default_config(db.n, db.stride / 16, n, dev->sms);
@@ -812,7 +819,7 @@ impir_status impir_autotune(int32_t h, const uint8_t* d_keys, const uint32_t* d_
         g_tune[key] = best_c;
     }
     if (best) *best = best_c;
-    return impir_set_config(h, &best_c);
+    return set_config(h, &best_c, true);
 }
 
 // ---- databases larger than HBM: streamed in chunks (§3.3) ----
@@ -833,7 +840,8 @@ impir_status impir_answer_streamed(const void* records, uint64_t N, uint32_t B, 
     const uint32_t stride = (B + 15u) & ~15u, words = stride / 16;
     const impir_config cfg = default_config(N, words, n, dev->sms);
     if (used) *used = cfg;
-    const uint64_t T = 32ull << cfg.lane_bits;  // warp tile: chunks hold whole tiles
+    const XorShape shape = xor_shape(cfg, true, N, words, n, dev->sms);
+    const uint64_t T = 32ull << shape.tile_bits();  // chunks hold whole tiles
     if (chunk_bytes == 0) chunk_bytes = 2ull << 30;  // default: 2 GiB (fewer launch tails, small first copy)
     uint64_t chunk = (chunk_bytes / stride) / T * T;
     if (chunk < T) chunk = T;
@@ -914,10 +922,9 @@ impir_status impir_answer_streamed(const void* records, uint64_t N, uint32_t B, 
         sp.n_records = N;
         sp.n_queries = n;
         sp.words = words;
-        sp.lane_bits = cfg.lane_bits;
-        sp.qpw = cfg.queries_per_warp;
-        sp.tile_lo = lo / T;
-        sp.tile_hi = (lo + cnt + T - 1) / T;
+        apply_shape(shape, dev->sms, &sp);
+        sp.rec_lo = lo;
+        sp.rec_hi = lo + cnt;
         sp.keep_acc = c > 0;
         sp.bounds = bounds_record();
         sp.keys_bytes = total;
@@ -933,20 +940,14 @@ impir_status impir_answer_streamed(const void* records, uint64_t N, uint32_t B, 
         fp.n_records = N;
         fp.n_queries = n;
         fp.words = words;
-        fp.lane_bits = cfg.lane_bits;
-        fp.bits_words = 1u << cfg.lane_bits;
         fp.rec_lo = lo;
-        std::memcpy(fp.mmo_rk, dev->mmo_rk, sizeof fp.mmo_rk);
         fp.bounds = sp.bounds;
         fp.db_words = bounds_db_words(cnt * words, words);
         fp.keys_bytes = total;
-        fp.smem_bytes = uint32_t(smem_for(cfg));
         if (e == cudaSuccess)
-            e = launch_fused(cfg.queries_per_warp, nk_xor(words, cfg.queries_per_warp), dim3(dev->sms),
-                             dim3(cfg.warps_per_cta * 32),
-                             smem_for(cfg), ks[b], fp);
+            e = launch_xor(shape, dev->sms, ks[b], fp);
         if (e == cudaSuccess) e = cudaEventRecord(consumed[b], ks[b]);
-        count_launches(2);
+        count_launches(shape.tc ? 3 : 2);
     }
     // join: stream 0 finalizes once stream 1's launches are done
     if (e == cudaSuccess) e = cudaEventRecord(done1, ks[1]);
@@ -963,7 +964,10 @@ impir_status impir_answer_streamed(const void* records, uint64_t N, uint32_t B, 
         e = launch_finalize(zp, ks[0]);
         count_launches(1);
     }
+    WsHeader hdr[2] = {};
     if (e == cudaSuccess) e = cudaMemcpyAsync(out, d_out, size_t(n) * B, cudaMemcpyDeviceToHost, ks[0]);
+    for (uint64_t b = 0; b < std::min<uint64_t>(nchunks, 2) && e == cudaSuccess; ++b)
+        e = cudaMemcpyAsync(&hdr[b], ws_of[b], sizeof(WsHeader), cudaMemcpyDeviceToHost, ks[0]);
     if (e == cudaSuccess) e = cudaStreamSynchronize(ks[0]);
     if (e != cudaSuccess) {
         // leave no work of this call behind on the cached streams
@@ -972,6 +976,8 @@ impir_status impir_answer_streamed(const void* records, uint64_t N, uint32_t B, 
         cudaStreamSynchronize(ks[1]);
         X.zeroed_stride = 0;
         st = cuda_fail(e, "streamed answer");
+    } else if (hdr[0].timed_out || hdr[1].timed_out) {
+        st = fail(IMPIR_ECUDA, "a wait inside the kernel ran out");
     }
     return st == IMPIR_OK ? bounds_verdict() : st;
 }

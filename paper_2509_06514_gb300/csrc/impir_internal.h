@@ -32,7 +32,12 @@ struct WsHeader {
     uint32_t n_groups;
     uint32_t n_segs;
     uint32_t bounds_failed;       // failed index checks of this launch (debug build only)
-    uint32_t pad[55];
+    uint32_t timed_out;           // a wait inside the kernel ran out: the answers are not valid
+    // the tensor-core kernel's share of the batch (fused_tc.cu): its segments come first
+    unsigned long long tc_counter, tc_units;
+    uint32_t tc_segs;
+    uint32_t first_seg;           // the warp kernel's first segment (it has n_segs of them)
+    uint32_t pad[48];
 };
 static_assert(sizeof(WsHeader) == 256, "header is 256 bytes");
 
@@ -46,12 +51,14 @@ struct GroupDesc {
 };
 
 // Work units u in [unit_lo, next segment's unit_lo) cover warp tiles
-// tile_lo + (u - unit_lo) / count with groups (u - unit_lo) % count.
+// tile_lo + (u - unit_lo) / count with groups (u - unit_lo) % count. `active` is the number of
+// sorted queries whose domains reach these tiles (the tensor-core kernel cuts them into `count`
+// groups of equal size by itself).
 struct SegDesc {
     unsigned long long tile_lo;
     unsigned long long unit_lo;
     uint32_t count;
-    uint32_t pad;
+    uint32_t active;
     unsigned long long pad2;
 };
 static_assert(sizeof(SegDesc) == 32, "segment descriptors are 32 bytes");
@@ -165,6 +172,48 @@ inline impir_config default_config(uint64_t n_records, uint32_t words, uint32_t 
     return c20.lane_bits == c16.lane_bits && c20.queries_per_warp == c16.queries_per_warp ? c20 : c16;
 }
 
+// ---- the tensor-core form of the XOR answer (fused_tc.cu) ----
+
+constexpr uint32_t kTcQueries = 128;   // most rows of a unit (rows of the tensor product)
+constexpr uint32_t kTcThreads = 768;   // 4 scan warps and 20 AES warps
+constexpr uint32_t kTcTasks = 32;      // AES tasks of a unit: 4 rows each
+constexpr uint32_t kTcLaneBits = 5;    // tiles of 32 << 5 = 1024 records
+
+// Fewest queries that must reach a tile for the tensor-core kernel to take it. Its scan costs the
+// same for 1 query as for 128, the warp kernels' grows with every query: measured on 2^22 records,
+// time of the fastest warp shape over the tensor-core kernel's at 32 / 48 / 64 / 128 queries: 0.95 /
+// 1.02 / 1.01 / 1.02 for 64-byte records, 0.97 / 1.04 / 1.04 / 1.07 for 256 bytes, 0.90 / 1.04 / 1.07 /
+// 1.15 for 512 bytes, 0.65 / 0.87 / 1.01 / 1.23 for 1 KiB.
+inline uint32_t tc_min_queries(uint32_t words) { return words <= 32 ? 48u : 96u; }
+
+// Fewest units for the tensor-core kernel to take any: units of 1024 records go to SMs whole, and with
+// fewer than four per SM the last round costs more than the scan gains for records up to 256 bytes
+// (0.92 to 0.97 at 2^18 records and 64 or 128 queries); wider ones gain from one and a half on.
+inline uint64_t tc_min_units(uint32_t words, int sms) { return uint64_t(sms) * (words <= 16 ? 8 : 3) / 2; }
+
+// How a batch is launched: the warp kernels of fused.cuh in the shape `c`, with tc after the
+// tensor-core kernel, which takes the tiles that enough queries reach (the setup kernel draws the
+// line: the keys' domains are on the device) in groups of at most tc_cap queries.
+struct XorShape {
+    impir_config c;
+    bool tc;
+    uint32_t tc_cap;
+    // tiles of both kernels divide 32 << tile_bits() records
+    uint32_t tile_bits() const { return tc ? std::max(kTcLaneBits, c.lane_bits) : c.lane_bits; }
+};
+
+// tc_allowed: the caller set no launch shape of its own.
+inline XorShape xor_shape(const impir_config& c, bool tc_allowed, uint64_t n_records, uint32_t words,
+                          uint32_t n_queries, int sms) {
+    XorShape s{c, false, 0};
+    if (!tc_allowed || c.queries_per_launch != 0 || n_queries < tc_min_queries(words)) return s;
+    const uint64_t groups = (n_queries + kTcQueries - 1) / kTcQueries;
+    if (groups * ((n_records + (32u << kTcLaneBits) - 1) >> (kTcLaneBits + 5)) < tc_min_units(words, sms)) return s;
+    s.tc = true;
+    s.tc_cap = uint32_t((n_queries + groups - 1) / groups);
+    return s;
+}
+
 struct SetupParams {
     const uint8_t* keys;
     const uint32_t* key_off;
@@ -175,11 +224,14 @@ struct SetupParams {
     uint32_t words;          // stride / 16
     uint32_t lane_bits;
     uint32_t qpw;            // queries per warp (group size)
-    // A chunk of a streamed database or a row shard: only warp tiles in [tile_lo, tile_hi)
-    // are scheduled (tile_hi == 0: no upper limit), and keep_acc != 0 keeps the accumulators
+    uint32_t group_cap;      // most queries of a tensor-core unit (0: the warp kernels take the whole batch)
+    uint32_t tc_min_queries; // see tc_min_queries() and tc_min_units()
+    unsigned long long tc_min_units;
+    // A chunk of a streamed database or a row shard: only tiles of records [rec_lo, rec_hi) are
+    // scheduled (whole tiles; rec_hi == 0: no upper limit), and keep_acc != 0 keeps the accumulators
     // of the previous chunks instead of zeroing them. Zero values give the whole-database
     // launch.
-    unsigned long long tile_lo, tile_hi;
+    unsigned long long rec_lo, rec_hi;
     uint32_t keep_acc;
     BoundsRecord* bounds;             // debug build: where failed checks are recorded
     unsigned long long keys_bytes;    // size of the key buffer (0: unknown)
@@ -197,7 +249,6 @@ struct FusedParams {
     uint32_t words;          // uint4 words per record (stride / 16)
     uint32_t lane_bits;
     uint32_t bits_words;     // 32-bit words of selection bits (additive: shares) per (warp, query slot)
-    uint32_t mmo_rk[2][44];  // round keys of the fixed MMO keys K_0, K_1
     unsigned long long rec_lo;  // global index of the record at db[0] (0 unless a chunk or a row shard)
     // extents for the debug build's index checks
     BoundsRecord* bounds;
@@ -225,6 +276,13 @@ BoundsRecord* bounds_record();
 // records a debug-build test withholds (IMPIR_BOUNDS_TEST_WITHHOLD_RECORDS) to see a check fire.
 unsigned long long bounds_db_words(unsigned long long n_words, uint32_t words_per_record);
 cudaError_t launch_finalize(const FinalizeParams& p, cudaStream_t s);
+// The XOR answer's fused launch in the given shape: sets the shape's fields of the setup
+// parameters (before launch_setup) and launches the kernel it names.
+void apply_shape(const XorShape& s, int sms, SetupParams* sp);
+cudaError_t launch_xor(const XorShape& s, int sms, cudaStream_t st, FusedParams& fp);
+cudaError_t launch_fused_tc(int sms, cudaStream_t s, const FusedParams& p);
+cudaError_t prepare_fused_tc();
+uint32_t tc_smem_bytes();
 // qpw in {1,2,4,8,16}, nk in {1,2,4,8} with qpw * nk <= 16.
 cudaError_t launch_fused(uint32_t qpw, uint32_t nk, dim3 grid, dim3 block, size_t smem, cudaStream_t s,
                          const FusedParams& p);

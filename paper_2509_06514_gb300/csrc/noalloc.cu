@@ -35,7 +35,6 @@ struct NoallocDevice {
     uint8_t* scratch = nullptr;   // device address of g_noalloc_scratch on this device
     uint32_t* te0 = nullptr;      // device address of g_noalloc_te0 on this device
     int sms = 0;
-    uint32_t mmo_rk[2][44];
     BoundsRecord* bounds = nullptr;  // debug build: the device's record of failed index checks
 };
 
@@ -66,8 +65,6 @@ impir_status device_setup(NoallocDevice** out) {
             return set_error(IMPIR_ECUDA, "T-table upload failed");
         if (cudaDeviceGetAttribute(&d.sms, cudaDevAttrMultiProcessorCount, dev) != cudaSuccess)
             return set_error(IMPIR_ECUDA, "SM count query failed");
-        host_aes_expand(reinterpret_cast<const uint8_t*>(IMPIR_MMO_KEY0), d.mmo_rk[0]);
-        host_aes_expand(reinterpret_cast<const uint8_t*>(IMPIR_MMO_KEY1), d.mmo_rk[1]);
         // every kernel a later call can launch: shared-memory limit set and code loaded on this
         // device now, so that no later call does first-use work
         if (prepare_xor_kernels() != cudaSuccess) {
@@ -110,9 +107,7 @@ extern "C" impir_status impir_answer_noalloc(const void* d_records, uint64_t n_r
     // launch shape: the asynchronous path's default for this database and batch
     const uint32_t words = stride_bytes / 16;
     const impir_config cfg = default_config(n_records, words, n_queries, dev->sms);
-    const uint32_t qpw = cfg.queries_per_warp, lane_bits = cfg.lane_bits;
-    const uint32_t nk = nk_xor(words, qpw);
-    const size_t smem = smem_for(cfg);
+    const XorShape shape = xor_shape(cfg, true, n_records, words, n_queries, dev->sms);
 
     SetupParams sp{};
     sp.keys = d_keys;
@@ -122,8 +117,7 @@ extern "C" impir_status impir_answer_noalloc(const void* d_records, uint64_t n_r
     sp.n_records = n_records;
     sp.n_queries = n_queries;
     sp.words = words;
-    sp.lane_bits = lane_bits;
-    sp.qpw = qpw;
+    apply_shape(shape, dev->sms, &sp);
     sp.bounds = dev->bounds;
     if (launch_setup(sp, st) != cudaSuccess) {
         cudaGetLastError();
@@ -140,14 +134,9 @@ extern "C" impir_status impir_answer_noalloc(const void* d_records, uint64_t n_r
     fp.n_records = n_records;
     fp.n_queries = n_queries;
     fp.words = words;
-    fp.lane_bits = lane_bits;
-    fp.bits_words = 1u << lane_bits;
-    for (int x = 0; x < 2; ++x)
-        for (int i = 0; i < 44; ++i) fp.mmo_rk[x][i] = dev->mmo_rk[x][i];
     fp.bounds = dev->bounds;
     fp.db_words = bounds_db_words(n_records * words, words);
-    fp.smem_bytes = uint32_t(smem);
-    if (launch_fused(qpw, nk, dim3(dev->sms), dim3(cfg.warps_per_cta * 32), smem, st, fp) != cudaSuccess) {
+    if (launch_xor(shape, dev->sms, st, fp) != cudaSuccess) {
         cudaGetLastError();
         return set_error(IMPIR_ECUDA, "fused kernel launch failed");
     }

@@ -67,7 +67,8 @@ struct Slot {
     uint8_t* d_ws = nullptr;
     size_t ws_bytes = 0;
     uint8_t* h_in = nullptr;   // pinned: keys then offsets
-    uint8_t* h_out = nullptr;  // pinned: answers
+    uint8_t* h_out = nullptr;  // pinned: answers, then the workspace header
+    WsHeader* h_hdr = nullptr;
     bool busy = false;
     std::vector<Request> reqs;
     uint32_t record_bytes = 0;
@@ -124,7 +125,7 @@ void harvest(impir_server* S) {
             Done d;
             d.tag = s.reqs[i].tag;
             d.db = s.reqs[i].db;
-            d.status = q == cudaSuccess ? IMPIR_OK : IMPIR_ECUDA;
+            d.status = q == cudaSuccess && !s.h_hdr->timed_out ? IMPIR_OK : IMPIR_ECUDA;
             d.answer.assign(s.h_out + i * s.record_bytes, s.h_out + (i + 1) * s.record_bytes);
             d.latency_ns = uint64_t(std::chrono::duration_cast<std::chrono::nanoseconds>(now - s.reqs[i].t_submit).count());
             d.batch = uint32_t(s.reqs.size());
@@ -206,6 +207,8 @@ void launch_ready(impir_server* S) {
                                            : IMPIR_ECUDA;
         if (st == IMPIR_OK)
             e = cudaMemcpyAsync(s.h_out, s.d_out, size_t(n) * rb, cudaMemcpyDeviceToHost, s.stream);
+        if (st == IMPIR_OK && e == cudaSuccess)
+            e = cudaMemcpyAsync(s.h_hdr, s.d_ws, sizeof(WsHeader), cudaMemcpyDeviceToHost, s.stream);
         if (st == IMPIR_OK && e == cudaSuccess) e = cudaEventRecord(s.done, s.stream);
         if (st != IMPIR_OK || e != cudaSuccess) {
             for (Request& r : take) {
@@ -275,7 +278,9 @@ impir_status impir_server_create(const impir_server_config* cfg, impir_server** 
         if (e == cudaSuccess) e = cudaMalloc(reinterpret_cast<void**>(&s.d_out), size_t(cfg->max_batch) * stride);
         if (e == cudaSuccess) e = cudaMalloc(reinterpret_cast<void**>(&s.d_ws), s.ws_bytes);
         if (e == cudaSuccess) e = cudaMallocHost(reinterpret_cast<void**>(&s.h_in), kb + size_t(cfg->max_batch) * 4);
-        if (e == cudaSuccess) e = cudaMallocHost(reinterpret_cast<void**>(&s.h_out), size_t(cfg->max_batch) * stride);
+        if (e == cudaSuccess)
+            e = cudaMallocHost(reinterpret_cast<void**>(&s.h_out), size_t(cfg->max_batch) * stride + sizeof(WsHeader));
+        s.h_hdr = reinterpret_cast<WsHeader*>(s.h_out + size_t(cfg->max_batch) * stride);
         if (e != cudaSuccess) {
             cudaGetLastError();
             for (Slot& t : S->slots) free_slot(t);

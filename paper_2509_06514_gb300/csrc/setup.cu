@@ -38,6 +38,7 @@ __global__ void __launch_bounds__(1024) setup_kernel(const SetupParams S) {
         s_nbad = 0;
         s_first_bad = 0xffffffffu;
         hdr->bounds_failed = 0;
+        hdr->timed_out = 0;
 #ifdef IMPIR_BOUNDS
         s_bctx = BoundsCtx{S.bounds, hdr, S.keys, S.keys_bytes, nullptr, 0, 0, 0};
 #endif
@@ -93,25 +94,64 @@ __global__ void __launch_bounds__(1024) setup_kernel(const SetupParams S) {
         }
         s_ngroups = g;
         const unsigned long long tbig = 32ull << S.lane_bits;
-        unsigned long long prev = 0, unit = 0;
         uint32_t nseg = 0;
+        // Tensor-core kernel: the tiles of the prefix that at least tc_min_queries queries reach
+        // (queries are sorted by domain, so that is all records below `split`), if they make enough
+        // units. The split is a multiple of both kernels' tiles (a domain of 2^m >= tbig records, or
+        // the database's end).
+        unsigned long long split = 0, tc_units = 0;
+        constexpr unsigned long long tc_tile = 32ull << kTcLaneBits;
+        const auto covered = [&](uint32_t m) { return S.n_records < (1ull << m) ? S.n_records : 1ull << m; };
+        if (S.group_cap) {
+            unsigned long long prev = 0, units = 0;
+            bool whole = true;  // prev is a place to split at
+            for (uint32_t m = 1; m <= kMaxDomainBits; ++m) {
+                if (hist[m] == 0) continue;
+                const unsigned long long end = covered(m);
+                const uint32_t active = bstart[m] + hist[m];  // queries with domain bits >= m
+                if (active < S.tc_min_queries && whole) break;
+                const unsigned long long lo = (prev > S.rec_lo ? prev : S.rec_lo) / tc_tile;
+                const unsigned long long hi = ((S.rec_hi && S.rec_hi < end ? S.rec_hi : end) + tc_tile - 1) / tc_tile;
+                if (hi > lo) units += (hi - lo) * ((active + S.group_cap - 1) / S.group_cap);
+                if (end > prev) prev = end;
+                whole = prev % tbig == 0 || prev == S.n_records;
+            }
+            if (whole && units >= S.tc_min_units) split = prev;
+        }
+        unsigned long long prev = 0, unit = 0;
+        for (uint32_t m = 1; m <= kMaxDomainBits && prev * tc_tile < split; ++m) {
+            if (hist[m] == 0) continue;
+            const unsigned long long end = covered(m), tiles = (end + tc_tile - 1) / tc_tile;
+            if (tiles <= prev) continue;
+            const uint32_t active = bstart[m] + hist[m];
+            const unsigned long long lo = prev > S.rec_lo / tc_tile ? prev : S.rec_lo / tc_tile;
+            const unsigned long long clip = (S.rec_hi + tc_tile - 1) / tc_tile;
+            const unsigned long long hi = S.rec_hi && clip < tiles ? clip : tiles;
+            if (!IMPIR_IN_BOUNDS(nseg < kMaxSegments, kSiteWorkspace, nseg)) break;
+            if (hi > lo) {
+                const uint32_t groups = (active + S.group_cap - 1) / S.group_cap;
+                segs[nseg++] = SegDesc{lo, tc_units, groups, active, 0};
+                tc_units += (hi - lo) * groups;
+            }
+            prev = tiles;
+        }
+        hdr->tc_counter = 0;
+        hdr->tc_units = tc_units;
+        hdr->tc_segs = nseg;
+        hdr->first_seg = nseg;
+        prev = (split + tbig - 1) / tbig;  // the warp kernels' tiles start here
+        const unsigned long long wlo = S.rec_lo / tbig, whi = (S.rec_hi + tbig - 1) / tbig;
         for (uint32_t m = 1; m <= kMaxDomainBits; ++m) {
             if (hist[m] == 0) continue;
-            const unsigned long long dom = 1ull << m;
-            const unsigned long long n_eff = S.n_records < dom ? S.n_records : dom;
-            const unsigned long long tiles = m >= 5 + S.lane_bits ? (n_eff + tbig - 1) / tbig : 1ull;
+            const unsigned long long tiles = m >= 5 + S.lane_bits ? (covered(m) + tbig - 1) / tbig : 1ull;
             if (tiles > prev) {
                 if (!IMPIR_IN_BOUNDS(nseg < kMaxSegments, kSiteWorkspace, nseg)) break;
                 const uint32_t gcum = gstart[m] + ngrp[m];  // groups with domain bits >= m
                 // clip to the tiles this launch covers (a chunk of a streamed database)
-                const unsigned long long lo = prev > S.tile_lo ? prev : S.tile_lo;
-                const unsigned long long hi = (S.tile_hi == 0 || tiles < S.tile_hi) ? tiles : S.tile_hi;
+                const unsigned long long lo = prev > wlo ? prev : wlo;
+                const unsigned long long hi = (S.rec_hi == 0 || tiles < whi) ? tiles : whi;
                 if (hi > lo) {
-                    segs[nseg].tile_lo = lo;
-                    segs[nseg].unit_lo = unit;
-                    segs[nseg].count = gcum;
-                    segs[nseg].pad = 0;
-                    segs[nseg].pad2 = 0;
+                    segs[nseg] = SegDesc{lo, unit, gcum, 0, 0};
                     unit += (hi - lo) * gcum;
                     ++nseg;
                 }
@@ -123,7 +163,7 @@ __global__ void __launch_bounds__(1024) setup_kernel(const SetupParams S) {
         hdr->n_bad = s_nbad;
         hdr->first_bad = s_first_bad;
         hdr->n_groups = g;
-        hdr->n_segs = nseg;
+        hdr->n_segs = nseg - hdr->first_seg;
     }
     __syncthreads();
 
@@ -136,7 +176,7 @@ __global__ void __launch_bounds__(1024) setup_kernel(const SetupParams S) {
             if (IMPIR_IN_BOUNDS(i < S.n_queries, kSiteWorkspace, i)) perm[i] = q;
         }
     }
-    // 4. group descriptors
+    // 4. group descriptors (the tensor-core kernel takes its groups from the sorted list itself)
     for (uint32_t gi = tid; gi < s_ngroups; gi += nthr) {
         uint32_t m = kMaxDomainBits;
         while (m > 1 && !(gi >= gstart[m] && gi < gstart[m] + ngrp[m])) --m;
@@ -220,8 +260,31 @@ cudaError_t launch_fused(uint32_t qpw, uint32_t nk, dim3 grid, dim3 block, size_
     }
 }
 
+void apply_shape(const XorShape& s, int sms, SetupParams* sp) {
+    sp->lane_bits = s.c.lane_bits;
+    sp->qpw = s.c.queries_per_warp;
+    sp->group_cap = s.tc ? s.tc_cap : 0;
+    sp->tc_min_queries = tc_min_queries(sp->words);
+    sp->tc_min_units = tc_min_units(sp->words, sms);
+}
+
+cudaError_t launch_xor(const XorShape& s, int sms, cudaStream_t st, FusedParams& fp) {
+    if (s.tc) {
+        fp.smem_bytes = tc_smem_bytes();
+        const cudaError_t e = launch_fused_tc(sms, st, fp);
+        if (e != cudaSuccess) return e;
+    }
+    fp.lane_bits = s.c.lane_bits;
+    fp.bits_words = 1u << s.c.lane_bits;
+    const size_t smem = smem_for(s.c);
+    fp.smem_bytes = uint32_t(smem);
+    return launch_fused(s.c.queries_per_warp, nk_xor(fp.words, s.c.queries_per_warp), dim3(sms),
+                        dim3(s.c.warps_per_cta * 32), smem, st, fp);
+}
+
 cudaError_t prepare_xor_kernels() {
     cudaError_t e = prepare_fused_q1();
+    if (e == cudaSuccess) e = prepare_fused_tc();
     if (e == cudaSuccess) e = prepare_fused_q2();
     if (e == cudaSuccess) e = prepare_fused_q4();
     if (e == cudaSuccess) e = prepare_fused_q8();
