@@ -639,7 +639,7 @@ struct AddWalk {
 // Advances the walk by ch leaves (ch >= 2, even): the shares (-1)^party low32(R(m, j)) of the
 // lane's next ch leaves go to shares[lane * ch + 0 .. ch - 1].
 template <int PRF>
-__device__ __forceinline__ void add_walk_chunk(const FusedParams& P, const uint8_t* kq, uint32_t m, uint32_t D,
+__device__ __forceinline__ void add_walk_chunk(const uint8_t* kq, uint32_t m, uint32_t D,
                                                uint32_t sq, AddWalk& w, uint32_t ch, uint32_t* shares, uint32_t lane,
                                                uint32_t L, uint32_t neg) {
     Blk node = w.node;
@@ -735,9 +735,9 @@ __device__ __forceinline__ void unit_add(const FusedParams& P, const GroupDesc& 
             if (uint32_t(q) < count) {
                 const uint8_t* kq = query_key(P, query_at(P, qidx, q));
                 if (kq[1] == 0)
-                    add_walk_chunk<0>(P, kq, m, D, sq, w[q], ch, shares + q * qstride, lane, L, neg[q]);
+                    add_walk_chunk<0>(kq, m, D, sq, w[q], ch, shares + q * qstride, lane, L, neg[q]);
                 else
-                    add_walk_chunk<1>(P, kq, m, D, sq, w[q], ch, shares + q * qstride, lane, L, neg[q]);
+                    add_walk_chunk<1>(kq, m, D, sq, w[q], ch, shares + q * qstride, lane, L, neg[q]);
             }
         __syncwarp();
         scan_chunk_add<QC, NK>(P, tile_base, nrec, shares, qstride, count, qidx, runs, run_len, sq, c * ch, acc_out,
@@ -809,7 +809,40 @@ __device__ __forceinline__ void scan_tile(const FusedParams& P, uint64_t tile_ba
 #pragma unroll
         for (int q = 0; q < QC; ++q) acc[q] = make_uint4(0, 0, 0, 0);
         const uint4* base = P.db + (tile_base - P.rec_lo) * W + lk;
-        for (uint32_t c0 = 0; c0 < nrec; c0 += 32) {
+        if constexpr (QC <= 2) {
+            // One or two queries: the scan is bound by memory latency, not by its XORs (one query reads
+            // 32 bytes of records for every AES block at 64-byte records, 128 at 256). 16 (8) loads in
+            // flight per lane, and records that no query selects are not read at all.
+            constexpr int LB = QC == 1 ? 16 : 8;
+#pragma unroll 1
+            for (uint32_t r0 = 0; r0 < nrec; r0 += LB * R) {
+                uint4 v[LB];
+                uint32_t pick[QC];  // bit u: the query selects this lane's u-th record
+#pragma unroll
+                for (int q = 0; q < QC; ++q) pick[q] = 0;
+#pragma unroll
+                for (int u = 0; u < LB; ++u) {
+                    const uint32_t rec = r0 + u * R + lr;
+                    v[u] = make_uint4(0, 0, 0, 0);
+                    if (on && rec < nrec) {
+                        bool any = false;
+#pragma unroll
+                        for (int q = 0; q < QC; ++q) {
+                            const uint32_t b = (ld_slice(&bits[q * bw + (rec >> 5)]) >> (rec & 31)) & 1u;
+                            pick[q] |= b << u;
+                            any |= b != 0;
+                        }
+                        if (any) v[u] = ld_db(base + size_t(rec) * W);
+                    }
+                }
+#pragma unroll
+                for (int u = 0; u < LB; ++u)
+#pragma unroll
+                    for (int q = 0; q < QC; ++q)
+                        if (QC == 1 || (pick[q] >> u & 1u)) acc[q] = bxor4(acc[q], v[u]);
+            }
+        }
+        for (uint32_t c0 = 0; QC > 2 && c0 < nrec; c0 += 32) {
             uint32_t sel[QC];
 #pragma unroll
             for (int q = 0; q < QC; ++q) sel[q] = ld_slice(&bits[q * bw + (c0 >> 5)]) >> lr;  // bit i*R: record c0+i*R+lr
@@ -900,11 +933,18 @@ __device__ __forceinline__ void scan_tile(const FusedParams& P, uint64_t tile_ba
                 for (int q = 0; q < QC; ++q) sh[q] = __brev(sel[q]);
                 for (uint32_t i0 = 0; i0 < nloc; i0 += RB) {
                     uint4 v[RB][NK];
+                    // (one or two queries: records that none selects are not read)
+                    uint32_t want = 0xffffffffu;
+                    if constexpr (QC <= 2) {
+                        want = sel[0];
+#pragma unroll
+                        for (int q = 1; q < QC; ++q) want |= sel[q];
+                    }
 #pragma unroll
                     for (int u = 0; u < RB; ++u)
 #pragma unroll
                         for (int c = 0; c < NK; ++c)
-                            v[u][c] = (kon[c] && i0 + u < nloc) ? ld_db(rp + size_t(i0 + u) * W + 32 * c)
+                            v[u][c] = (kon[c] && i0 + u < nloc && (want >> (i0 + u) & 1u)) ? ld_db(rp + size_t(i0 + u) * W + 32 * c)
                                                                 : make_uint4(0, 0, 0, 0);
                     if constexpr (NK <= 2) {
 #pragma unroll
@@ -998,7 +1038,7 @@ __global__ void __launch_bounds__((NK == 1 && QC <= 8) ? 640 : 512, 1)
 #endif
     SegDesc* segs = reinterpret_cast<SegDesc*>(g_smem + kTableBytes);
     uint32_t n_segs = hdr->n_segs;
-    const uint32_t first_seg = hdr->first_seg;
+    const uint32_t first_seg = hdr->first_seg, lane_bits = hdr->lane_bits;
     if (!IMPIR_IN_BOUNDS(first_seg + n_segs <= kMaxSegments, kSiteSchedule, n_segs)) n_segs = 0;
     const SegDesc* gsegs = reinterpret_cast<const SegDesc*>(P.ws + P.lay.off_segs) + first_seg;
     for (uint32_t i = tid; i < n_segs; i += nthr) segs[i] = gsegs[i];
@@ -1011,9 +1051,17 @@ __global__ void __launch_bounds__((NK == 1 && QC <= 8) ? 640 : 512, 1)
     uint32_t* bits = reinterpret_cast<uint32_t*>(g_smem + kTableBytes + kSegSmemBytes) + warp * QC * P.bits_words;
     const uint32_t L = lane * 4;
 
+    // a warp's first unit is fixed, SM by SM (where the batch has fewer units than the grid has warps
+    // they spread evenly over the SMs), the later ones come from the counter
+    uint32_t taken = 0;
+#pragma unroll 1
     for (;;) {
         unsigned long long u = 0;
-        if (lane == 0) u = atomicAdd(&hdr->counter, 1ull);
+        if (lane == 0)
+            u = taken ? gridDim.x * (nthr >> 5) + atomicAdd(&hdr->counter, 1ull)
+                      : (unsigned long long)warp * gridDim.x + blockIdx.x;
+        taken = 1;
+        asm volatile("" : "+r"(taken));  // (keeps the compiler from peeling the first unit: twice the code)
         u = __shfl_sync(0xffffffffu, u, 0);
         if (u >= n_units) break;
         uint32_t j = 0;
@@ -1021,11 +1069,20 @@ __global__ void __launch_bounds__((NK == 1 && QC <= 8) ? 640 : 512, 1)
         const unsigned long long off = u - segs[j].unit_lo;
         const unsigned long long tile = segs[j].tile_lo + off / segs[j].count;
         const uint32_t gi = uint32_t(off % segs[j].count);
-        if (!IMPIR_IN_BOUNDS(gi < hdr->n_groups, kSiteSchedule, gi)) continue;
-        const GroupDesc gd = groups[gi];
+        GroupDesc gd;
+        if (MODE == 0 && segs[j].active) {
+            // domains of at least one tile, of any mix of sizes: the queries at these sorted positions
+            gd = {gi * QC, min(uint32_t(QC), segs[j].active - gi * QC), kMaxDomainBits, 0};
+            if (!IMPIR_IN_BOUNDS(gi * QC < segs[j].active, kSiteSchedule, gi)) continue;
+        } else {
+            if (!IMPIR_IN_BOUNDS(gi < hdr->n_groups, kSiteSchedule, gi)) continue;
+            gd = groups[gi];
+        }
 
+        // m, D and Dt are the group's (a mixed group: those of the largest domain, which give the
+        // tile's shape); each query's own follow from its key
         const uint32_t m = gd.m;
-        const uint32_t sq = m >= 5 ? min(P.lane_bits, m - 5) : 0u;
+        const uint32_t sq = m >= 5 ? min(lane_bits, m - 5) : 0u;
         const uint32_t D = m - sq;
         const unsigned long long dom = 1ull << m;
         const unsigned long long n_eff = P.n_records < dom ? P.n_records : dom;
@@ -1037,12 +1094,12 @@ __global__ void __launch_bounds__((NK == 1 && QC <= 8) ? 640 : 512, 1)
         const bool lane_on = lane < lanes && (sub << sq) < n_eff;
         const uint32_t nwords = uint32_t((TT + 31) >> 5);
 
-        // Cooperative walk (selection-bit answers, lane subtrees of >= 64 leaves, at most 8
+        // Cooperative walk (selection-bit answers, at most 8
         // queries per warp: with 16 the kernel sits at its register limit and runs slower): the warp
         // expands the 5 levels between the warp-tile root and the lane subtree roots for all
         // the group's queries at once, level by level, in place in the (not yet used) bit area;
         // otherwise each lane walks them itself for every query.
-        const bool coop = MODE == 0 && QC <= 8 && P.bits_words >= 64 && m >= 5;
+        const bool coop = MODE == 0 && QC <= 8 && m >= 5;
         if (MODE == 0 && !coop) {
             for (int q = 0; q < QC; ++q)
                 for (uint32_t w = lane; w < nwords; w += 32)
@@ -1057,12 +1114,13 @@ __global__ void __launch_bounds__((NK == 1 && QC <= 8) ? 640 : 512, 1)
         Blk top{0, 0, 0, 0};
         if (lane < gd.count) {
             const uint8_t* kq = query_key(P, query_at(P, qidx, lane));
-            top = cw_load(kq, m, 0, 0, 0);  // R(0,0) = C_0[0][0], Eq. (2)
+            const uint32_t mq = kq[2], dt = mq > sq + 5 ? mq - sq - 5 : 0;
+            top = cw_load(kq, mq, 0, 0, 0);  // R(0,0) = C_0[0][0], Eq. (2)
 #pragma unroll 1
-            for (uint32_t d = 1; d <= Dt; ++d) {
-                const uint32_t x = uint32_t(tile >> (Dt - d)) & 1u;
+            for (uint32_t d = 1; d <= dt; ++d) {
+                const uint32_t x = uint32_t(tile >> (dt - d)) & 1u;
                 const Blk f = kq[1] == 0 ? keyed_one(top, x, L) : mmo_one(top, x, L, c_mmo.rk);
-                top = bxor(f, cw_load(kq, m, top.x & 1u, x, d));
+                top = bxor(f, cw_load(kq, mq, top.x & 1u, x, d));
             }
         }
         if constexpr (MODE == 1) {
@@ -1093,8 +1151,8 @@ __global__ void __launch_bounds__((NK == 1 && QC <= 8) ? 640 : 512, 1)
                     if (act) {
                         const uint8_t* kq = query_key(P, query_at(P, qidx, q));
                         const Blk par{pv.x, pv.y, pv.z, pv.w};
-                        const uint32_t t = par.x & 1u, d = Dt + k + 1;
-                        const Blk c0 = cw_load(kq, m, t, 0, d), c1 = cw_load(kq, m, t, 1, d);
+                        const uint32_t mq = kq[2], t = par.x & 1u, d = mq - sq - 5 + k + 1;
+                        const Blk c0 = cw_load(kq, mq, t, 0, d), c1 = cw_load(kq, mq, t, 1, d);
                         Blk a, b;
                         if (kq[1] == 0)
                             keyed_pair(par, L, c0, c1, a, b);
@@ -1111,7 +1169,7 @@ __global__ void __launch_bounds__((NK == 1 && QC <= 8) ? 640 : 512, 1)
 #pragma unroll 1
             for (uint32_t qi = 0; qi < gd.count; ++qi) {
                 const uint8_t* kq = query_key(P, query_at(P, qidx, qi));
-                const uint32_t prf = kq[1];
+                const uint32_t prf = kq[1], mq = kq[2], Dq = mq - sq;
                 // lane l's parent at level 4 is node l >> 1; its subtree root is child l & 1
                 uint4 pv = make_uint4(0, 0, 0, 0);
                 if (slice_ok(nodes + qi * slot + (lane >> 1) * 16, 16))
@@ -1123,23 +1181,23 @@ __global__ void __launch_bounds__((NK == 1 && QC <= 8) ? 640 : 512, 1)
                 const Blk start{pv.x, pv.y, pv.z, pv.w};
                 if (lane_on) {
                     if (prf == 0)
-                        lane_eval<0>(kq, m, D, sub, sq, bits + qi * P.bits_words, lane, L, start, D - 1);
+                        lane_eval<0>(kq, mq, Dq, sub, sq, bits + qi * P.bits_words, lane, L, start, Dq - 1);
                     else
-                        lane_eval<1>(kq, m, D, sub, sq, bits + qi * P.bits_words, lane, L, start, D - 1);
+                        lane_eval<1>(kq, mq, Dq, sub, sq, bits + qi * P.bits_words, lane, L, start, Dq - 1);
                 }
             }
         } else {
 #pragma unroll 1
             for (uint32_t qi = 0; qi < gd.count; ++qi) {
                 const uint8_t* kq = query_key(P, query_at(P, qidx, qi));
-                const uint32_t prf = kq[1];
+                const uint32_t prf = kq[1], mq = kq[2], Dq = mq - sq;
                 const Blk start{__shfl_sync(0xffffffffu, top.x, qi), __shfl_sync(0xffffffffu, top.y, qi),
                                 __shfl_sync(0xffffffffu, top.z, qi), __shfl_sync(0xffffffffu, top.w, qi)};
                 if (lane_on) {
                     if (prf == 0)
-                        lane_eval<0>(kq, m, D, sub, sq, bits + qi * P.bits_words, lane, L, start, Dt);
+                        lane_eval<0>(kq, mq, Dq, sub, sq, bits + qi * P.bits_words, lane, L, start, mq > sq + 5 ? mq - sq - 5 : 0);
                     else
-                        lane_eval<1>(kq, m, D, sub, sq, bits + qi * P.bits_words, lane, L, start, Dt);
+                        lane_eval<1>(kq, mq, Dq, sub, sq, bits + qi * P.bits_words, lane, L, start, mq > sq + 5 ? mq - sq - 5 : 0);
                 }
             }
         }

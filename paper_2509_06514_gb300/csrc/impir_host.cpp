@@ -284,6 +284,7 @@ impir_status launch_batch(const DeviceState& dev, const Db& db, const impir_conf
     sp.n_queries = n;
     sp.words = db.stride / 16;
     apply_shape(shape, dev.sms, &sp);
+    sp.mixed = mode == 0;
     sp.rec_lo = shard ? db.row_lo : 0;
     sp.rec_hi = shard ? db.row_lo + db.n : 0;
     sp.bounds = bounds_record();
@@ -315,7 +316,6 @@ impir_status launch_batch(const DeviceState& dev, const Db& db, const impir_conf
         CK(launch_xor(shape, dev.sms, st, fp), "fused kernel launch");
     } else {
         const size_t smem = smem_add(cfg);
-        fp.lane_bits = cfg.lane_bits;
         fp.bits_words = add_share_words(cfg);
         fp.smem_bytes = uint32_t(smem);
         CK(launch_fused_add(cfg.queries_per_warp, nk_need(fp.words), dim3(dev.sms), dim3(cfg.warps_per_cta * 32), smem,

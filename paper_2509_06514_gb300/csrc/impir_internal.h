@@ -37,7 +37,8 @@ struct WsHeader {
     unsigned long long tc_counter, tc_units;
     uint32_t tc_segs;
     uint32_t first_seg;           // the warp kernel's first segment (it has n_segs of them)
-    uint32_t pad[48];
+    uint32_t lane_bits;           // of the warp kernels' tiles: at most the launch shape's
+    uint32_t pad[47];
 };
 static_assert(sizeof(WsHeader) == 256, "header is 256 bytes");
 
@@ -52,8 +53,8 @@ struct GroupDesc {
 
 // Work units u in [unit_lo, next segment's unit_lo) cover warp tiles
 // tile_lo + (u - unit_lo) / count with groups (u - unit_lo) % count. `active` is the number of
-// sorted queries whose domains reach these tiles (the tensor-core kernel cuts them into `count`
-// groups of equal size by itself).
+// sorted queries whose domains reach these tiles, which the kernels cut into `count` groups by
+// themselves (0: the groups are listed in descriptors).
 struct SegDesc {
     unsigned long long tile_lo;
     unsigned long long unit_lo;
@@ -133,43 +134,61 @@ inline uint32_t nk_xor(uint32_t words, uint32_t qpw) {
 // with one column pass (records of at most 512 bytes) and at most 8 queries per warp, else 16.
 inline uint32_t max_warps(uint32_t qpw, uint32_t words) { return nk_need(words) == 1 && qpw <= 8 ? 20u : 16u; }
 
+// 32-bit words of a query's slot in a warp's bit area: its selection bits, or the 16 nodes that the
+// cooperative walk (at most 8 queries per warp) keeps there before.
+inline uint32_t bits_words(const impir_config& c) {
+    return std::max(1u << c.lane_bits, c.queries_per_warp <= 8 ? 64u : 1u);
+}
+
 // Dynamic shared memory of the XOR kernels: T-tables, segment table, per-warp selection bits.
 inline size_t smem_for(const impir_config& c) {
-    return kTableBytes + kSegSmemBytes + size_t(c.warps_per_cta) * c.queries_per_warp * (size_t(1) << c.lane_bits) * 4;
+    return kTableBytes + kSegSmemBytes + size_t(c.warps_per_cta) * c.queries_per_warp * bits_words(c) * 4;
 }
 
-// Largest lane_bits that keeps enough warp tiles for every warp of the grid busy.
-inline impir_config default_config_warps(uint64_t n_records, uint32_t words, uint32_t n_queries, int sms,
-                                         uint32_t warps) {
-    impir_config c{};
-    c.warps_per_cta = warps;
-    c.queries_per_launch = 0;
-    uint32_t qpw = 8;
-    while (qpw > 1 && (qpw * nk_xor(words, qpw) > 16 || qpw > n_queries)) qpw >>= 1;
-    c.queries_per_warp = qpw;
-    const double all_warps = double(sms) * c.warps_per_cta;
-    const double groups = std::ceil(double(n_queries) / qpw);
-    c.lane_bits = 0;
-    for (uint32_t s = kMaxLaneBits; s + 1 > 0; --s) {
-        impir_config t = c;
-        t.lane_bits = s;
-        if (smem_for(t) > kSmemMax) continue;
-        const double tiles = std::ceil(double(n_records) / double(32ull << s));
-        if (groups * tiles >= 3.0 * all_warps || s == 0) {
-            c.lane_bits = s;
-            break;
-        }
-    }
-    if (c.lane_bits > 8) c.lane_bits = 8;
-    return c;
+// Estimated time of a batch in the shape c, in SM clocks. A unit (a warp tile for a group of queries)
+// costs `steps` node pairs of a warp: the walk to the tile, the cooperative levels and the lanes'
+// subtrees, and the scan's share of the ALU pipe. A pair takes about 330 clocks of an SM's time for
+// each warp that runs there (the lookups' shared-memory port) plus 700 of latency; units go to the
+// warps whole, so the last, partly filled round counts in full.
+// The scan's reads: every group reads the tiles it covers, the first from HBM, the others from L2 if
+// the tiles in work at a time fit there.
+inline double shape_clocks(const impir_config& c, uint64_t n_records, uint32_t words, uint32_t n_queries, int sms) {
+    const double slots = c.queries_per_warp, s = c.lane_bits;
+    const double groups = std::ceil(n_queries / slots), tiles = std::ceil(double(n_records) / double(32ull << c.lane_bits));
+    const double q = n_queries / groups, m = std::ceil(std::log2(double(n_records)));
+    double coop = 0;
+    for (int k = 0; k < 4; ++k) coop += 1.3 * std::ceil(q * double(1 << k) / 32);
+    const double lane = q * (0.8 + std::exp2(s) - 1);
+    const double scan = std::exp2(s) * words * (4.3 * slots + 4) / 560;
+    const double steps = (std::max(0.0, m - s - 5) + coop + lane + scan) * (1 + 0.012 * slots);
+    const double units = groups * tiles;
+    const double w = c.warps_per_cta, full = std::floor(units / (sms * w));
+    const double rest = std::ceil((units - full * sms * w) / sms);
+    const double pairs = full * (330 * w + 700) + (rest > 0 ? 330 * rest + (full > 0 ? 1400 : 700) : 0);
+    const double record = words * 16.0 * (c.queries_per_warp == 1 ? 0.5 : 1.0), pass = double(n_records) * record;
+    const double live = std::min(units, sms * w) / groups * double(32ull << c.lane_bits) * record;
+    const double mem = pass * (groups > 1 && live > 64e6 ? groups : 1.0) / 3300 + pass * groups / 5000;
+    return steps * pairs + mem;
 }
 
-// 20 warps per CTA where the kernel allows it and the lane subtrees stay as large as with 16.
+// The shape with the smallest estimate (lane subtrees of at most 2^8 leaves).
 inline impir_config default_config(uint64_t n_records, uint32_t words, uint32_t n_queries, int sms) {
-    const impir_config c16 = default_config_warps(n_records, words, n_queries, sms, 16);
-    if (max_warps(c16.queries_per_warp, words) < 20) return c16;
-    const impir_config c20 = default_config_warps(n_records, words, n_queries, sms, 20);
-    return c20.lane_bits == c16.lane_bits && c20.queries_per_warp == c16.queries_per_warp ? c20 : c16;
+    impir_config best{};
+    double best_t = 0;
+    for (uint32_t qpw = 1; qpw <= 8; qpw *= 2) {
+        if (qpw * nk_xor(words, qpw) > 16 || (qpw > 1 && qpw / 2 >= n_queries)) continue;
+        for (uint32_t w = 16; w <= max_warps(qpw, words); w += 4)
+            for (uint32_t b = 0; b <= 8; ++b) {
+                const impir_config c{b, qpw, w, 0};
+                if (smem_for(c) > kSmemMax) continue;
+                const double t = shape_clocks(c, n_records, words, n_queries, sms);
+                if (best_t == 0 || t < best_t) {
+                    best_t = t;
+                    best = c;
+                }
+            }
+    }
+    return best;
 }
 
 // ---- the tensor-core form of the XOR answer (fused_tc.cu) ----
@@ -198,6 +217,7 @@ struct XorShape {
     impir_config c;
     bool tc;
     uint32_t tc_cap;
+    uint64_t want_units;  // see SetupParams
     // tiles of both kernels divide 32 << tile_bits() records
     uint32_t tile_bits() const { return tc ? std::max(kTcLaneBits, c.lane_bits) : c.lane_bits; }
 };
@@ -205,7 +225,12 @@ struct XorShape {
 // tc_allowed: the caller set no launch shape of its own.
 inline XorShape xor_shape(const impir_config& c, bool tc_allowed, uint64_t n_records, uint32_t words,
                           uint32_t n_queries, int sms) {
-    XorShape s{c, false, 0};
+    XorShape s{c, false, 0, 0};
+    // as many units as a batch that covers the database has, but 16 per SM are enough
+    const uint64_t T = 32ull << c.lane_bits;
+    if (tc_allowed)
+        s.want_units = std::min<uint64_t>(16ull * sms, ((n_records + T - 1) / T) *
+                                                           ((n_queries + c.queries_per_warp - 1) / c.queries_per_warp));
     if (!tc_allowed || c.queries_per_launch != 0 || n_queries < tc_min_queries(words)) return s;
     const uint64_t groups = (n_queries + kTcQueries - 1) / kTcQueries;
     if (groups * ((n_records + (32u << kTcLaneBits) - 1) >> (kTcLaneBits + 5)) < tc_min_units(words, sms)) return s;
@@ -224,6 +249,8 @@ struct SetupParams {
     uint32_t words;          // stride / 16
     uint32_t lane_bits;
     uint32_t qpw;            // queries per warp (group size)
+    uint32_t mixed;          // groups mix domain sizes (the XOR answer)
+    unsigned long long want_units;  // units the launch shape was chosen for (0: lane_bits as it is)
     uint32_t group_cap;      // most queries of a tensor-core unit (0: the warp kernels take the whole batch)
     uint32_t tc_min_queries; // see tc_min_queries() and tc_min_units()
     unsigned long long tc_min_units;
@@ -247,7 +274,6 @@ struct FusedParams {
     uint64_t n_records;
     uint32_t n_queries;
     uint32_t words;          // uint4 words per record (stride / 16)
-    uint32_t lane_bits;
     uint32_t bits_words;     // 32-bit words of selection bits (additive: shares) per (warp, query slot)
     unsigned long long rec_lo;  // global index of the record at db[0] (0 unless a chunk or a row shard)
     // extents for the debug build's index checks
