@@ -31,22 +31,13 @@ __global__ void __launch_bounds__(512, 1) aes_bench_kernel(const __grid_constant
                                                            uint4* out, uint32_t iters, uint32_t n_threads) {
     const uint32_t tid = threadIdx.x, nthr = blockDim.x;
 #ifdef IMPIR_BOUNDS
-    if (tid == 0) s_bctx = BoundsCtx{P.bounds, nullptr, nullptr, 0, nullptr, 0, kTableBytes, 0};
+    if (tid == 0) s_bctx = BoundsCtx{P.bounds, nullptr, nullptr, 0, nullptr, 0, kHighAt - kSmemBase, 0, 0};
 #endif
-    for (uint32_t i = tid; i < 256 * 32; i += nthr) {
-        const uint32_t x = i >> 5, l = i & 31;
-        const uint32_t t0 = __ldg(P.te0 + x);
-        uint32_t* ra = reinterpret_cast<uint32_t*>(g_smem + x * 256);
-        uint32_t* rb = reinterpret_cast<uint32_t*>(g_smem + 65536 + x * 256);
-        ra[l] = t0;
-        ra[32 + l] = __funnelshift_l(t0, t0, 8);
-        rb[l] = __funnelshift_l(t0, t0, 16);
-        rb[32 + l] = __funnelshift_l(t0, t0, 24);
-    }
+    if (!fill_tables(P.te0, tid, nthr)) return;
     __syncthreads();
     const uint32_t g = blockIdx.x * blockDim.x + tid;
     if (g >= n_threads) return;
-    const uint32_t L = (tid & 31) * 4;
+    const uint32_t L = lane_base(tid & 31);
     const uint4 s0 = seeds[g];
     Blk p{s0.x, s0.y, s0.z, s0.w};
     const Blk zero{0, 0, 0, 0};
@@ -280,13 +271,13 @@ extern "C" impir_status impir_aes_calibrate(int prf, uint32_t iters, uint32_t n_
         fp.bounds = bounds_record();
         const unsigned blocks = (n_threads + threads_per_cta - 1) / threads_per_cta;
         auto k = prf == 0 ? aes_bench_kernel<0> : aes_bench_kernel<1>;
-        e = cudaFuncSetAttribute(k, cudaFuncAttributeMaxDynamicSharedMemorySize, int(kTableBytes));
+        e = cudaFuncSetAttribute(k, cudaFuncAttributeMaxDynamicSharedMemorySize, int(kHighAt - kSmemBase));
         if (e == cudaSuccess) {
-            k<<<blocks, threads_per_cta, kTableBytes>>>(fp, d_seeds, d_out, 1, n_threads);  // warm-up
+            k<<<blocks, threads_per_cta, kHighAt - kSmemBase>>>(fp, d_seeds, d_out, 1, n_threads);  // warm-up
             e = cudaEventRecord(e0);
         }
         if (e == cudaSuccess) {
-            k<<<blocks, threads_per_cta, kTableBytes>>>(fp, d_seeds, d_out, iters, n_threads);
+            k<<<blocks, threads_per_cta, kHighAt - kSmemBase>>>(fp, d_seeds, d_out, iters, n_threads);
             e = cudaGetLastError();
         }
         if (e == cudaSuccess) e = cudaEventRecord(e1);

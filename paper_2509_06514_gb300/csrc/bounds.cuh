@@ -25,6 +25,7 @@ struct BoundsCtx {
     unsigned long long db_words;
     uint32_t smem_bytes;             // dynamic shared memory of the launch
     uint32_t warp_slice_bytes;       // each warp's slice of the bit / node / share buffer
+    uint32_t slices_low;             // slices below the tables
 };
 
 __shared__ BoundsCtx s_bctx;

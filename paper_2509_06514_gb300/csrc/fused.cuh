@@ -32,6 +32,13 @@
 // one PRMT builds it from the state word, and the 32 lanes of a warp always hit 32 distinct
 // banks. Region A holds Te0|Te1, region B Te2|Te3 (128 KiB). S-box values are read from the
 // byte of a T-table entry that equals S[x] (Te2 byte 0, Te3 byte 1, Te0 byte 2, Te1 byte 3).
+//
+// The tables stand at a fixed shared-memory address, 64 KiB: the PRMT that puts the state byte into
+// address byte 1 and the lane into byte 0 also puts a 1 into byte 2, and the lookup is one load at
+// that register plus a constant. With the tables at the start of the dynamic shared memory, an
+// address only the linker knows, the compiler spent an integer add on the FMA pipe per lookup in
+// most kernels: 635 instructions per AES block against 485 (26 queries on 2^22 one-byte records:
+// 4.11 ms, with the fixed address 3.67). Everything else lies below and above the tables.
 #pragma once
 
 #include <atomic>
@@ -44,14 +51,51 @@ namespace impir {
 
 extern __shared__ __align__(16) uint8_t g_smem[];
 
+__device__ __forceinline__ uint32_t smem32(const void* p) { return uint32_t(__cvta_generic_to_shared(p)); }
+
+// The dynamic shared memory at a shared-memory address.
+__device__ __forceinline__ uint8_t* smem_at(uint32_t addr) { return g_smem + (addr - smem32(g_smem)); }
+
+// Fills the replicated T-tables from the 256 entries of Te0 (all threads of the block; the caller
+// synchronizes). False if the shared memory does not begin where the launch's size assumes.
+__device__ __forceinline__ bool fill_tables(const uint32_t* te0, uint32_t tid, uint32_t nthr) {
+    const uint32_t base = smem32(g_smem);
+#ifdef IMPIR_BOUNDS
+    if (base < kSmemBase || base > kSmemBase + kSmemStatic) return false;
+#else
+    if (base != kSmemBase) return false;
+#endif
+    for (uint32_t i = tid; i < 256 * 32; i += nthr) {
+        const uint32_t x = i >> 5, l = i & 31;
+        const uint32_t t0 = __ldg(te0 + x);
+        uint32_t* ra = reinterpret_cast<uint32_t*>(smem_at(kTableAt + x * 256));
+        uint32_t* rb = reinterpret_cast<uint32_t*>(smem_at(kTableAt + 65536 + x * 256));
+        ra[l] = t0;
+        ra[32 + l] = __funnelshift_l(t0, t0, 8);
+        rb[l] = __funnelshift_l(t0, t0, 16);
+        rb[32 + l] = __funnelshift_l(t0, t0, 24);
+    }
+    return true;
+}
+
+// What tix() joins with a state byte: the lane's offset in a table row and byte 2 of the tables'
+// address. Volatile, so that no lookup (which needs it) moves above the barrier after fill_tables.
+__device__ __forceinline__ uint32_t lane_base(uint32_t lane) {
+    uint32_t v = lane * 4 | (kTableAt >> 8);
+    asm volatile("" : "+r"(v)::"memory");
+    return v;
+}
+
 // Debug build: n bytes at p lie inside the calling warp's slice of the bit / node / share
 // buffer (and inside the launch's dynamic shared memory).
 __device__ __forceinline__ bool slice_ok(const void* p, uint32_t n) {
 #ifdef IMPIR_BOUNDS
     const long long o = static_cast<const uint8_t*>(p) - g_smem;
-    const long long lo = kTableBytes + kSegSmemBytes + (long long)(threadIdx.x >> 5) * s_bctx.warp_slice_bytes;
-    return IMPIR_IN_BOUNDS(o >= lo && o + n <= lo + s_bctx.warp_slice_bytes && o + n <= s_bctx.smem_bytes, kSiteBits,
-                           o);
+    const uint32_t warp = threadIdx.x >> 5, low = s_bctx.slices_low;
+    const long long lo = warp < low ? kSegSmemBytes + (long long)warp * s_bctx.warp_slice_bytes
+                                    : kHighAt - smem32(g_smem) + (long long)(warp - low) * s_bctx.warp_slice_bytes;
+    const long long end = warp < low ? kTableAt - smem32(g_smem) : s_bctx.smem_bytes;
+    return IMPIR_IN_BOUNDS(o >= lo && o + n <= lo + s_bctx.warp_slice_bytes && o + n <= end, kSiteBits, o);
 #else
     return true;
 #endif
@@ -66,16 +110,25 @@ struct Blk {
 
 __device__ __forceinline__ Blk bxor(const Blk a, const Blk b) { return {a.x ^ b.x, a.y ^ b.y, a.z ^ b.z, a.w ^ b.w}; }
 
-// Byte offset of lane L's copy of Te[byte b of w]: (byte << 8) | lane4.
-__device__ __forceinline__ uint32_t tix(uint32_t w, uint32_t lane4, int b) {
-    return __byte_perm(w, lane4, 0x5504u | (uint32_t(b) << 4));
+// Shared-memory address of the lane's copy of Te[byte b of w] (first table): lane base's bytes 0, 1
+// and 3 (zero) in bytes 0, 2 and 3, the state byte in byte 1.
+__device__ __forceinline__ uint32_t tix(uint32_t w, uint32_t lbase, int b) {
+    return __byte_perm(w, lbase, 0x7504u | (uint32_t(b) << 4));
 }
 
 template <int K>
-__device__ __forceinline__ uint32_t T(uint32_t off) {
-    const uint32_t o = off + (K & 1) * 128 + (K >> 1) * 65536;
-    if (!IMPIR_IN_BOUNDS(o + 4 <= kTableBytes, kSiteTable, o)) return 0;
-    return *reinterpret_cast<const uint32_t*>(g_smem + o);
+__device__ __forceinline__ uint32_t T(uint32_t addr) {
+    constexpr uint32_t table = (K & 1) * 128 + (K >> 1) * 65536;
+    if (!IMPIR_IN_BOUNDS(addr >= kTableAt && addr + table + 4 <= kHighAt, kSiteTable, addr)) return 0;
+#if defined(IMPIR_TABLE_POINTER) && !defined(IMPIR_BOUNDS)
+    // the tensor-core kernel, whose walk got no address adds this way either: 64 queries on 2^20 records
+    // of 256 bytes take 2.60 ms, with the load below 2.66, the warp kernels 3 to 11 % more with this one
+    return *reinterpret_cast<const uint32_t*>(g_smem + (addr - kSmemBase) + table);
+#else
+    uint32_t v;
+    asm("ld.shared.u32 %0, [%1+%2];" : "=r"(v) : "r"(addr), "n"(table));
+    return v;
+#endif
 }
 
 // One full round: SubBytes, ShiftRows, MixColumns, AddRoundKey (FIPS-197 §5.1).
@@ -558,38 +611,55 @@ __device__ __forceinline__ void scan_chunk_add(const FusedParams& P, uint64_t ti
     }
 }
 
-// Selection bits of lane's subtree: root -> depth D walk (Eq. (3) one edge per level), then
-// a depth-first expansion down to the leaves at depth m; bit r of `bits` (relative to the
-// warp tile) is lsb(R(m, tile_first_leaf + r)).
-// The walk starts from `start`, the node at depth d0 on the lane's path (the root with d0 = 0,
-// or the warp-tile root the warp computed once for this query).
+// ---- tree steps, Eq. (3) ----
+// The subtree walk is a function of its own, so that the kernels hold its rounds once and it has
+// registers of its own; the other two, used at the walks' tops, measured the same either way.
+
+// Child x of node n of key kq (domain bits m); the child is at depth d.
 template <int PRF>
-__device__ __forceinline__ Blk walk_down(const uint8_t* kq, uint32_t m, uint32_t D, uint64_t sub,
-                                         uint32_t L, const Blk start, uint32_t d0) {
-    Blk node = start;
-#pragma unroll 1
-    for (uint32_t d = d0 + 1; d <= D; ++d) {
-        const uint32_t x = uint32_t(sub >> (D - d)) & 1u;
-        const uint32_t t = node.x & 1u;
-        const Blk c = cw_load(kq, m, t, x, d);
-        const Blk f = PRF == 0 ? keyed_one(node, x, L) : mmo_one(node, x, L, c_mmo.rk);
-        node = bxor(f, c);
-    }
-    return node;
+__device__ __forceinline__ Blk child_node(const uint8_t* kq, uint32_t m, Blk n, uint32_t x, uint32_t d, uint32_t L) {
+    const Blk c = cw_load(kq, m, n.x & 1u, x, d);
+    return bxor(PRF == 0 ? keyed_one(n, x, L) : mmo_one(n, x, L, c_mmo.rk), c);
 }
 
+__device__ __forceinline__ Blk child_node(uint32_t prf, const uint8_t* kq, uint32_t m, Blk n, uint32_t x, uint32_t d,
+                                          uint32_t L) {
+    return prf == 0 ? child_node<0>(kq, m, n, x, d, L) : child_node<1>(kq, m, n, x, d, L);
+}
+
+struct NodePair {
+    Blk a, b;
+};
+
+// Both children, at depth d.
 template <int PRF>
-__device__ __forceinline__ void lane_eval(const uint8_t* kq, uint32_t m, uint32_t D,
-                                          uint64_t sub, uint32_t sq, uint32_t* bits, uint32_t lane, uint32_t L,
-                                          const Blk start, uint32_t d0) {
-    Blk node = walk_down<PRF>(kq, m, D, sub, L, start, d0);
-    if (sq == 0) {
-        if (slice_ok(&bits[lane >> 5], 4)) atomicOr(&bits[lane >> 5], (node.x & 1u) << (lane & 31));
-        return;
-    }
-    Blk stk[kMaxLaneBits];
-    uint32_t depth = D, p = 0, acc = 0;
-    const uint32_t npairs = 1u << (sq - 1);
+__device__ __forceinline__ NodePair child_nodes(const uint8_t* kq, uint32_t m, Blk n, uint32_t d, uint32_t L) {
+    const uint32_t t = n.x & 1u;
+    const Blk c0 = cw_load(kq, m, t, 0, d), c1 = cw_load(kq, m, t, 1, d);
+    NodePair p;
+    if (PRF == 0)
+        keyed_pair(n, L, c0, c1, p.a, p.b);
+    else
+        mmo_pair(n, L, c_mmo.rk, c0, c1, p.a, p.b);
+    return p;
+}
+
+__device__ __forceinline__ NodePair child_nodes(uint32_t prf, const uint8_t* kq, uint32_t m, Blk n, uint32_t d, uint32_t L) {
+    return prf == 0 ? child_nodes<0>(kq, m, n, d, L) : child_nodes<1>(kq, m, n, d, L);
+}
+
+// Selection bits of the 2^s leaves (1 <= s <= 5) below `node` (at depth m - s), leaf r in bit r. Depth
+// first; the right child of a depth m - 2 node waits in registers, only those above it go through the
+// (local-memory) stack.
+template <int PRF>
+__device__ __noinline__ uint32_t subtree_word(const uint8_t* kq, uint32_t m, uint32_t s, Blk node, uint32_t L) {
+    Blk stk[5];
+    Blk wait{0, 0, 0, 0};                // right child at depth m - 1
+    // the leaf codewords' lowest bits, bit 2 t + x for C_t[x][m]
+    const uint32_t lsbs = cw_lsb(kq, m, 0, 0, m) | cw_lsb(kq, m, 0, 1, m) << 1 | cw_lsb(kq, m, 1, 0, m) << 2 |
+                          cw_lsb(kq, m, 1, 1, m) << 3;
+    uint32_t left = s - 1, p = 0, acc = 0;  // levels between the node and the leaves' parents; leaf pairs done
+#pragma unroll 1
     for (;;) {
         const uint32_t t = node.x & 1u;
         Key4 k;
@@ -598,32 +668,78 @@ __device__ __forceinline__ void lane_eval(const uint8_t* kq, uint32_t m, uint32_
             keyed_rounds18(node, L, k, a, b);
         else
             mmo_rounds18(node, L, c_mmo.rk, a, b);
-        if (depth == m - 1) {
+        if (left == 0) {
             uint32_t b2 = PRF == 0 ? keyed_leaf_bits_tail(L, k, a, b) : mmo_leaf_bits_tail(node, L, c_mmo.rk, a, b);
-            b2 ^= cw_lsb(kq, m, t, 0, m) | (cw_lsb(kq, m, t, 1, m) << 1);
-            acc |= b2 << ((2 * p) & 31);
+            b2 = (b2 ^ (lsbs >> (2 * t))) & 3u;
+            acc |= b2 << (2 * p);
             ++p;
-            if (sq >= 5 && (p & 15) == 0) {
-                uint32_t* w = &bits[(lane << (sq - 5)) + ((p - 1) >> 4)];
-                if (slice_ok(w, 4)) *w = acc;
-                acc = 0;
-            }
-            if (p == npairs) break;
-            depth = m - 1 - (__ffs(int(p)) - 1);
-            if (IMPIR_IN_BOUNDS(depth - D < kMaxLaneBits, kSiteStack, depth - D)) node = stk[depth - D];
+            if (p >> (s - 1)) return acc;
+            left = __ffs(int(p)) - 1;
+            if (left == 0)
+                node = wait;
+            else if (IMPIR_IN_BOUNDS(left < 5, kSiteStack, left))
+                node = stk[left];
         } else {
-            const Blk c0 = cw_load(kq, m, t, 0, depth + 1);
-            const Blk c1 = cw_load(kq, m, t, 1, depth + 1);
+            const Blk c0 = cw_load(kq, m, t, 0, m - left), c1 = cw_load(kq, m, t, 1, m - left);
             if (PRF == 0)
                 keyed_pair_tail(L, k, c0, c1, a, b);
             else
                 mmo_pair_tail(node, L, c_mmo.rk, c0, c1, a, b);
-            ++depth;
-            if (IMPIR_IN_BOUNDS(depth - D < kMaxLaneBits, kSiteStack, depth - D)) stk[depth - D] = b;
+            --left;
+            if (left == 0)
+                wait = b;
+            else if (IMPIR_IN_BOUNDS(left < 5, kSiteStack, left))
+                stk[left] = b;
             node = a;
         }
     }
-    if (sq < 5 && slice_ok(&bits[(lane << sq) >> 5], 4)) atomicOr(&bits[(lane << sq) >> 5], acc << ((lane << sq) & 31));
+}
+
+__device__ __forceinline__ uint32_t subtree_word(uint32_t prf, const uint8_t* kq, uint32_t m, uint32_t s, Blk node,
+                                                 uint32_t L) {
+    return prf == 0 ? subtree_word<0>(kq, m, s, node, L) : subtree_word<1>(kq, m, s, node, L);
+}
+
+// From `start`, the node at depth d0 on the path to node `sub` of depth D (the root with d0 = 0, or the
+// warp-tile root the warp computed once for this query), down to that node, one edge per level.
+__device__ __forceinline__ Blk walk_down(uint32_t prf, const uint8_t* kq, uint32_t m, uint32_t D, uint64_t sub,
+                                         uint32_t L, Blk node, uint32_t d0) {
+#pragma unroll 1
+    for (uint32_t d = d0 + 1; d <= D; ++d) node = child_node(prf, kq, m, node, uint32_t(sub >> (D - d)) & 1u, d, L);
+    return node;
+}
+
+// Selection bits of the lane's subtree of 2^sq leaves below node `sub` of depth D: bit r of `bits`
+// (relative to the warp tile) is lsb(R(m, tile_first_leaf + r)). Subtrees above 32 leaves go depth
+// first down to those of 32.
+__device__ __forceinline__ void lane_eval(uint32_t prf, const uint8_t* kq, uint32_t m, uint32_t D, uint64_t sub,
+                                          uint32_t sq, uint32_t* bits, uint32_t lane, uint32_t L, const Blk start,
+                                          uint32_t d0) {
+    Blk node = walk_down(prf, kq, m, D, sub, L, start, d0);
+    if (sq < 5) {
+        const uint32_t word = sq == 0 ? node.x & 1u : subtree_word(prf, kq, m, sq, node, L);
+        if (slice_ok(&bits[(lane << sq) >> 5], 4)) atomicOr(&bits[(lane << sq) >> 5], word << ((lane << sq) & 31));
+        return;
+    }
+    Blk stk[kMaxLaneBits - 5 + 1];
+    uint32_t left = sq - 5, w = 0;  // levels between the node and the 32-leaf subtrees; words done
+#pragma unroll 1
+    for (;;) {
+        if (left) {
+            const NodePair p = child_nodes(prf, kq, m, node, m - 5 - left + 1, L);
+            --left;
+            if (IMPIR_IN_BOUNDS(left <= kMaxLaneBits - 5, kSiteStack, left)) stk[left] = p.b;
+            node = p.a;
+            continue;
+        }
+        uint32_t* out = &bits[(lane << (sq - 5)) + w];
+        const uint32_t word = subtree_word(prf, kq, m, 5, node, L);
+        if (slice_ok(out, 4)) *out = word;
+        ++w;
+        if (w >> (sq - 5)) return;
+        left = __ffs(int(w)) - 1;
+        if (IMPIR_IN_BOUNDS(left <= kMaxLaneBits - 5, kSiteStack, left)) node = stk[left];
+    }
 }
 
 // ---- additive answer (MODE 1) ----
@@ -712,8 +828,7 @@ __device__ __forceinline__ void unit_add(const FusedParams& P, const GroupDesc& 
             const uint8_t* kq = query_key(P, query_at(P, qidx, q));
             const Blk start{__shfl_sync(0xffffffffu, top.x, q), __shfl_sync(0xffffffffu, top.y, q),
                             __shfl_sync(0xffffffffu, top.z, q), __shfl_sync(0xffffffffu, top.w, q)};
-            w[q].node = kq[1] == 0 ? walk_down<0>(kq, m, D, sub, L, start, Dt)
-                                   : walk_down<1>(kq, m, D, sub, L, start, Dt);
+            w[q].node = walk_down(kq[1], kq, m, D, sub, L, start, Dt);
             w[q].depth = D;
             w[q].p = 0;
             neg[q] = kq[3] ? 0xffffffffu : 0u;  // party 1 negates its shares (mod 2^32)
@@ -1015,16 +1130,9 @@ __global__ void __launch_bounds__((NK == 1 && QC <= 8) ? 640 : 512, 1)
 
     WsHeader* hdr = reinterpret_cast<WsHeader*>(P.ws);
     if (hdr->n_units == 0) return;  // every tile was the tensor-core kernel's (or no key was well formed)
-    // Replicated T-tables (see the layout note at the top of this file).
-    for (uint32_t i = tid; i < 256 * 32; i += nthr) {
-        const uint32_t x = i >> 5, l = i & 31;
-        const uint32_t t0 = __ldg(P.te0 + x);
-        uint32_t* ra = reinterpret_cast<uint32_t*>(g_smem + x * 256);
-        uint32_t* rb = reinterpret_cast<uint32_t*>(g_smem + 65536 + x * 256);
-        ra[l] = t0;
-        ra[32 + l] = __funnelshift_l(t0, t0, 8);
-        rb[l] = __funnelshift_l(t0, t0, 16);
-        rb[32 + l] = __funnelshift_l(t0, t0, 24);
+    if (!fill_tables(P.te0, tid, nthr)) {
+        hdr->timed_out = 1;
+        return;
     }
 #ifdef IMPIR_BOUNDS
     if (tid == 0) {
@@ -1036,10 +1144,11 @@ __global__ void __launch_bounds__((NK == 1 && QC <= 8) ? 640 : 512, 1)
         s_bctx.db_words = P.db_words;
         s_bctx.smem_bytes = P.smem_bytes;
         s_bctx.warp_slice_bytes = QC * P.bits_words * 4;
+        s_bctx.slices_low = P.slices_low;
     }
     __syncthreads();
 #endif
-    SegDesc* segs = reinterpret_cast<SegDesc*>(g_smem + kTableBytes);
+    SegDesc* segs = reinterpret_cast<SegDesc*>(g_smem);
     uint32_t n_segs = hdr->n_segs;
     const uint32_t first_seg = hdr->first_seg, lane_bits = hdr->lane_bits;
     if (!IMPIR_IN_BOUNDS(first_seg + n_segs <= kMaxSegments, kSiteSchedule, n_segs)) n_segs = 0;
@@ -1051,8 +1160,11 @@ __global__ void __launch_bounds__((NK == 1 && QC <= 8) ? 640 : 512, 1)
     const uint32_t* perm = reinterpret_cast<const uint32_t*>(P.ws + P.lay.off_perm);
     const GroupDesc* groups = reinterpret_cast<const GroupDesc*>(P.ws + P.lay.off_groups);
     uint4* acc_out = reinterpret_cast<uint4*>(P.ws + P.lay.off_acc);
-    uint32_t* bits = reinterpret_cast<uint32_t*>(g_smem + kTableBytes + kSegSmemBytes) + warp * QC * P.bits_words;
-    const uint32_t L = lane * 4;
+    // the warp's slice of the bit / node / share area: the first ones below the tables, the others above
+    uint32_t* bits = warp < P.slices_low
+                         ? reinterpret_cast<uint32_t*>(g_smem + kSegSmemBytes) + warp * QC * P.bits_words
+                         : reinterpret_cast<uint32_t*>(smem_at(kHighAt)) + (warp - P.slices_low) * QC * P.bits_words;
+    const uint32_t L = lane_base(lane);
 
     // a warp's first unit is fixed, SM by SM (where the batch has fewer units than the grid has warps
     // they spread evenly over the SMs), the later ones come from the counter
@@ -1121,9 +1233,7 @@ __global__ void __launch_bounds__((NK == 1 && QC <= 8) ? 640 : 512, 1)
             top = cw_load(kq, mq, 0, 0, 0);  // R(0,0) = C_0[0][0], Eq. (2)
 #pragma unroll 1
             for (uint32_t d = 1; d <= dt; ++d) {
-                const uint32_t x = uint32_t(tile >> (dt - d)) & 1u;
-                const Blk f = kq[1] == 0 ? keyed_one(top, x, L) : mmo_one(top, x, L, c_mmo.rk);
-                top = bxor(f, cw_load(kq, mq, top.x & 1u, x, d));
+                top = child_node(kq[1], kq, mq, top, uint32_t(tile >> (dt - d)) & 1u, d, L);
             }
         }
         if constexpr (MODE == 1) {
@@ -1154,13 +1264,8 @@ __global__ void __launch_bounds__((NK == 1 && QC <= 8) ? 640 : 512, 1)
                     if (act) {
                         const uint8_t* kq = query_key(P, query_at(P, qidx, q));
                         const Blk par{pv.x, pv.y, pv.z, pv.w};
-                        const uint32_t mq = kq[2], t = par.x & 1u, d = mq - sq - 5 + k + 1;
-                        const Blk c0 = cw_load(kq, mq, t, 0, d), c1 = cw_load(kq, mq, t, 1, d);
-                        Blk a, b;
-                        if (kq[1] == 0)
-                            keyed_pair(par, L, c0, c1, a, b);
-                        else
-                            mmo_pair(par, L, c_mmo.rk, c0, c1, a, b);
+                        const NodePair p = child_nodes(kq[1], kq, kq[2], par, kq[2] - sq - 5 + k + 1, L);
+                        const Blk &a = p.a, &b = p.b;
                         if (slice_ok(nodes + q * slot + (2 * i) * 16, 32)) {
                             *reinterpret_cast<uint4*>(nodes + q * slot + (2 * i) * 16) = make_uint4(a.x, a.y, a.z, a.w);
                             *reinterpret_cast<uint4*>(nodes + q * slot + (2 * i + 1) * 16) = make_uint4(b.x, b.y, b.z, b.w);
@@ -1183,10 +1288,7 @@ __global__ void __launch_bounds__((NK == 1 && QC <= 8) ? 640 : 512, 1)
                 __syncwarp();
                 const Blk start{pv.x, pv.y, pv.z, pv.w};
                 if (lane_on) {
-                    if (prf == 0)
-                        lane_eval<0>(kq, mq, Dq, sub, sq, bits + qi * P.bits_words, lane, L, start, Dq - 1);
-                    else
-                        lane_eval<1>(kq, mq, Dq, sub, sq, bits + qi * P.bits_words, lane, L, start, Dq - 1);
+                    lane_eval(prf, kq, mq, Dq, sub, sq, bits + qi * P.bits_words, lane, L, start, Dq - 1);
                 }
             }
         } else {
@@ -1197,10 +1299,7 @@ __global__ void __launch_bounds__((NK == 1 && QC <= 8) ? 640 : 512, 1)
                 const Blk start{__shfl_sync(0xffffffffu, top.x, qi), __shfl_sync(0xffffffffu, top.y, qi),
                                 __shfl_sync(0xffffffffu, top.z, qi), __shfl_sync(0xffffffffu, top.w, qi)};
                 if (lane_on) {
-                    if (prf == 0)
-                        lane_eval<0>(kq, mq, Dq, sub, sq, bits + qi * P.bits_words, lane, L, start, mq > sq + 5 ? mq - sq - 5 : 0);
-                    else
-                        lane_eval<1>(kq, mq, Dq, sub, sq, bits + qi * P.bits_words, lane, L, start, mq > sq + 5 ? mq - sq - 5 : 0);
+                    lane_eval(prf, kq, mq, Dq, sub, sq, bits + qi * P.bits_words, lane, L, start, mq > sq + 5 ? mq - sq - 5 : 0);
                 }
             }
         }

@@ -32,6 +32,7 @@
 //     16-byte load into 128 bytes), two MMAs of 128 x 256 x 32 each, and at the tile's end the
 //     parities are read back and XORed into the per-query accumulators in global memory.
 // No selection bit leaves the SM.
+#define IMPIR_TABLE_POINTER
 #include "fused.cuh"
 
 namespace impir {
@@ -67,16 +68,16 @@ struct Ctl {
     uint32_t pad;
 };
 static_assert(sizeof(Ctl) <= 256, "control block");
-// shared memory after the T-tables
-constexpr uint32_t kOffCtl = kTableBytes;
-constexpr uint32_t kOffBits = kOffCtl + 256;                          // [2][128][32] words
-constexpr uint32_t kOffNodes = kOffBits + 2 * kTcQueries * 32 * 4;    // [2][8][128] nodes
-constexpr uint32_t kOffQuery = kOffNodes + 2 * 8 * kTcQueries * 16;   // [2][128] {key offset, query}
-constexpr uint32_t kOffStage = kOffQuery + 2 * kTcQueries * 8;
-constexpr uint32_t kTcSmem = kOffStage + kStages * kStageBytes;
-static_assert(kTcSmem <= kSmemMax, "shared memory");
-
-__device__ __forceinline__ uint32_t smem32(const void* p) { return uint32_t(__cvta_generic_to_shared(p)); }
+// Shared memory, by address: below the T-tables the operand tiles and 15 of the 16 node arrays, above
+// them the last node array, the selection bits, the units' key offsets and the control block.
+constexpr uint32_t kNodeArray = kTcQueries * 16;
+constexpr uint32_t kAtStage = kSmemBase + kSmemStatic;
+constexpr uint32_t kAtNodes = kAtStage + kStages * kStageBytes;  // [2][8][128] nodes, the last array at kHighAt
+constexpr uint32_t kAtBits = kHighAt + kNodeArray;               // [2][128][32] words
+constexpr uint32_t kAtKey = kAtBits + 2 * kTcQueries * 32 * 4; // [2][128] key offsets
+constexpr uint32_t kAtCtl = kAtKey + 2 * kTcQueries * 4;
+constexpr uint32_t kTcSmem = kAtCtl + 256 - kSmemBase;
+static_assert(kAtNodes + 15 * kNodeArray <= kTableAt && kTcSmem <= kSmemMax, "shared memory");
 
 __device__ __forceinline__ void mbar_init(unsigned long long* b, uint32_t n) {
     asm volatile("mbarrier.init.shared::cta.b64 [%0], %1;" ::"r"(smem32(b)), "r"(n) : "memory");
@@ -132,90 +133,39 @@ __device__ __forceinline__ bool scan_bar_or(bool bad) {
     return r != 0;
 }
 
-// Debug build: n bytes at offset o lie inside the part of shared memory that starts at lo.
+// Debug build: n bytes at shared-memory address o lie inside [lo, hi).
 __device__ __forceinline__ bool smem_ok(uint32_t o, uint32_t n, uint32_t lo, uint32_t hi) {
     return IMPIR_IN_BOUNDS(o >= lo && o + n <= hi, kSiteBits, o);
 }
 
 // Word w (32 records) of query row q in bits buffer b: rows of 32 words, swizzled so that both a
 // warp writing one row and a warp reading one word of 32 rows touch 32 banks.
-__device__ __forceinline__ uint32_t bits_off(uint32_t b, uint32_t q, uint32_t w) {
-    return kOffBits + ((b * kTcQueries + q) * 32 + (w ^ (q & 31))) * 4;
+__device__ __forceinline__ uint32_t bits_at(uint32_t b, uint32_t q, uint32_t w) {
+    return kAtBits + ((b * kTcQueries + q) * 32 + (w ^ (q & 31))) * 4;
 }
 
-__device__ __forceinline__ uint32_t node_off(uint32_t b, uint32_t i, uint32_t q) {
-    return kOffNodes + ((b * 8 + i) * kTcQueries + q) * 16;
+// The key offsets of a unit's queries.
+__device__ __forceinline__ uint32_t* unit_keys(uint32_t b) {
+    return reinterpret_cast<uint32_t*>(smem_at(kAtKey)) + b * kTcQueries;
+}
+
+__device__ __forceinline__ uint32_t node_at(uint32_t b, uint32_t i, uint32_t q) {
+    const uint32_t array = b * 8 + i;
+    return (array < 15 ? kAtNodes + array * kNodeArray : kHighAt) + q * 16;
+}
+
+__device__ __forceinline__ bool node_ok(uint32_t o) {
+    return IMPIR_IN_BOUNDS((o >= kAtNodes && o + 16 <= kTableAt) || (o >= kHighAt && o + 16 <= kAtBits), kSiteBits, o);
 }
 
 __device__ __forceinline__ Blk ld_node(uint32_t o) {
-    if (!smem_ok(o, 16, kOffNodes, kOffQuery)) return {0, 0, 0, 0};
-    const uint4 v = *reinterpret_cast<const uint4*>(g_smem + o);
+    if (!node_ok(o)) return {0, 0, 0, 0};
+    const uint4 v = *reinterpret_cast<const uint4*>(smem_at(o));
     return {v.x, v.y, v.z, v.w};
 }
 
 __device__ __forceinline__ void st_node(uint32_t o, const Blk v) {
-    if (smem_ok(o, 16, kOffNodes, kOffQuery)) *reinterpret_cast<uint4*>(g_smem + o) = make_uint4(v.x, v.y, v.z, v.w);
-}
-
-// Both children of a node at depth d - 1 (Eq. (3)).
-__device__ __forceinline__ void expand(const FusedParams& P, const uint8_t* kq, uint32_t prf, uint32_t m, const Blk n,
-                                       uint32_t d, uint32_t L, Blk& a, Blk& b) {
-    const uint32_t t = n.x & 1u;
-    const Blk c0 = cw_load(kq, m, t, 0, d), c1 = cw_load(kq, m, t, 1, d);
-    if (prf == 0)
-        keyed_pair(n, L, c0, c1, a, b);
-    else
-        mmo_pair(n, L, c_mmo.rk, c0, c1, a, b);
-}
-
-// Selection bits of the 2^S leaves below `node` (at depth m - S), leaf r in bit r; kq: the wire
-// key. Depth first; the right child of a depth m - 2 node waits in registers, only those above it
-// go through the (local-memory) stack. A function of its own, not inlined: inlined into the
-// kernel its loops carried 89 register moves per AES block (16.9 against 15.4 ms for 104
-// queries on 2^22 records of 256 bytes).
-template <int PRF>
-__device__ __noinline__ uint32_t subtree_bits(const uint8_t* kq, uint32_t m, Blk node, uint32_t L) {
-    Blk stk[S];
-    Blk wait{0, 0, 0, 0};                // right child at depth m - 1
-    // the leaf codewords' lowest bits, bit 2 t + x for C_t[x][m]
-    const uint32_t lsbs = cw_lsb(kq, m, 0, 0, m) | cw_lsb(kq, m, 0, 1, m) << 1 | cw_lsb(kq, m, 1, 0, m) << 2 |
-                          cw_lsb(kq, m, 1, 1, m) << 3;
-    uint32_t depth = 0, p = 0, acc = 0;  // depth below the subtree root; leaf pairs done
-#pragma unroll 1
-    for (;;) {
-        const uint32_t t = node.x & 1u;
-        Key4 k;
-        Blk a, b;
-        if (PRF == 0)
-            keyed_rounds18(node, L, k, a, b);
-        else
-            mmo_rounds18(node, L, c_mmo.rk, a, b);
-        if (depth == S - 1) {
-            uint32_t b2 = PRF == 0 ? keyed_leaf_bits_tail(L, k, a, b) : mmo_leaf_bits_tail(node, L, c_mmo.rk, a, b);
-            b2 = (b2 ^ (lsbs >> (2 * t))) & 3u;
-            acc |= b2 << (2 * p);
-            ++p;
-            if (p == (1u << (S - 1))) return acc;
-            depth = S - __ffs(int(p));
-            if (depth == S - 1)
-                node = wait;
-            else if (IMPIR_IN_BOUNDS(depth < S, kSiteStack, depth))
-                node = stk[depth];
-        } else {
-            const uint32_t d = m - S + depth + 1;
-            const Blk c0 = cw_load(kq, m, t, 0, d), c1 = cw_load(kq, m, t, 1, d);
-            if (PRF == 0)
-                keyed_pair_tail(L, k, c0, c1, a, b);
-            else
-                mmo_pair_tail(node, L, c_mmo.rk, c0, c1, a, b);
-            ++depth;
-            if (depth == S - 1)
-                wait = b;
-            else if (IMPIR_IN_BOUNDS(depth < S, kSiteStack, depth))
-                stk[depth] = b;
-            node = a;
-        }
-    }
+    if (node_ok(o)) *reinterpret_cast<uint4*>(smem_at(o)) = make_uint4(v.x, v.y, v.z, v.w);
 }
 
 // Selection bits of a domain smaller than a tile, every leaf by its own walk from the root: lane r
@@ -232,8 +182,7 @@ __device__ __noinline__ uint32_t small_domain_bits(const FusedParams& P, const u
 #pragma unroll 1
         for (uint32_t d = 1; d <= m; ++d) {
             const uint32_t x = (j >> (m - d)) & 1u;
-            const Blk cw = cw_load(kq, m, n.x & 1u, x, d);
-            n = bxor(prf == 0 ? keyed_one(n, x, L) : mmo_one(n, x, L, c_mmo.rk), cw);
+            n = child_node(prf, kq, m, n, x, d, L);
         }
         const uint32_t w = __ballot_sync(0xffffffffu, j < leaves && (n.x & 1u));
         if (lane == r) word = w;
@@ -253,37 +202,39 @@ __device__ __forceinline__ Blk shfl_child(const Blk& a, const Blk& c, uint32_t s
 // One AES task: the selection bits of up to 4 queries of a unit.
 __device__ __forceinline__ void aes_task(const FusedParams& P, uint32_t b, uint32_t q0, uint32_t nq,
                                          unsigned long long tile, uint32_t lane, uint32_t L) {
-    const uint2* query = reinterpret_cast<const uint2*>(g_smem + kOffQuery) + b * kTcQueries;
+    const uint32_t* query = unit_keys(b);
     Blk a{0, 0, 0, 0}, c{0, 0, 0, 0};
     if ((lane >> 3) < nq) {  // level 3 -> 4 below the tile's node, 8 lanes per query
         const uint32_t q = q0 + (lane >> 3);
-        const uint8_t* kq = P.keys + query[q].x;
+        const uint8_t* kq = P.keys + query[q];
         const uint32_t m = kq[2];
-        if (m >= LG) expand(P, kq, kq[1], m, ld_node(node_off(b, lane & 7, q)), m - LG + 4, L, a, c);
+        if (m >= LG) {
+            const NodePair p = child_nodes(kq[1], kq, m, ld_node(node_at(b, lane & 7, q)), m - LG + 4, L);
+            a = p.a;
+            c = p.b;
+        }
     }
     __syncwarp();
 #pragma unroll 1
     for (uint32_t i = 0; i < nq; ++i) {
         const uint32_t q = q0 + i;
-        const uint8_t* kq = P.keys + query[q].x;
+        const uint8_t* kq = P.keys + query[q];
         const uint32_t prf = kq[1], m = kq[2];
         uint32_t word = 0;
         if (m >= LG) {
             // lane l's parent at level 4 is node l >> 1: child (l >> 1) & 1 of level-3 node l >> 2
             Blk n = shfl_child(a, c, i * 8 + (lane >> 2), (lane >> 1) & 1);
             if (tile * K + (lane << S) < P.n_records) {
-                const uint32_t x = lane & 1u;
-                const Blk cw = cw_load(kq, m, n.x & 1u, x, m - S);
-                n = bxor(prf == 0 ? keyed_one(n, x, L) : mmo_one(n, x, L, c_mmo.rk), cw);
-                word = prf == 0 ? subtree_bits<0>(kq, m, n, L) : subtree_bits<1>(kq, m, n, L);
+                n = child_node(prf, kq, m, n, lane & 1u, m - S, L);
+                word = subtree_word(prf, kq, m, S, n, L);
             }
             __syncwarp();
         } else {
             // a domain smaller than a tile (tile 0 only): every leaf by its own walk from the root
             word = small_domain_bits(P, kq, prf, m, lane, L);
         }
-        const uint32_t o = bits_off(b, q, lane);
-        if (smem_ok(o, 4, kOffBits, kOffNodes)) *reinterpret_cast<uint32_t*>(g_smem + o) = word;
+        const uint32_t o = bits_at(b, q, lane);
+        if (smem_ok(o, 4, kAtBits, kAtKey)) *reinterpret_cast<uint32_t*>(smem_at(o)) = word;
     }
 }
 
@@ -335,26 +286,23 @@ __device__ __forceinline__ void prepare_unit(const FusedParams& P, Ctl* ctl, uin
     if (tid < d.count) {
         const uint32_t qi = query_at(P, reinterpret_cast<const uint32_t*>(P.ws + P.lay.off_perm) + d.first, tid);
         const uint8_t* kq = query_key(P, qi);
-        reinterpret_cast<uint2*>(g_smem + kOffQuery)[b * kTcQueries + tid] = make_uint2(uint32_t(kq - P.keys), qi);
+        unit_keys(b)[tid] = uint32_t(kq - P.keys);
         const uint32_t prf = kq[1], m = kq[2];
         if (m >= LG) {
             const uint32_t Dt = m - LG;
             Blk n = cw_load(kq, m, 0, 0, 0);  // R(0,0) = C_0[0][0], Eq. (2)
 #pragma unroll 1
             for (uint32_t e = 1; e <= Dt; ++e) {
-                const uint32_t x = uint32_t(d.tile >> (Dt - e)) & 1u;
-                const Blk cw = cw_load(kq, m, n.x & 1u, x, e);
-                n = bxor(prf == 0 ? keyed_one(n, x, L) : mmo_one(n, x, L, c_mmo.rk), cw);
+                n = child_node(prf, kq, m, n, uint32_t(d.tile >> (Dt - e)) & 1u, e, L);
             }
-            st_node(node_off(b, 0, tid), n);
+            st_node(node_at(b, 0, tid), n);
             // 3 levels: parents 0 | 1 0 | 3 2 1 0; children 2p, 2p + 1 overwrite only nodes already expanded
 #pragma unroll 1
             for (uint32_t e = 1; e < 8; ++e) {
                 const uint32_t k = 31 - __clz(int(e)), p = (2u << k) - 1 - e;
-                Blk l, r;
-                expand(P, kq, prf, m, ld_node(node_off(b, p, tid)), Dt + k + 1, L, l, r);
-                st_node(node_off(b, 2 * p, tid), l);
-                st_node(node_off(b, 2 * p + 1, tid), r);
+                const NodePair c = child_nodes(prf, kq, m, ld_node(node_at(b, p, tid)), Dt + k + 1, L);
+                st_node(node_at(b, 2 * p, tid), c.a);
+                st_node(node_at(b, 2 * p + 1, tid), c.b);
             }
         }
     }
@@ -434,12 +382,13 @@ __device__ __forceinline__ void scan_role(const FusedParams& P, Ctl* ctl, uint32
             if (u.stop) return;
             bad = !mbar_wait(&ctl->full[b], ((i - 2) >> 1) & 1, ctl, 1000);
             if (scan_bar_or(bad)) return;
-            if (tid < u.count) qi = reinterpret_cast<const uint2*>(g_smem + kOffQuery)[b * kTcQueries + tid].y;
+            if (tid < u.count)
+                qi = query_at(P, reinterpret_cast<const uint32_t*>(P.ws + P.lay.off_perm) + u.first, tid);
             // selection bits -> operand A: byte 4 i + j of a 32-record chunk is bit 8 j + i of its word
 #pragma unroll 1
             for (uint32_t w = 0; w < K / 32; ++w) {
-                const uint32_t o = bits_off(b, tid, w);
-                const uint32_t s = smem_ok(o, 4, kOffBits, kOffNodes) ? *reinterpret_cast<const uint32_t*>(g_smem + o) : 0u;
+                const uint32_t o = bits_at(b, tid, w);
+                const uint32_t s = smem_ok(o, 4, kAtBits, kAtKey) ? *reinterpret_cast<const uint32_t*>(smem_at(o)) : 0u;
                 asm volatile("tcgen05.st.sync.aligned.32x32b.x8.b32 [%0], {%1,%2,%3,%4,%5,%6,%7,%8};" ::"r"(acol + lanes + w * 8),
                              "r"(s & 0x01010101u), "r"((s >> 1) & 0x01010101u), "r"((s >> 2) & 0x01010101u),
                              "r"((s >> 3) & 0x01010101u), "r"((s >> 4) & 0x01010101u), "r"((s >> 5) & 0x01010101u),
@@ -477,9 +426,9 @@ __device__ __forceinline__ void scan_role(const FusedParams& P, Ctl* ctl, uint32
                 const uint4 v2 = load();
                 const uint32_t st = use % kStages;
                 bad = use >= kStages && !mbar_wait(&ctl->empty[st], ((use / kStages) - 1) & 1, ctl);
-                const uint32_t so = kOffStage + st * kStageBytes;
-                if (!bad && (two || h == 0) && smem_ok(so + dst + 7 * 1024, 16, kOffStage, kTcSmem)) {
-                    uint8_t* o = g_smem + so + dst;
+                const uint32_t so = kAtStage + st * kStageBytes;
+                if (!bad && (two || h == 0) && smem_ok(so + dst + 7 * 1024, 16, kAtStage, kAtNodes)) {
+                    uint8_t* o = smem_at(so + dst);
 #pragma unroll
                     for (int j = 0; j < 7; ++j) {
                         const uint32_t msk = 0x01010101u << j;
@@ -499,7 +448,7 @@ __device__ __forceinline__ void scan_role(const FusedParams& P, Ctl* ctl, uint32
 #pragma unroll
                     for (uint32_t j = 0; j < 2; ++j) {
                         // 128 B between groups of 8 records, 1024 B between blocks of 16 columns, no swizzle
-                        const uint64_t desc = uint64_t(((smem32(g_smem) + so + j * 512) >> 4) & 0x3fff) |
+                        const uint64_t desc = uint64_t(((so + j * 512) >> 4) & 0x3fff) |
                                               (uint64_t(128 >> 4) << 16) | (uint64_t(1024 >> 4) << 32) | (1ull << 46);
                         mma_f8(dcol, acol + (c * 2 + j) * 8, desc, idesc, (c | j) ? 1u : 0u);
                     }
@@ -525,17 +474,11 @@ __global__ void __launch_bounds__(kTcThreads, 1) fused_tc_kernel(const __grid_co
     const uint32_t tid = threadIdx.x, nthr = blockDim.x, lane = tid & 31, warp = tid >> 5;
     WsHeader* hdr = reinterpret_cast<WsHeader*>(P.ws);
     if (hdr->tc_units == 0) return;  // every tile is the warp kernel's
-    for (uint32_t i = tid; i < 256 * 32; i += nthr) {
-        const uint32_t x = i >> 5, l = i & 31;
-        const uint32_t t0 = __ldg(P.te0 + x);
-        uint32_t* ra = reinterpret_cast<uint32_t*>(g_smem + x * 256);
-        uint32_t* rb = reinterpret_cast<uint32_t*>(g_smem + 65536 + x * 256);
-        ra[l] = t0;
-        ra[32 + l] = __funnelshift_l(t0, t0, 8);
-        rb[l] = __funnelshift_l(t0, t0, 16);
-        rb[32 + l] = __funnelshift_l(t0, t0, 24);
+    if (!fill_tables(P.te0, tid, nthr)) {
+        hdr->timed_out = 1;
+        return;
     }
-    Ctl* ctl = reinterpret_cast<Ctl*>(g_smem + kOffCtl);
+    Ctl* ctl = reinterpret_cast<Ctl*>(smem_at(kAtCtl));
     if (warp == 0) {
         asm volatile("tcgen05.alloc.cta_group::1.sync.aligned.shared::cta.b32 [%0], 512;" ::"r"(smem32(&ctl->tmem)) : "memory");
         asm volatile("tcgen05.relinquish_alloc_permit.cta_group::1.sync.aligned;" ::: "memory");
@@ -550,6 +493,7 @@ __global__ void __launch_bounds__(kTcThreads, 1) fused_tc_kernel(const __grid_co
         s_bctx.db_words = P.db_words;
         s_bctx.smem_bytes = P.smem_bytes;
         s_bctx.warp_slice_bytes = 0;
+        s_bctx.slices_low = 0;
 #endif
         for (int j = 0; j < 2; ++j) {
             mbar_init(&ctl->ready[j], kScanThreads);
@@ -566,10 +510,11 @@ __global__ void __launch_bounds__(kTcThreads, 1) fused_tc_kernel(const __grid_co
     asm volatile("tcgen05.fence::after_thread_sync;" ::: "memory");
     const uint32_t tmem = ctl->tmem;
 
+    const uint32_t L = lane_base(lane);
     if (warp < kScanThreads / 32)
-        scan_role(P, ctl, tid, lane * 4);
+        scan_role(P, ctl, tid, L);
     else
-        aes_role(P, ctl, lane, lane * 4);
+        aes_role(P, ctl, lane, L);
 
     __syncthreads();
     if (ctl->abort && tid == 0) {

@@ -315,10 +315,11 @@ impir_status launch_batch(const DeviceState& dev, const Db& db, const impir_conf
     if (mode == 0) {
         CK(launch_xor(shape, dev.sms, st, fp), "fused kernel launch");
     } else {
-        const size_t smem = smem_add(cfg);
         fp.bits_words = add_share_words(cfg);
-        fp.smem_bytes = uint32_t(smem);
-        CK(launch_fused_add(cfg.queries_per_warp, nk_need(fp.words), dim3(dev.sms), dim3(cfg.warps_per_cta * 32), smem,
+        const SmemSplit sm = split_smem(cfg.warps_per_cta, size_t(cfg.queries_per_warp) * fp.bits_words * 4);
+        fp.slices_low = sm.low;
+        fp.smem_bytes = sm.bytes;
+        CK(launch_fused_add(cfg.queries_per_warp, nk_need(fp.words), dim3(dev.sms), dim3(sm.warps * 32), sm.bytes,
                             st, fp),
            "fused kernel launch (additive)");
     }

@@ -16,6 +16,11 @@ constexpr uint32_t kMaxDomainBits = 40;
 constexpr uint32_t kMaxLaneBits = 10;     // 2^10 leaves per lane at most
 constexpr uint32_t kMaxSegments = 48;     // one per distinct domain size (<= 41) + slack
 constexpr uint32_t kTableBytes = 128 * 1024;
+// Shared-memory addresses of the kernels: the T-tables at 64 KiB, the rest below and above them. The
+// dynamic shared memory begins behind the 1 KiB the system reserves and the kernel's static shared
+// memory (none, or the debug build's check context).
+constexpr uint32_t kTableAt = 0x10000, kHighAt = kTableAt + kTableBytes;
+constexpr uint32_t kSmemBase = 1024, kSmemStatic = 128;
 
 // Largest byte count of a database, a workspace or an answer buffer the library accepts
 // (1 PiB): products of record counts and strides are checked against it before any
@@ -143,6 +148,23 @@ inline uint32_t bits_words(const impir_config& c) {
 // Dynamic shared memory of the XOR kernels: T-tables, segment table, per-warp selection bits.
 inline size_t smem_for(const impir_config& c) {
     return kTableBytes + kSegSmemBytes + size_t(c.warps_per_cta) * c.queries_per_warp * bits_words(c) * 4;
+}
+
+// Where the warps' slices of the bit area go: as many as fit between the segment table and the
+// T-tables, the others above the tables; the launch's dynamic shared memory. Warps whose slices fit
+// neither place (12 warps of 8 KiB, 6 of 16 KiB: one each) are left out of the launch.
+struct SmemSplit {
+    uint32_t low, warps, bytes;
+};
+inline SmemSplit split_smem(uint32_t warps, size_t slice) {
+    constexpr size_t below = kTableAt - kSmemBase - kSmemStatic - kSegSmemBytes;
+    constexpr size_t above = kSmemMax + kSmemBase - kHighAt;
+    SmemSplit s;
+    s.low = uint32_t(std::min<size_t>(warps, below / slice));
+    const uint32_t high = uint32_t(std::min<size_t>(warps - s.low, above / slice));
+    s.warps = s.low + high;
+    s.bytes = uint32_t(kHighAt - kSmemBase + high * slice);
+    return s;
 }
 
 // Estimated time of a batch in the shape c, in SM clocks. A unit (a warp tile for a group of queries)
@@ -275,6 +297,7 @@ struct FusedParams {
     uint32_t n_queries;
     uint32_t words;          // uint4 words per record (stride / 16)
     uint32_t bits_words;     // 32-bit words of selection bits (additive: shares) per (warp, query slot)
+    uint32_t slices_low;     // warps whose slice of those lies below the tables
     unsigned long long rec_lo;  // global index of the record at db[0] (0 unless a chunk or a row shard)
     // extents for the debug build's index checks
     BoundsRecord* bounds;

@@ -42,7 +42,7 @@ __global__ void __launch_bounds__(1024) setup_kernel(const SetupParams S) {
         hdr->bounds_failed = 0;
         hdr->timed_out = 0;
 #ifdef IMPIR_BOUNDS
-        s_bctx = BoundsCtx{S.bounds, hdr, S.keys, S.keys_bytes, nullptr, 0, 0, 0};
+        s_bctx = BoundsCtx{S.bounds, hdr, S.keys, S.keys_bytes, nullptr, 0, 0, 0, 0};
 #endif
     }
     __syncthreads();
@@ -252,7 +252,7 @@ __global__ void __launch_bounds__(1024) setup_kernel(const SetupParams S) {
 
 __global__ void finalize_kernel(const FinalizeParams F) {
 #ifdef IMPIR_BOUNDS
-    if (threadIdx.x == 0) s_bctx = BoundsCtx{F.bounds, nullptr, nullptr, 0, nullptr, 0, 0, 0};
+    if (threadIdx.x == 0) s_bctx = BoundsCtx{F.bounds, nullptr, nullptr, 0, nullptr, 0, 0, 0, 0};
     __syncthreads();
 #endif
     const uint8_t* acc = F.ws + F.lay.off_acc;
@@ -334,10 +334,11 @@ cudaError_t launch_xor(const XorShape& s, int sms, cudaStream_t st, FusedParams&
         if (e != cudaSuccess) return e;
     }
     fp.bits_words = bits_words(s.c);
-    const size_t smem = smem_for(s.c);
-    fp.smem_bytes = uint32_t(smem);
-    return launch_fused(s.c.queries_per_warp, nk_xor(fp.words, s.c.queries_per_warp), dim3(sms),
-                        dim3(s.c.warps_per_cta * 32), smem, st, fp);
+    const SmemSplit sp = split_smem(s.c.warps_per_cta, size_t(s.c.queries_per_warp) * fp.bits_words * 4);
+    fp.slices_low = sp.low;
+    fp.smem_bytes = sp.bytes;
+    return launch_fused(s.c.queries_per_warp, nk_xor(fp.words, s.c.queries_per_warp), dim3(sms), dim3(sp.warps * 32),
+                        sp.bytes, st, fp);
 }
 
 cudaError_t prepare_xor_kernels() {
