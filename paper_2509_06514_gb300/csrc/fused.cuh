@@ -46,6 +46,7 @@
 
 #include "bounds.cuh"
 #include "impir_internal.h"
+#include "launch.cuh"
 
 namespace impir {
 
@@ -1129,8 +1130,13 @@ __global__ void __launch_bounds__((NK == 1 && QC <= 8) ? 640 : 512, 1)
     const uint32_t lane = tid & 31, warp = tid >> 5;
 
     WsHeader* hdr = reinterpret_cast<WsHeader*>(P.ws);
-    if (hdr->n_units == 0) return;  // every tile was the tensor-core kernel's (or no key was well formed)
-    if (!fill_tables(P.te0, tid, nthr)) {
+    // behind the setup kernel the tables are filled while it runs; behind the tensor-core kernel there
+    // may be nothing left to do
+    if (P.after_tc) grid_wait();
+    if (P.after_tc && hdr->n_units == 0) return;
+    const bool tables = fill_tables(P.te0, tid, nthr);
+    grid_wait();
+    if (!tables) {
         hdr->timed_out = 1;
         return;
     }
@@ -1336,8 +1342,7 @@ template <int QC, int NK, int MODE = 0>
 cudaError_t launch_fused_t(dim3 grid, dim3 block, size_t smem, cudaStream_t s, const FusedParams& p) {
     const cudaError_t attr = prepare_fused_t<QC, NK, MODE>();
     if (attr != cudaSuccess) return attr;
-    fused_kernel<QC, NK, MODE><<<grid, block, smem, s>>>(p);
-    return cudaGetLastError();
+    return launch_after(fused_kernel<QC, NK, MODE>, grid, block, smem, s, p);
 }
 
 }  // namespace impir

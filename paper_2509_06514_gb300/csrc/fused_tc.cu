@@ -473,8 +473,10 @@ __device__ __forceinline__ void scan_role(const FusedParams& P, Ctl* ctl, uint32
 __global__ void __launch_bounds__(kTcThreads, 1) fused_tc_kernel(const __grid_constant__ FusedParams P) {
     const uint32_t tid = threadIdx.x, nthr = blockDim.x, lane = tid & 31, warp = tid >> 5;
     WsHeader* hdr = reinterpret_cast<WsHeader*>(P.ws);
+    const bool tables = fill_tables(P.te0, tid, nthr);
+    grid_wait();
     if (hdr->tc_units == 0) return;  // every tile is the warp kernel's
-    if (!fill_tables(P.te0, tid, nthr)) {
+    if (!tables) {
         hdr->timed_out = 1;
         return;
     }
@@ -549,8 +551,7 @@ cudaError_t prepare_fused_tc() {
 cudaError_t launch_fused_tc(int sms, cudaStream_t s, const FusedParams& p) {
     const cudaError_t e = prepare_fused_tc();
     if (e != cudaSuccess) return e;
-    fused_tc_kernel<<<sms, kTcThreads, kTcSmem, s>>>(p);
-    return cudaGetLastError();
+    return launch_after(fused_tc_kernel, dim3(sms), dim3(kTcThreads), kTcSmem, s, p);
 }
 
 }  // namespace impir

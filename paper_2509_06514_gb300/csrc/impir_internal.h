@@ -222,10 +222,10 @@ constexpr uint32_t kTcLaneBits = 5;    // tiles of 32 << 5 = 1024 records
 
 // Fewest queries that must reach a tile for the tensor-core kernel to take it. Its scan costs the
 // same for 1 query as for 128, the warp kernels' grows with every query: measured on 2^22 records,
-// time of the fastest warp shape over the tensor-core kernel's at 32 / 48 / 64 / 128 queries: 0.95 /
-// 1.02 / 1.01 / 1.02 for 64-byte records, 0.97 / 1.04 / 1.04 / 1.07 for 256 bytes, 0.90 / 1.04 / 1.07 /
-// 1.15 for 512 bytes, 0.65 / 0.87 / 1.01 / 1.23 for 1 KiB.
-inline uint32_t tc_min_queries(uint32_t words) { return words <= 32 ? 48u : 96u; }
+// time of the fastest warp shape over the tensor-core kernel's at 48 / 64 / 96 / 128 queries: 0.95 /
+// 0.99 / 1.02 / 1.01 for 64-byte records, 0.94 / 1.01 / 1.05 / 1.06 for 256 bytes, 0.95 / 1.03 / 1.09 /
+// 1.12 for 512 bytes; for 1 KiB 0.87 / 0.98 / 1.18 / 1.22 (4 KiB on 2^20: 1.06 at 96).
+inline uint32_t tc_min_queries(uint32_t words) { return words <= 32 ? 64u : 96u; }
 
 // Fewest units for the tensor-core kernel to take any: units of 1024 records go to SMs whole, and with
 // fewer than four per SM the last round costs more than the scan gains for records up to 256 bytes
@@ -297,6 +297,7 @@ struct FusedParams {
     uint32_t n_queries;
     uint32_t words;          // uint4 words per record (stride / 16)
     uint32_t bits_words;     // 32-bit words of selection bits (additive: shares) per (warp, query slot)
+    uint32_t after_tc;       // the tensor-core kernel is the one before this in the stream
     uint32_t slices_low;     // warps whose slice of those lies below the tables
     unsigned long long rec_lo;  // global index of the record at db[0] (0 unless a chunk or a row shard)
     // extents for the debug build's index checks

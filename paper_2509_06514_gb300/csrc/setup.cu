@@ -14,6 +14,7 @@
 
 #include "bounds.cuh"
 #include "impir_internal.h"
+#include "launch.cuh"
 
 namespace impir {
 
@@ -28,6 +29,7 @@ __global__ void __launch_bounds__(1024) setup_kernel(const SetupParams S) {
     __shared__ uint32_t s_nbad, s_first_bad, s_ngroups;
     __shared__ unsigned long long s_present;  // bit m: some query has domain bits m
     const uint32_t tid = threadIdx.x, nthr = blockDim.x;
+    grid_launch_next();
     WsHeader* hdr = reinterpret_cast<WsHeader*>(S.ws);
     uint32_t* perm = reinterpret_cast<uint32_t*>(S.ws + S.lay.off_perm);
     uint32_t* qm = reinterpret_cast<uint32_t*>(S.ws + S.lay.off_qm);
@@ -251,6 +253,7 @@ __global__ void __launch_bounds__(1024) setup_kernel(const SetupParams S) {
 }
 
 __global__ void finalize_kernel(const FinalizeParams F) {
+    grid_wait();
 #ifdef IMPIR_BOUNDS
     if (threadIdx.x == 0) s_bctx = BoundsCtx{F.bounds, nullptr, nullptr, 0, nullptr, 0, 0, 0, 0};
     __syncthreads();
@@ -301,8 +304,7 @@ cudaError_t launch_setup(const SetupParams& p, cudaStream_t s) {
 cudaError_t launch_finalize(const FinalizeParams& p, cudaStream_t s) {
     const size_t n = size_t(p.n_queries) * p.record_bytes;
     const unsigned blocks = unsigned(n / 256 + 1 < 1024 ? n / 256 + 1 : 1024);
-    finalize_kernel<<<blocks, 256, 0, s>>>(p);
-    return cudaGetLastError();
+    return launch_after(finalize_kernel, dim3(blocks), dim3(256), 0, s, p);
 }
 
 cudaError_t launch_fused(uint32_t qpw, uint32_t nk, dim3 grid, dim3 block, size_t smem, cudaStream_t s,
@@ -333,6 +335,7 @@ cudaError_t launch_xor(const XorShape& s, int sms, cudaStream_t st, FusedParams&
         const cudaError_t e = launch_fused_tc(sms, st, fp);
         if (e != cudaSuccess) return e;
     }
+    fp.after_tc = s.tc ? 1u : 0u;
     fp.bits_words = bits_words(s.c);
     const SmemSplit sp = split_smem(s.c.warps_per_cta, size_t(s.c.queries_per_warp) * fp.bits_words * 4);
     fp.slices_low = sp.low;
