@@ -87,12 +87,12 @@ __device__ __forceinline__ uint32_t lane_base(uint32_t lane) {
     return v;
 }
 
-// Debug build: n bytes at p lie inside the calling warp's slice of the bit / node / share
+// Debug build: n bytes at p lie inside the warp's (the calling one's) slice of the bit / node / share
 // buffer (and inside the launch's dynamic shared memory).
-__device__ __forceinline__ bool slice_ok(const void* p, uint32_t n) {
+__device__ __forceinline__ bool slice_ok(const void* p, uint32_t n, uint32_t warp = threadIdx.x >> 5) {
 #ifdef IMPIR_BOUNDS
     const long long o = static_cast<const uint8_t*>(p) - g_smem;
-    const uint32_t warp = threadIdx.x >> 5, low = s_bctx.slices_low;
+    const uint32_t low = s_bctx.slices_low;
     const long long lo = warp < low ? kSegSmemBytes + (long long)warp * s_bctx.warp_slice_bytes
                                     : kHighAt - smem32(g_smem) + (long long)(warp - low) * s_bctx.warp_slice_bytes;
     const long long end = warp < low ? kTableAt - smem32(g_smem) : s_bctx.smem_bytes;
@@ -179,11 +179,11 @@ __device__ __forceinline__ uint32_t sbox0_lsb(uint32_t v, uint32_t L) { return T
 // constant cache so the rolled round loops spend no ALU work on them.
 __constant__ uint32_t c_rcon[11] = {0x00, 0x01, 0x02, 0x04, 0x08, 0x10, 0x20, 0x40, 0x80, 0x1b, 0x36};
 
-// The round loops below are rolled, or unrolled by two where that measured faster (the node
-// pairs and leaf pairs of the keyed PRF: half the loop overhead; -2 % time at 256-byte records):
-// the fully unrolled PRF variants overflow the instruction cache of the persistent kernel's hot
-// loop, and unrolling by four, or the additive leaf words' loop by two, measured slower.
-
+// The round loops below are rolled, or unrolled where that measured faster (rounds 1-8 of the node and
+// leaf pairs by two: half the loop overhead, -2 % time at 256-byte records; the single child of the
+// walks by three: 2 us of a 43 us query on 2^16 records): the fully unrolled PRF variants overflow the
+// instruction cache of the persistent kernel's hot loop, and unrolling by four, or the additive leaf
+// words' loop by two, measured slower.
 
 struct Key4 {
     uint32_t a, b, c, d;
@@ -288,7 +288,7 @@ __device__ __forceinline__ uint32_t keyed_leaf_bits_tail(uint32_t L, const Key4&
 __device__ __forceinline__ Blk keyed_one(const Blk p, uint32_t x, uint32_t L) {
     Key4 k{p.x, p.y, p.z, p.w};
     Blk s{p.x ^ x, p.y, p.z, p.w};
-#pragma unroll 1
+#pragma unroll 3
     for (int r = 1; r <= 9; ++r) {
         ks_next(k, c_rcon[r], L);
         s = aes_round(s, L, k.a, k.b, k.c, k.d);
@@ -613,12 +613,18 @@ __device__ __forceinline__ void scan_chunk_add(const FusedParams& P, uint64_t ti
 }
 
 // ---- tree steps, Eq. (3) ----
-// The subtree walk is a function of its own, so that the kernels hold its rounds once and it has
-// registers of its own; the other two, used at the walks' tops, measured the same either way.
+// Functions of their own: the compiler copies the loops around them (108 KB of code for one query per
+// warp with the steps inlined), and the rounds would be copied along. The tensor-core kernel, which
+// calls the two small ones once each, inlines those (0.5 % faster).
+#ifdef IMPIR_TABLE_POINTER
+#define IMPIR_TREE_STEP __forceinline__
+#else
+#define IMPIR_TREE_STEP __noinline__
+#endif
 
 // Child x of node n of key kq (domain bits m); the child is at depth d.
 template <int PRF>
-__device__ __forceinline__ Blk child_node(const uint8_t* kq, uint32_t m, Blk n, uint32_t x, uint32_t d, uint32_t L) {
+__device__ IMPIR_TREE_STEP Blk child_node(const uint8_t* kq, uint32_t m, Blk n, uint32_t x, uint32_t d, uint32_t L) {
     const Blk c = cw_load(kq, m, n.x & 1u, x, d);
     return bxor(PRF == 0 ? keyed_one(n, x, L) : mmo_one(n, x, L, c_mmo.rk), c);
 }
@@ -634,7 +640,7 @@ struct NodePair {
 
 // Both children, at depth d.
 template <int PRF>
-__device__ __forceinline__ NodePair child_nodes(const uint8_t* kq, uint32_t m, Blk n, uint32_t d, uint32_t L) {
+__device__ IMPIR_TREE_STEP NodePair child_nodes(const uint8_t* kq, uint32_t m, Blk n, uint32_t d, uint32_t L) {
     const uint32_t t = n.x & 1u;
     const Blk c0 = cw_load(kq, m, t, 0, d), c1 = cw_load(kq, m, t, 1, d);
     NodePair p;
@@ -1166,15 +1172,23 @@ __global__ void __launch_bounds__((NK == 1 && QC <= 8) ? 640 : 512, 1)
     const uint32_t* perm = reinterpret_cast<const uint32_t*>(P.ws + P.lay.off_perm);
     const GroupDesc* groups = reinterpret_cast<const GroupDesc*>(P.ws + P.lay.off_groups);
     uint4* acc_out = reinterpret_cast<uint4*>(P.ws + P.lay.off_acc);
-    // the warp's slice of the bit / node / share area: the first ones below the tables, the others above
-    uint32_t* bits = warp < P.slices_low
-                         ? reinterpret_cast<uint32_t*>(g_smem + kSegSmemBytes) + warp * QC * P.bits_words
-                         : reinterpret_cast<uint32_t*>(smem_at(kHighAt)) + (warp - P.slices_low) * QC * P.bits_words;
+    // a warp's slice of the bit / node / share area: the first ones below the tables, the others above
+    const auto slice_of = [&](uint32_t w) {
+        return w < P.slices_low ? reinterpret_cast<uint32_t*>(g_smem + kSegSmemBytes) + w * QC * P.bits_words
+                                : reinterpret_cast<uint32_t*>(smem_at(kHighAt)) + (w - P.slices_low) * QC * P.bits_words;
+    };
+    uint32_t* bits = slice_of(warp);
+    UnitInfo* info = reinterpret_cast<UnitInfo*>(g_smem + kMaxSegments * sizeof(SegDesc));
     const uint32_t L = lane_base(lane);
 
-    // a warp's first unit is fixed, SM by SM (where the batch has fewer units than the grid has warps
-    // they spread evenly over the SMs), the later ones come from the counter
-    uint32_t taken = 0;
+    // A warp's first unit is fixed, SM by SM (where the batch has fewer units than the grid has warps
+    // they spread evenly over the SMs), the later ones come from the counter. The walks down to the
+    // block's first units and their cooperative levels are shared among its warps (`cta`): a lookup
+    // takes the shared-memory port as long for one lane as for 32, so 14 warps walking with one lane
+    // each hold one another up (16 queries on 2^18 records of 64 bytes: 228 us with each warp on its own,
+    // 214 together; 1 on 2^22 of 256 bytes 322 and 308). With four units or fewer per block there is
+    // nothing to share and the block's barriers cost 2 us more than they save.
+    uint32_t cta = MODE == 0 && QC <= 8 && n_units > 4 * gridDim.x, taken = 0;
 #pragma unroll 1
     for (;;) {
         unsigned long long u = 0;
@@ -1182,22 +1196,28 @@ __global__ void __launch_bounds__((NK == 1 && QC <= 8) ? 640 : 512, 1)
             u = taken ? gridDim.x * (nthr >> 5) + atomicAdd(&hdr->counter, 1ull)
                       : (unsigned long long)warp * gridDim.x + blockIdx.x;
         taken = 1;
-        asm volatile("" : "+r"(taken));  // (keeps the compiler from peeling the first unit: twice the code)
+        asm volatile("" : "+r"(taken), "+r"(cta));  // (keeps the compiler from peeling the first unit: twice the code)
         u = __shfl_sync(0xffffffffu, u, 0);
-        if (u >= n_units) break;
+        bool have = u < n_units;
+        if (!have && !cta) break;
         uint32_t j = 0;
-        while (j + 1 < n_segs && segs[j + 1].unit_lo <= u) ++j;
-        const unsigned long long off = u - segs[j].unit_lo;
-        const unsigned long long tile = segs[j].tile_lo + off / segs[j].count;
-        const uint32_t gi = uint32_t(off % segs[j].count);
-        GroupDesc gd;
-        if (MODE == 0 && segs[j].active) {
-            // domains of at least one tile, of any mix of sizes: the queries at these sorted positions
-            gd = {gi * QC, min(uint32_t(QC), segs[j].active - gi * QC), kMaxDomainBits, 0};
-            if (!IMPIR_IN_BOUNDS(gi * QC < segs[j].active, kSiteSchedule, gi)) continue;
-        } else {
-            if (!IMPIR_IN_BOUNDS(gi < hdr->n_groups, kSiteSchedule, gi)) continue;
-            gd = groups[gi];
+        unsigned long long tile = 0;
+        GroupDesc gd{0, 0, kMaxDomainBits, 0};
+        if (have) {
+            while (j + 1 < n_segs && segs[j + 1].unit_lo <= u) ++j;
+            const unsigned long long off = u - segs[j].unit_lo;
+            tile = segs[j].tile_lo + off / segs[j].count;
+            const uint32_t gi = uint32_t(off % segs[j].count);
+            if (MODE == 0 && segs[j].active) {
+                // domains of at least one tile, of any mix of sizes: the queries at these sorted positions
+                gd.first = gi * QC;
+                gd.count = min(uint32_t(QC), segs[j].active - gi * QC);
+                have = IMPIR_IN_BOUNDS(gi * QC < segs[j].active, kSiteSchedule, gi);
+            } else {
+                have = IMPIR_IN_BOUNDS(gi < hdr->n_groups, kSiteSchedule, gi);
+                if (have) gd = groups[gi];
+            }
+            if (!have && !cta) continue;
         }
 
         // m, D and Dt are the group's (a mixed group: those of the largest domain, which give the
@@ -1215,11 +1235,8 @@ __global__ void __launch_bounds__((NK == 1 && QC <= 8) ? 640 : 512, 1)
         const bool lane_on = lane < lanes && (sub << sq) < n_eff;
         const uint32_t nwords = uint32_t((TT + 31) >> 5);
 
-        // Cooperative walk (selection-bit answers, at most 8
-        // queries per warp: with 16 the kernel sits at its register limit and runs slower): the warp
-        // expands the 5 levels between the warp-tile root and the lane subtree roots for all
-        // the group's queries at once, level by level, in place in the (not yet used) bit area;
-        // otherwise each lane walks them itself for every query.
+        // Cooperative walk: selection-bit answers with at most 8 queries per warp (with 16 the kernel sits
+        // at its register limit and runs slower).
         const bool coop = MODE == 0 && QC <= 8 && m >= 5;
         if (MODE == 0 && !coop) {
             for (int q = 0; q < QC; ++q)
@@ -1229,18 +1246,74 @@ __global__ void __launch_bounds__((NK == 1 && QC <= 8) ? 640 : 512, 1)
         __syncwarp();
         const uint32_t* qidx = perm + gd.first;
         // Shared top of the walk: the 32 lane subtrees of a warp tile hang below one node at
-        // depth Dt = D - 5; lane q walks root -> that node for query q of the group, so all the
-        // group's queries take one pass, and the nodes are then broadcast to every lane.
+        // depth Dt = D - 5, walked to once per query. Cooperative units: node 0 of query q's slot in
+        // the (not yet used) bit area, from where the five levels below are expanded level by
+        // level, in place. Else lane q walks for query q, and the nodes are broadcast to every lane.
         const uint32_t Dt = D > 5 ? D - 5 : 0;
+        const uint32_t slot = P.bits_words * 4;
         Blk top{0, 0, 0, 0};
-        if (lane < gd.count) {
+        if constexpr (MODE == 0 && QC <= 8) {
+            if (lane == 0) info[warp] = UnitInfo{tile, gd.first, have && coop ? gd.count : 0u, sq, {0, 0, 0}};
+            const uint32_t nw = cta ? nthr >> 5 : 1u, w0 = cta ? 0u : warp, rank = cta ? tid : lane;
+            const uint32_t size = cta ? nthr : 32u, per_w = cta ? uint32_t(QC) : max(gd.count, 1u), n = nw * per_w;
+            const auto sync = [&]() {
+                if (cta)
+                    __syncthreads();
+                else
+                    __syncwarp();
+            };
+            sync();
+#pragma unroll 1
+            for (uint32_t t = rank; t < n; t += size) {
+                const uint32_t w = w0 + t / per_w, q = t % per_w;
+                const UnitInfo ui = info[w];
+                if (q >= ui.count) continue;
+                const uint8_t* kq = query_key(P, query_at(P, perm + ui.first, q));
+                const uint32_t mq = kq[2], dt = mq > ui.sq + 5 ? mq - ui.sq - 5 : 0;
+                Blk r = cw_load(kq, mq, 0, 0, 0);  // R(0,0) = C_0[0][0], Eq. (2)
+#pragma unroll 1
+                for (uint32_t d = 1; d <= dt; ++d) r = child_node(kq[1], kq, mq, r, uint32_t(ui.tile >> (dt - d)) & 1u, d, L);
+                uint8_t* nodes = reinterpret_cast<uint8_t*>(slice_of(w)) + q * slot;
+                if (slice_ok(nodes, 16, w)) *reinterpret_cast<uint4*>(nodes) = make_uint4(r.x, r.y, r.z, r.w);
+            }
+            sync();
+#pragma unroll 1
+            for (uint32_t k = 0; k < 4; ++k) {  // level k -> k + 1 below the warp-tile root
+                const uint32_t per = 1u << k, items = n * per;
+                // parents in descending index order: children 2i, 2i+1 overwrite only parents
+                // already read (in this chunk, before any write) or expanded (earlier chunks)
+#pragma unroll 1
+                for (uint32_t f0 = 0; f0 < items; f0 += size) {
+                    const uint32_t f = f0 + rank, t = f % n, i = per - 1 - min(f / n, per - 1);
+                    const uint32_t w = w0 + t / per_w, q = t % per_w;
+                    const UnitInfo ui = info[w];
+                    const bool act = f < items && q < ui.count;
+                    uint8_t* nodes = reinterpret_cast<uint8_t*>(slice_of(w)) + q * slot;
+                    uint4 pv = make_uint4(0, 0, 0, 0);
+                    if (act && slice_ok(nodes + i * 16, 16, w)) pv = *reinterpret_cast<const uint4*>(nodes + i * 16);
+                    sync();
+                    if (act) {
+                        const uint8_t* kq = query_key(P, query_at(P, perm + ui.first, q));
+                        const Blk par{pv.x, pv.y, pv.z, pv.w};
+                        const NodePair p = child_nodes(kq[1], kq, kq[2], par, kq[2] - ui.sq - 5 + k + 1, L);
+                        if (slice_ok(nodes + 2 * i * 16, 32, w)) {
+                            *reinterpret_cast<uint4*>(nodes + 2 * i * 16) = make_uint4(p.a.x, p.a.y, p.a.z, p.a.w);
+                            *reinterpret_cast<uint4*>(nodes + (2 * i + 1) * 16) = make_uint4(p.b.x, p.b.y, p.b.z, p.b.w);
+                        }
+                    }
+                    sync();
+                }
+            }
+            cta = 0;
+            if (!have) continue;
+            // (domains below 32 leaves: the root is the top)
+            if (!coop && lane < gd.count) top = cw_load(query_key(P, query_at(P, qidx, lane)), m, 0, 0, 0);
+        } else if (lane < gd.count) {
             const uint8_t* kq = query_key(P, query_at(P, qidx, lane));
             const uint32_t mq = kq[2], dt = mq > sq + 5 ? mq - sq - 5 : 0;
-            top = cw_load(kq, mq, 0, 0, 0);  // R(0,0) = C_0[0][0], Eq. (2)
+            top = cw_load(kq, mq, 0, 0, 0);
 #pragma unroll 1
-            for (uint32_t d = 1; d <= dt; ++d) {
-                top = child_node(kq[1], kq, mq, top, uint32_t(tile >> (dt - d)) & 1u, d, L);
-            }
+            for (uint32_t d = 1; d <= dt; ++d) top = child_node(kq[1], kq, mq, top, uint32_t(tile >> (dt - d)) & 1u, d, L);
         }
         if constexpr (MODE == 1) {
             unit_add<QC, NK>(P, gd, qidx, tile_base, nrec, sub, sq, D, Dt, top, bits, acc_out, lane, L);
@@ -1248,38 +1321,7 @@ __global__ void __launch_bounds__((NK == 1 && QC <= 8) ? 640 : 512, 1)
             continue;
         }
         if (coop) {
-            uint8_t* nodes = reinterpret_cast<uint8_t*>(bits);  // query q's nodes at q * slot
-            const uint32_t slot = P.bits_words * 4;
-            if (lane < gd.count && slice_ok(nodes + lane * slot, 16))
-                *reinterpret_cast<uint4*>(nodes + lane * slot) = make_uint4(top.x, top.y, top.z, top.w);
-            __syncwarp();
-#pragma unroll 1
-            for (uint32_t k = 0; k < 4; ++k) {  // level k -> k + 1 below the warp-tile root
-                const uint32_t per = 1u << k, items = gd.count * per;
-                // parents in descending index order: children 2i, 2i+1 overwrite only parents
-                // already read (in this chunk, before any write) or expanded (earlier chunks)
-#pragma unroll 1
-                for (uint32_t f0 = 0; f0 < items; f0 += 32) {
-                    const uint32_t f = f0 + lane;
-                    const bool act = f < items;
-                    const uint32_t q = act ? f % gd.count : 0, i = act ? (per - 1) - f / gd.count : 0;
-                    uint4 pv = make_uint4(0, 0, 0, 0);
-                    if (act && slice_ok(nodes + q * slot + i * 16, 16))
-                        pv = *reinterpret_cast<const uint4*>(nodes + q * slot + i * 16);
-                    __syncwarp();
-                    if (act) {
-                        const uint8_t* kq = query_key(P, query_at(P, qidx, q));
-                        const Blk par{pv.x, pv.y, pv.z, pv.w};
-                        const NodePair p = child_nodes(kq[1], kq, kq[2], par, kq[2] - sq - 5 + k + 1, L);
-                        const Blk &a = p.a, &b = p.b;
-                        if (slice_ok(nodes + q * slot + (2 * i) * 16, 32)) {
-                            *reinterpret_cast<uint4*>(nodes + q * slot + (2 * i) * 16) = make_uint4(a.x, a.y, a.z, a.w);
-                            *reinterpret_cast<uint4*>(nodes + q * slot + (2 * i + 1) * 16) = make_uint4(b.x, b.y, b.z, b.w);
-                        }
-                    }
-                    __syncwarp();
-                }
-            }
+            const uint8_t* nodes = reinterpret_cast<const uint8_t*>(bits);
 #pragma unroll 1
             for (uint32_t qi = 0; qi < gd.count; ++qi) {
                 const uint8_t* kq = query_key(P, query_at(P, qidx, qi));

@@ -68,7 +68,16 @@ struct SegDesc {
     unsigned long long pad2;
 };
 static_assert(sizeof(SegDesc) == 32, "segment descriptors are 32 bytes");
-constexpr uint32_t kSegSmemBytes = kMaxSegments * sizeof(SegDesc);
+// A warp's unit, for the other warps of its block (they expand the tops of the block's first units together).
+struct UnitInfo {
+    unsigned long long tile;
+    uint32_t first, count;  // sorted positions of its queries; 0: no unit, or one without the cooperative walk
+    uint32_t sq, pad[3];
+};
+static_assert(sizeof(UnitInfo) == 32, "unit descriptors are 32 bytes");
+constexpr uint32_t kMaxWarps = 20;
+// segment table and the warps' unit descriptors, at the start of the warp kernels' shared memory
+constexpr uint32_t kSegSmemBytes = kMaxSegments * sizeof(SegDesc) + kMaxWarps * sizeof(UnitInfo);
 
 // Failed index checks of the debug build (compiled with IMPIR_BOUNDS), one record per device:
 // how many failed since the record was last cleared, and the site and index of the first.
@@ -168,29 +177,42 @@ inline SmemSplit split_smem(uint32_t warps, size_t slice) {
 }
 
 // Estimated time of a batch in the shape c, in SM clocks. A unit (a warp tile for a group of queries)
-// costs `steps` node pairs of a warp: the walk to the tile, the cooperative levels and the lanes'
-// subtrees, and the scan's share of the ALU pipe. A pair takes about 330 clocks of an SM's time for
-// each warp that runs there (the lookups' shared-memory port) plus 700 of latency; units go to the
-// warps whole, so the last, partly filled round counts in full.
+// costs a warp the walk to the tile, four cooperative levels, the lanes' subtrees and the scan's share
+// of the ALU pipe, counted in node pairs. A pair takes a warp 2000 clocks by itself (a single child
+// 1750), and an SM's warps together 330 each (the lookups' shared-memory port); a round of record
+// loads 900. Where every unit finds
+// a warp at once, the block's warps share the walk and the cooperative levels if it has more than four
+// units (fused.cuh); else units go to the warps whole, so the last, partly filled round counts in full.
 // The scan's reads: every group reads the tiles it covers, the first from HBM, the others from L2 if
 // the tiles in work at a time fit there.
 inline double shape_clocks(const impir_config& c, uint64_t n_records, uint32_t words, uint32_t n_queries, int sms) {
-    const double slots = c.queries_per_warp, s = c.lane_bits;
+    const double slots = c.queries_per_warp, s = c.lane_bits, w = c.warps_per_cta;
     const double groups = std::ceil(n_queries / slots), tiles = std::ceil(double(n_records) / double(32ull << c.lane_bits));
     const double q = n_queries / groups, m = std::ceil(std::log2(double(n_records)));
-    double coop = 0;
-    for (int k = 0; k < 4; ++k) coop += 1.3 * std::ceil(q * double(1 << k) / 32);
-    const double lane = q * (0.8 + std::exp2(s) - 1);
+    const double units = groups * tiles, top = std::max(0.0, m - s - 5);
     const double scan = std::exp2(s) * words * (4.3 * slots + 4) / 560;
-    const double steps = (std::max(0.0, m - s - 5) + coop + lane + scan) * (1 + 0.012 * slots);
-    const double units = groups * tiles;
-    const double w = c.warps_per_cta, full = std::floor(units / (sms * w));
-    const double rest = std::ceil((units - full * sms * w) / sms);
-    const double pairs = full * (330 * w + 700) + (rest > 0 ? 330 * rest + (full > 0 ? 1400 : 700) : 0);
+    const double lanes = q * (0.8 + std::exp2(s) - 1), slow = 1 + 0.012 * slots;
+    const uint32_t nk = nk_xor(words, c.queries_per_warp);
+    const double per_load = nk == 1 ? (slots == 1 ? 16 : slots == 2 ? 8 : 4) * std::max(1u, 32 / words) : nk <= 2 ? 4 : nk == 4 ? 2 : 1;
+    const double loads = std::ceil(32 * std::exp2(s) / per_load) * std::ceil(words / (32.0 * nk));
+    double clocks, hbm = 3300;
+    if (units <= sms * w) {
+        const double n = std::ceil(units / sms), shared = n > 4 ? n : 1;  // warps whose levels are expanded together
+        clocks = top * std::max(1750.0, 200 * std::ceil(shared * q / 32) * (n > 4 ? 1 : n)) +
+                 slow * lanes * std::max(2000.0, 330 * n + 700) +
+                 std::max(slow * scan * std::max(2000.0, 330 * n + 700), 900 * loads);
+        hbm = std::min(hbm, 400 * n);
+        for (int k = 0; k < 4; ++k)
+            clocks += std::max(2500.0, 330 * std::ceil(shared * q * double(1 << k) / 32) * (n > 4 ? 1 : n));
+    } else {
+        double coop = 0;
+        for (int k = 0; k < 4; ++k) coop += 1.3 * std::ceil(q * double(1 << k) / 32);
+        const double full = std::floor(units / (sms * w)), left = std::ceil((units - full * sms * w) / sms);
+        clocks = (top + coop + lanes + scan) * slow * (full * (330 * w + 700) + (left > 0 ? 330 * left + 1400 : 0));
+    }
     const double record = words * 16.0 * (c.queries_per_warp == 1 ? 0.5 : 1.0), pass = double(n_records) * record;
     const double live = std::min(units, sms * w) / groups * double(32ull << c.lane_bits) * record;
-    const double mem = pass * (groups > 1 && live > 64e6 ? groups : 1.0) / 3300 + pass * groups / 5000;
-    return steps * pairs + mem;
+    return clocks + pass * (groups > 1 && live > 64e6 ? groups : 1.0) / hbm + pass * groups / 5000;
 }
 
 // The shape with the smallest estimate (lane subtrees of at most 2^8 leaves).
@@ -203,6 +225,10 @@ inline impir_config default_config(uint64_t n_records, uint32_t words, uint32_t 
             for (uint32_t b = 0; b <= 8; ++b) {
                 const impir_config c{b, qpw, w, 0};
                 if (smem_for(c) > kSmemMax) continue;
+                // groups that share a database above L2's size: tiles of at most 512 KiB, read again while
+                // they are there (18 queries on 2^21 x 256 B: 1395 us with tiles of 1 MiB, 1086 with 256 KiB)
+                if (b > 0 && n_queries > qpw && uint64_t(n_records) * words > (64u << 20) / 16 && (uint64_t(words) << (b + 9)) > (512u << 10))
+                    continue;
                 const double t = shape_clocks(c, n_records, words, n_queries, sms);
                 if (best_t == 0 || t < best_t) {
                     best_t = t;
