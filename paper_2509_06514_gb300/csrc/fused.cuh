@@ -1171,7 +1171,7 @@ __global__ void __launch_bounds__((NK == 1 && QC <= 8) ? 640 : 512, 1)
     const unsigned long long n_units = hdr->n_units;
     const uint32_t* perm = reinterpret_cast<const uint32_t*>(P.ws + P.lay.off_perm);
     const GroupDesc* groups = reinterpret_cast<const GroupDesc*>(P.ws + P.lay.off_groups);
-    uint4* acc_out = reinterpret_cast<uint4*>(P.ws + P.lay.off_acc);
+    uint4* acc_out = P.acc;
     // a warp's slice of the bit / node / share area: the first ones below the tables, the others above
     const auto slice_of = [&](uint32_t w) {
         return w < P.slices_low ? reinterpret_cast<uint32_t*>(g_smem + kSegSmemBytes) + w * QC * P.bits_words

@@ -361,7 +361,7 @@ __device__ __forceinline__ uint4 read_parities(uint32_t taddr) {
 __device__ __forceinline__ void scan_role(const FusedParams& P, Ctl* ctl, uint32_t tid, uint32_t L) {
     const uint32_t lane = tid & 31, warp = tid >> 5, W = P.words;
     const uint32_t dcol = ctl->tmem, acol = ctl->tmem + 256, lanes = (warp * 32) << 16;
-    uint4* acc_out = reinterpret_cast<uint4*>(P.ws + P.lay.off_acc);
+    uint4* acc_out = P.acc;
     // this thread's place in an operand tile of 64 records x 2 words: record row k (k groups of 8
     // rows: 8 lanes fill 128 contiguous bytes) and word h. Row p = 4 i + j of 32 holds record 8 j + i,
     // the order in which masking a selection word by bytes leaves its bits.

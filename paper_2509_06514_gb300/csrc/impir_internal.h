@@ -291,6 +291,7 @@ struct SetupParams {
     const uint8_t* keys;
     const uint32_t* key_off;
     uint8_t* ws;
+    uint4* acc;              // the per-query accumulators (in the workspace, or the caller's answers)
     WsLayout lay;
     uint64_t n_records;
     uint32_t n_queries;
@@ -317,6 +318,7 @@ struct FusedParams {
     const uint8_t* keys;
     const uint32_t* key_off;
     uint8_t* ws;
+    uint4* acc;              // as in SetupParams
     const uint32_t* te0;     // 256-entry AES T-table (global memory), see host_aes.cpp
     WsLayout lay;
     uint64_t n_records;

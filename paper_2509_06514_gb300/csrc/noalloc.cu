@@ -113,6 +113,7 @@ extern "C" impir_status impir_answer_noalloc(const void* d_records, uint64_t n_r
     sp.keys = d_keys;
     sp.key_off = d_key_offsets;
     sp.ws = dev->scratch;
+    sp.acc = reinterpret_cast<uint4*>(dev->scratch + lay.off_acc);
     sp.lay = lay;
     sp.n_records = n_records;
     sp.n_queries = n_queries;
@@ -129,6 +130,7 @@ extern "C" impir_status impir_answer_noalloc(const void* d_records, uint64_t n_r
     fp.keys = d_keys;
     fp.key_off = d_key_offsets;
     fp.ws = dev->scratch;
+    fp.acc = sp.acc;
     fp.te0 = dev->te0;
     fp.lay = lay;
     fp.n_records = n_records;

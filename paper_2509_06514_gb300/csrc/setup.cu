@@ -35,7 +35,7 @@ __global__ void __launch_bounds__(1024) setup_kernel(const SetupParams S) {
     uint32_t* qm = reinterpret_cast<uint32_t*>(S.ws + S.lay.off_qm);
     GroupDesc* groups = reinterpret_cast<GroupDesc*>(S.ws + S.lay.off_groups);
     SegDesc* segs = reinterpret_cast<SegDesc*>(S.ws + S.lay.off_segs);
-    uint4* acc = reinterpret_cast<uint4*>(S.ws + S.lay.off_acc);
+    uint4* acc = S.acc;
 
     if (tid <= kMaxDomainBits) hist[tid] = cursor[tid] = 0;
     if (tid == 0) {
