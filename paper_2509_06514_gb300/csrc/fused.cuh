@@ -490,6 +490,11 @@ __device__ __forceinline__ void mad4(uint4& a, const uint4 v, uint32_t s) {
     a.w += v.w * s;
 }
 
+__device__ __forceinline__ uint4 shfl_down4(const uint4 v, uint32_t by) {
+    return make_uint4(__shfl_down_sync(0xffffffffu, v.x, by), __shfl_down_sync(0xffffffffu, v.y, by),
+                      __shfl_down_sync(0xffffffffu, v.z, by), __shfl_down_sync(0xffffffffu, v.w, by));
+}
+
 __device__ __forceinline__ uint4 add4(const uint4 a, const uint4 b) {
     return make_uint4(a.x + b.x, a.y + b.y, a.z + b.z, a.w + b.w);
 }
@@ -552,23 +557,18 @@ __device__ __forceinline__ void scan_chunk_add(const FusedParams& P, uint64_t ti
                 }
             }
         }
-        if (R * W == 32) {
-            for (uint32_t off = W; off < 32; off <<= 1)
+        // the R record rows of the warp to row 0 (for record widths that do not divide the warp too: one
+        // addition per word and query instead of R, all to the same few addresses)
+        for (uint32_t o = 1; o < R; o <<= 1)
 #pragma unroll
-                for (int q = 0; q < QC; ++q)
-                    acc[q] = add4(acc[q], make_uint4(__shfl_xor_sync(0xffffffffu, acc[q].x, off),
-                                                     __shfl_xor_sync(0xffffffffu, acc[q].y, off),
-                                                     __shfl_xor_sync(0xffffffffu, acc[q].z, off),
-                                                     __shfl_xor_sync(0xffffffffu, acc[q].w, off)));
-            if (lr == 0)
-#pragma unroll
-                for (int q = 0; q < QC; ++q)
-                    if (uint32_t(q) < count) acc_add(P, acc_out, query_at(P, qidx, q), lk, acc[q]);
-        } else if (on) {
+            for (int q = 0; q < QC; ++q) {
+                const uint4 v = shfl_down4(acc[q], o * W);
+                if (lr + o < R) acc[q] = add4(acc[q], v);
+            }
+        if (lr == 0)
 #pragma unroll
             for (int q = 0; q < QC; ++q)
                 if (uint32_t(q) < count) acc_add(P, acc_out, query_at(P, qidx, q), lk, acc[q]);
-        }
     } else {
         // W > 32: the whole warp reads one record per step, NK words per lane, in column passes
         for (uint32_t k0 = 0; k0 < W; k0 += 32 * NK) {
@@ -909,11 +909,6 @@ __device__ __forceinline__ uint4 bxor4(const uint4 a, const uint4 b) {
     return make_uint4(a.x ^ b.x, a.y ^ b.y, a.z ^ b.z, a.w ^ b.w);
 }
 
-__device__ __forceinline__ uint4 shfl_xor4(const uint4 v, int off) {
-    return make_uint4(__shfl_xor_sync(0xffffffffu, v.x, off), __shfl_xor_sync(0xffffffffu, v.y, off),
-                      __shfl_xor_sync(0xffffffffu, v.z, off), __shfl_xor_sync(0xffffffffu, v.w, off));
-}
-
 // dpXOR of one warp tile for the group's queries: records [tile_base, tile_base + nrec).
 // Selection bits are read one 32-bit word (32 records) per query at a time.
 template <int QC, int NK>
@@ -1013,19 +1008,18 @@ __device__ __forceinline__ void scan_tile(const FusedParams& P, uint64_t tile_ba
                 }
             }
         }
-        if (R * W == 32) {
-            for (uint32_t off = W; off < 32; off <<= 1)
+        // the R record rows of the warp to row 0 (for record widths that do not divide the warp too: one
+        // query on 2^19 records of 77 bytes spent a third of its 109 us on R atomics per word)
+        for (uint32_t o = 1; o < R; o <<= 1)
 #pragma unroll
-                for (int q = 0; q < QC; ++q) acc[q] = bxor4(acc[q], shfl_xor4(acc[q], int(off)));
-            if (lr == 0)
-#pragma unroll
-                for (int q = 0; q < QC; ++q)
-                    if (uint32_t(q) < count) acc_xor(P, acc_out, query_at(P, qidx, q), lk, acc[q]);
-        } else if (on) {
+            for (int q = 0; q < QC; ++q) {
+                const uint4 v = shfl_down4(acc[q], o * W);
+                if (lr + o < R) acc[q] = bxor4(acc[q], v);
+            }
+        if (lr == 0)
 #pragma unroll
             for (int q = 0; q < QC; ++q)
                 if (uint32_t(q) < count) acc_xor(P, acc_out, query_at(P, qidx, q), lk, acc[q]);
-        }
     } else {
         // W > 32: the whole warp reads one record per step, NK words per lane, in column
         // passes; a record's selection bits are warp-uniform. The compiler predicates a

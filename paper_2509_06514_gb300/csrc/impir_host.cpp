@@ -239,26 +239,23 @@ impir_config add_config(impir_config c, uint32_t words) {
     return c;
 }
 
-// Default shape of the additive answer: as many queries per unit as the record size allows
-// (up to 2, and no more than the batch), and the largest lane subtree, up to 256 leaves, that
-// still leaves three units per resident warp.
+// Default shape of the additive answer: the smallest estimate (lane subtrees of at most 2^8 leaves).
+// Before, as many queries per unit as possible and three units per warp: 9 queries on 2^16 x 64 B 185 us
+// against 63 in the shape chosen now, 64 on 2^20 x 256 B 3606 against 3358.
 impir_config default_add_config(uint64_t n_records, uint32_t words, uint32_t n_queries, int sms) {
-    impir_config c{};
-    c.warps_per_cta = 16;
-    c.queries_per_warp = max_add_qpw(words);
-    while (c.queries_per_warp > 1 && c.queries_per_warp > n_queries) c.queries_per_warp >>= 1;
-    c.queries_per_launch = 0;
-    const double warps = double(sms) * c.warps_per_cta;
-    const double groups = std::ceil(double(n_queries) / c.queries_per_warp);
-    c.lane_bits = 0;
-    for (uint32_t s = 8; s > 0; --s) {
-        const double tiles = std::ceil(double(n_records) / double(32ull << s));
-        if (groups * tiles >= 3.0 * warps) {
-            c.lane_bits = s;
-            break;
-        }
-    }
-    return c;
+    impir_config best{};
+    double best_t = 0;
+    for (uint32_t qpw = 1; qpw <= std::min(max_add_qpw(words), n_queries); qpw *= 2)
+        for (uint32_t w = 16; w <= (nk_need(words) == 1 ? 20u : 16u); w += 4)
+            for (uint32_t b = 0; b <= 8; ++b) {
+                const impir_config c{b, qpw, w, 0};
+                const double t = shape_clocks(c, n_records, words, n_queries, sms, true);
+                if (best_t == 0 || t < best_t) {
+                    best_t = t;
+                    best = c;
+                }
+            }
+    return best;
 }
 
 size_t smem_add(const impir_config& c) {
@@ -284,11 +281,11 @@ bool answers_fit(const Db& db, const uint8_t* d_out) {
 // build's index checks use it)
 impir_status launch_batch(const DeviceState& dev, const Db& db, const impir_config& cfg, const uint8_t* d_keys,
                           const uint32_t* d_off, uint32_t n, uint8_t* d_out, uint8_t* d_ws, cudaStream_t st,
-                          int mode = 0, size_t keys_bytes = 0, bool tc_allowed = false) {
+                          int mode = 0, size_t keys_bytes = 0, bool free_shape = false) {
     const WsLayout lay = ws_layout(n, db.stride);
     // a row shard covers the warp tiles of its rows (shard bounds are whole tiles) of a
     // database of n_total records; its device rows start at global row row_lo
-    const XorShape shape = xor_shape(cfg, mode == 0 && tc_allowed, db.n, db.stride / 16, n, dev.sms);
+    const XorShape shape = xor_shape(cfg, free_shape, db.n, db.stride / 16, n, dev.sms, mode == 1);
     const bool shard = db.row_lo != 0 || db.n_total != db.n;
     SetupParams sp{};
     sp.keys = d_keys;
@@ -385,7 +382,7 @@ impir_status answer_async_impl(const Db& db, const impir_config* cfg_in, const u
     }
     if (impir_status s = check_config(cfg, db.stride / 16, mode)) return s;
     // a shape that the caller set is launched as it is
-    const bool tc_allowed = !cfg_in && (!db.cfg_set || db.cfg_tuned);
+    const bool free_shape = !cfg_in && (!db.cfg_set || db.cfg_tuned);
     if (cfg.queries_per_launch == 1) {
         if (direct_out) return fail(IMPIR_EINVAL, "direct answers need one launch for the batch");
         if (ws_bytes < ws_layout(1, db.stride).total) return fail(IMPIR_ENOMEM, "workspace too small");
@@ -399,7 +396,7 @@ impir_status answer_async_impl(const Db& db, const impir_config* cfg_in, const u
         return fail(IMPIR_ENOMEM, "workspace of %zu bytes is smaller than the %zu needed", ws_bytes,
                     ws_layout(n, db.stride).total);
     return launch_batch(*dev, db, cfg, d_keys, d_off, n, direct_out ? nullptr : d_out, static_cast<uint8_t*>(d_ws), st,
-                        mode, keys_bytes, tc_allowed);
+                        mode, keys_bytes, free_shape);
 }
 
 // ---- synchronous path context: cached device and pinned buffers ----

@@ -185,28 +185,32 @@ inline SmemSplit split_smem(uint32_t warps, size_t slice) {
 // units (fused.cuh); else units go to the warps whole, so the last, partly filled round counts in full.
 // The scan's reads: every group reads the tiles it covers, the first from HBM, the others from L2 if
 // the tiles in work at a time fit there.
-inline double shape_clocks(const impir_config& c, uint64_t n_records, uint32_t words, uint32_t n_queries, int sms) {
+// The additive answer (add): every lane walks the last five levels by itself, for each query.
+inline double shape_clocks(const impir_config& c, uint64_t n_records, uint32_t words, uint32_t n_queries, int sms,
+                           bool add = false) {
     const double slots = c.queries_per_warp, s = c.lane_bits, w = c.warps_per_cta;
     const double groups = std::ceil(n_queries / slots), tiles = std::ceil(double(n_records) / double(32ull << c.lane_bits));
     const double q = n_queries / groups, m = std::ceil(std::log2(double(n_records)));
     const double units = groups * tiles, top = std::max(0.0, m - s - 5);
-    const double scan = std::exp2(s) * words * (4.3 * slots + 4) / 560;
-    const double lanes = q * (0.8 + std::exp2(s) - 1), slow = 1 + 0.012 * slots;
+    const double scan = std::exp2(s) * words * (4.3 * slots + (add ? 14 : 4)) / 560;
+    const double lanes = q * (0.8 + (add ? 4 * 0.65 : 0) + std::exp2(s) - 1), slow = 1 + 0.012 * slots;
     const uint32_t nk = nk_xor(words, c.queries_per_warp);
     const double per_load = nk == 1 ? (slots == 1 ? 16 : slots == 2 ? 8 : 4) * std::max(1u, 32 / words) : nk <= 2 ? 4 : nk == 4 ? 2 : 1;
     const double loads = std::ceil(32 * std::exp2(s) / per_load) * std::ceil(words / (32.0 * nk));
     double clocks, hbm = 3300;
     if (units <= sms * w) {
-        const double n = std::ceil(units / sms), shared = n > 4 ? n : 1;  // warps whose levels are expanded together
-        clocks = top * std::max(1750.0, 200 * std::ceil(shared * q / 32) * (n > 4 ? 1 : n)) +
+        const double n = std::ceil(units / sms);
+        const bool cta = n > 4 && !add;
+        const double shared = cta ? n : 1;  // warps whose levels are expanded together
+        clocks = top * std::max(1750.0, 200 * std::ceil(shared * q / 32) * (cta ? 1 : n)) +
                  slow * lanes * std::max(2000.0, 330 * n + 700) +
                  std::max(slow * scan * std::max(2000.0, 330 * n + 700), 900 * loads);
         hbm = std::min(hbm, 400 * n);
-        for (int k = 0; k < 4; ++k)
-            clocks += std::max(2500.0, 330 * std::ceil(shared * q * double(1 << k) / 32) * (n > 4 ? 1 : n));
+        for (int k = 0; k < 4 && !add; ++k)
+            clocks += std::max(2500.0, 330 * std::ceil(shared * q * double(1 << k) / 32) * (cta ? 1 : n));
     } else {
         double coop = 0;
-        for (int k = 0; k < 4; ++k) coop += 1.3 * std::ceil(q * double(1 << k) / 32);
+        for (int k = 0; k < 4 && !add; ++k) coop += 1.3 * std::ceil(q * double(1 << k) / 32);
         const double full = std::floor(units / (sms * w)), left = std::ceil((units - full * sms * w) / sms);
         clocks = (top + coop + lanes + scan) * slow * (full * (330 * w + 700) + (left > 0 ? 330 * left + 1400 : 0));
     }
@@ -270,16 +274,16 @@ struct XorShape {
     uint32_t tile_bits() const { return tc ? std::max(kTcLaneBits, c.lane_bits) : c.lane_bits; }
 };
 
-// tc_allowed: the caller set no launch shape of its own.
-inline XorShape xor_shape(const impir_config& c, bool tc_allowed, uint64_t n_records, uint32_t words,
-                          uint32_t n_queries, int sms) {
+// free_shape: the caller set no launch shape of its own; add: the additive answer (warp kernels only).
+inline XorShape xor_shape(const impir_config& c, bool free_shape, uint64_t n_records, uint32_t words,
+                          uint32_t n_queries, int sms, bool add = false) {
     XorShape s{c, false, 0, 0};
     // as many units as a batch that covers the database has, but 16 per SM are enough
     const uint64_t T = 32ull << c.lane_bits;
-    if (tc_allowed)
+    if (free_shape)
         s.want_units = std::min<uint64_t>(16ull * sms, ((n_records + T - 1) / T) *
                                                            ((n_queries + c.queries_per_warp - 1) / c.queries_per_warp));
-    if (!tc_allowed || c.queries_per_launch != 0 || n_queries < tc_min_queries(words)) return s;
+    if (!free_shape || add || c.queries_per_launch != 0 || n_queries < tc_min_queries(words)) return s;
     const uint64_t groups = (n_queries + kTcQueries - 1) / kTcQueries;
     if (groups * ((n_records + (32u << kTcLaneBits) - 1) >> (kTcLaneBits + 5)) < tc_min_units(words, sms)) return s;
     s.tc = true;
