@@ -655,12 +655,13 @@ __device__ __forceinline__ NodePair child_nodes(uint32_t prf, const uint8_t* kq,
     return prf == 0 ? child_nodes<0>(kq, m, n, d, L) : child_nodes<1>(kq, m, n, d, L);
 }
 
-// Selection bits of the 2^s leaves (1 <= s <= 5) below `node` (at depth m - s), leaf r in bit r. Depth
-// first; the right child of a depth m - 2 node waits in registers, only those above it go through the
-// (local-memory) stack.
+// Selection bits of the 2^s leaves (s >= 1) below `node` (at depth m - s), leaf r in bit r: returned for
+// s <= 5, else stored at out[0 ...], a word per 32 leaves. Depth first; the right child of a depth m - 2
+// node waits in registers, only those above it go through the (local-memory) stack.
 template <int PRF>
-__device__ __noinline__ uint32_t subtree_word(const uint8_t* kq, uint32_t m, uint32_t s, Blk node, uint32_t L) {
-    Blk stk[5];
+__device__ __noinline__ uint32_t subtree_bits(const uint8_t* kq, uint32_t m, uint32_t s, Blk node, uint32_t L,
+                                              uint32_t* out) {
+    Blk stk[kMaxLaneBits];
     Blk wait{0, 0, 0, 0};                // right child at depth m - 1
     // the leaf codewords' lowest bits, bit 2 t + x for C_t[x][m]
     const uint32_t lsbs = cw_lsb(kq, m, 0, 0, m) | cw_lsb(kq, m, 0, 1, m) << 1 | cw_lsb(kq, m, 1, 0, m) << 2 |
@@ -678,13 +679,18 @@ __device__ __noinline__ uint32_t subtree_word(const uint8_t* kq, uint32_t m, uin
         if (left == 0) {
             uint32_t b2 = PRF == 0 ? keyed_leaf_bits_tail(L, k, a, b) : mmo_leaf_bits_tail(node, L, c_mmo.rk, a, b);
             b2 = (b2 ^ (lsbs >> (2 * t))) & 3u;
-            acc |= b2 << (2 * p);
+            acc |= b2 << (2 * p & 31);
             ++p;
+            if (s > 5 && (p & 15) == 0) {
+                if (slice_ok(out, 4)) *out = acc;
+                ++out;
+                acc = 0;
+            }
             if (p >> (s - 1)) return acc;
             left = __ffs(int(p)) - 1;
             if (left == 0)
                 node = wait;
-            else if (IMPIR_IN_BOUNDS(left < 5, kSiteStack, left))
+            else if (IMPIR_IN_BOUNDS(left < kMaxLaneBits, kSiteStack, left))
                 node = stk[left];
         } else {
             const Blk c0 = cw_load(kq, m, t, 0, m - left), c1 = cw_load(kq, m, t, 1, m - left);
@@ -695,16 +701,16 @@ __device__ __noinline__ uint32_t subtree_word(const uint8_t* kq, uint32_t m, uin
             --left;
             if (left == 0)
                 wait = b;
-            else if (IMPIR_IN_BOUNDS(left < 5, kSiteStack, left))
+            else if (IMPIR_IN_BOUNDS(left < kMaxLaneBits, kSiteStack, left))
                 stk[left] = b;
             node = a;
         }
     }
 }
 
-__device__ __forceinline__ uint32_t subtree_word(uint32_t prf, const uint8_t* kq, uint32_t m, uint32_t s, Blk node,
-                                                 uint32_t L) {
-    return prf == 0 ? subtree_word<0>(kq, m, s, node, L) : subtree_word<1>(kq, m, s, node, L);
+__device__ __forceinline__ uint32_t subtree_bits(uint32_t prf, const uint8_t* kq, uint32_t m, uint32_t s, Blk node,
+                                                 uint32_t L, uint32_t* out = nullptr) {
+    return prf == 0 ? subtree_bits<0>(kq, m, s, node, L, out) : subtree_bits<1>(kq, m, s, node, L, out);
 }
 
 // From `start`, the node at depth d0 on the path to node `sub` of depth D (the root with d0 = 0, or the
@@ -717,35 +723,17 @@ __device__ __forceinline__ Blk walk_down(uint32_t prf, const uint8_t* kq, uint32
 }
 
 // Selection bits of the lane's subtree of 2^sq leaves below node `sub` of depth D: bit r of `bits`
-// (relative to the warp tile) is lsb(R(m, tile_first_leaf + r)). Subtrees above 32 leaves go depth
-// first down to those of 32.
+// (relative to the warp tile) is lsb(R(m, tile_first_leaf + r)).
 __device__ __forceinline__ void lane_eval(uint32_t prf, const uint8_t* kq, uint32_t m, uint32_t D, uint64_t sub,
                                           uint32_t sq, uint32_t* bits, uint32_t lane, uint32_t L, const Blk start,
                                           uint32_t d0) {
-    Blk node = walk_down(prf, kq, m, D, sub, L, start, d0);
+    const Blk node = walk_down(prf, kq, m, D, sub, L, start, d0);
+    uint32_t* w = &bits[(lane << sq) >> 5];
+    const uint32_t word = sq == 0 ? node.x & 1u : subtree_bits(prf, kq, m, sq, node, L, w);
     if (sq < 5) {
-        const uint32_t word = sq == 0 ? node.x & 1u : subtree_word(prf, kq, m, sq, node, L);
-        if (slice_ok(&bits[(lane << sq) >> 5], 4)) atomicOr(&bits[(lane << sq) >> 5], word << ((lane << sq) & 31));
-        return;
-    }
-    Blk stk[kMaxLaneBits - 5 + 1];
-    uint32_t left = sq - 5, w = 0;  // levels between the node and the 32-leaf subtrees; words done
-#pragma unroll 1
-    for (;;) {
-        if (left) {
-            const NodePair p = child_nodes(prf, kq, m, node, m - 5 - left + 1, L);
-            --left;
-            if (IMPIR_IN_BOUNDS(left <= kMaxLaneBits - 5, kSiteStack, left)) stk[left] = p.b;
-            node = p.a;
-            continue;
-        }
-        uint32_t* out = &bits[(lane << (sq - 5)) + w];
-        const uint32_t word = subtree_word(prf, kq, m, 5, node, L);
-        if (slice_ok(out, 4)) *out = word;
-        ++w;
-        if (w >> (sq - 5)) return;
-        left = __ffs(int(w)) - 1;
-        if (IMPIR_IN_BOUNDS(left <= kMaxLaneBits - 5, kSiteStack, left)) node = stk[left];
+        if (slice_ok(w, 4)) atomicOr(w, word << ((lane << sq) & 31));
+    } else if (sq == 5 && slice_ok(w, 4)) {
+        *w = word;
     }
 }
 

@@ -226,7 +226,7 @@ __device__ __forceinline__ void aes_task(const FusedParams& P, uint32_t b, uint3
             Blk n = shfl_child(a, c, i * 8 + (lane >> 2), (lane >> 1) & 1);
             if (tile * K + (lane << S) < P.n_records) {
                 n = child_node(prf, kq, m, n, lane & 1u, m - S, L);
-                word = subtree_word(prf, kq, m, S, n, L);
+                word = subtree_bits(prf, kq, m, S, n, L);
             }
             __syncwarp();
         } else {

@@ -193,7 +193,7 @@ inline double shape_clocks(const impir_config& c, uint64_t n_records, uint32_t w
     const double q = n_queries / groups, m = std::ceil(std::log2(double(n_records)));
     const double units = groups * tiles, top = std::max(0.0, m - s - 5);
     const double scan = std::exp2(s) * words * (4.3 * slots + (add ? 14 : 4)) / 560;
-    const double lanes = q * (0.8 + (add ? 4 * 0.65 : 0) + std::exp2(s) - 1), slow = 1 + 0.012 * slots;
+    const double lanes = q * (0.8 + (add ? 4 * 0.65 : 0) + std::exp2(s) - 1), slow = 1 + 0.010 * slots;
     const uint32_t nk = nk_xor(words, c.queries_per_warp);
     const double per_load = nk == 1 ? (slots == 1 ? 16 : slots == 2 ? 8 : 4) * std::max(1u, 32 / words) : nk <= 2 ? 4 : nk == 4 ? 2 : 1;
     const double loads = std::ceil(32 * std::exp2(s) / per_load) * std::ceil(words / (32.0 * nk));
@@ -212,11 +212,12 @@ inline double shape_clocks(const impir_config& c, uint64_t n_records, uint32_t w
         double coop = 0;
         for (int k = 0; k < 4 && !add; ++k) coop += 1.3 * std::ceil(q * double(1 << k) / 32);
         const double full = std::floor(units / (sms * w)), left = std::ceil((units - full * sms * w) / sms);
-        clocks = (top + coop + lanes + scan) * slow * (full * (330 * w + 700) + (left > 0 ? 330 * left + 1400 : 0));
+        clocks = (1.3 * (top + coop) + lanes + scan) * slow * (full * (330 * w + 700) + (left > 0 ? 330 * left + 1400 : 0));
     }
     const double record = words * 16.0 * (c.queries_per_warp == 1 ? 0.5 : 1.0), pass = double(n_records) * record;
     const double live = std::min(units, sms * w) / groups * double(32ull << c.lane_bits) * record;
-    return clocks + pass * (groups > 1 && live > 64e6 ? groups : 1.0) / hbm + pass * groups / 5000;
+    const double passes = 1 + (groups - 1) * std::min(1.0, std::max(0.0, (live - 64e6) / 192e6));
+    return clocks + pass * passes / hbm + pass * groups / 5000;
 }
 
 // The shape with the smallest estimate (lane subtrees of at most 2^8 leaves).
@@ -278,10 +279,10 @@ struct XorShape {
 inline XorShape xor_shape(const impir_config& c, bool free_shape, uint64_t n_records, uint32_t words,
                           uint32_t n_queries, int sms, bool add = false) {
     XorShape s{c, false, 0, 0};
-    // as many units as a batch that covers the database has, but 16 per SM are enough
+    // as many units as a batch that covers the database has, but 40 per SM are enough
     const uint64_t T = 32ull << c.lane_bits;
     if (free_shape)
-        s.want_units = std::min<uint64_t>(16ull * sms, ((n_records + T - 1) / T) *
+        s.want_units = std::min<uint64_t>(40ull * sms, ((n_records + T - 1) / T) *
                                                            ((n_queries + c.queries_per_warp - 1) / c.queries_per_warp));
     if (!free_shape || add || c.queries_per_launch != 0 || n_queries < tc_min_queries(words)) return s;
     const uint64_t groups = (n_queries + kTcQueries - 1) / kTcQueries;
