@@ -173,14 +173,16 @@ size_t impir_workspace_bytes(uint32_t n_queries, uint32_t stride_bytes);
  * completes. The device checks each key's header, column 0 and 8-byte alignment, not the
  * extent of d_keys (the call has no length for it): the caller guarantees that every offset
  * starts a whole key, impir_key_bytes(m) bytes for the m in its header, inside d_keys.
- * Launch errors return ECUDA. */
+ * Launch errors return ECUDA. Where records carry no padding and d_out is 16-byte aligned memory of
+ * the current device, the answers are accumulated in d_out itself while the call's kernels run. */
 impir_status impir_answer_async(int32_t db_handle, const uint8_t* d_keys, const uint32_t* d_key_offsets,
                                 uint32_t n_queries, uint8_t* d_out, void* d_workspace, size_t workspace_bytes,
                                 void* cuda_stream);
 
 /* Reads the device-side status of the last asynchronous answer that used d_workspace
  * (synchronizes with the device). *n_bad = number of malformed keys, *first_bad = the
- * smallest index among them (UINT32_MAX when none). */
+ * smallest index among them (UINT32_MAX when none). ECUDA also when a wait between the warps of the
+ * tensor-core kernel ran out (20 s): the answers are then not valid. */
 impir_status impir_workspace_status(const void* d_workspace, uint32_t* n_bad, uint32_t* first_bad);
 
 /* ---- Launch configuration and autotuning ---- */
@@ -206,7 +208,10 @@ typedef struct {
 
 /* Gets the configuration a batch of n_queries keys would be launched with on this database
  * (the one set or tuned for it, else the built-in default for that batch size), or sets one
- * for all later batches (set validates it: EINVAL). */
+ * for all later batches (set validates it: EINVAL). A shape that was set is launched as it is.
+ * Otherwise tiles that 64 or more queries reach (96 for records above 512 bytes) go to the
+ * tensor-core kernel, which has one shape, and the configuration describes the launch for the
+ * others; its lane_bits is then an upper limit (queries whose domains end early get smaller tiles). */
 impir_status impir_get_config(int32_t db_handle, uint32_t n_queries, impir_config* cfg);
 impir_status impir_set_config(int32_t db_handle, const impir_config* cfg);
 

@@ -7,24 +7,26 @@
 // How (GB300 mapping of the paper's subtree split and two-stage reduction):
 //   * Work unit = (warp tile, query group). A warp tile is 32 * 2^s consecutive leaves: lane l
 //     owns the perfect subtree of 2^s leaves rooted at depth m - s (the paper's worker
-//     subtrees, §3.2). A query group is up to QC queries of one domain size (§3.4 batching).
+//     subtrees, §3.2). A query group is up to QC queries (§3.4 batching), of any mix of domain sizes
+//     of at least one tile.
 //   * The path root -> warp-tile root (the branch-parallel walk, one AES per level) is walked
-//     once per query of the group (lane q for query q); the warp then expands the five levels
-//     below it for the whole group together, so that every lane holds its subtree root for
-//     every query. Each lane expands its subtree depth-first, two children per AES key
-//     schedule, and writes the 2^s selection bits of its leaves into shared memory. Selection
-//     bits never touch HBM.
+//     once per query of the group, lane by lane; the warp then expands four levels below it for the
+//     whole group together (for a block's first units all its warps do both together), and every lane
+//     takes the fifth to its subtree root for every query. Each lane expands its subtree depth-first,
+//     two children per AES key schedule, and writes the 2^s selection bits of its leaves into shared
+//     memory. Selection bits never touch HBM.
 //   * The warp then reads the tile's records once (coalesced 16-byte loads, several in flight
-//     per lane) and XORs each record into the QC per-query accumulators held in registers
-//     (TaskletXOR), folds lanes with warp shuffles (MasterXOR), and XORs the result into the
-//     per-query answer in global memory with 64-bit atomic XOR (AggregateSubresults; XOR is
-//     order-independent, so the result is bit-exact whatever the order).
+//     per lane; with one or two queries only the selected ones) and XORs each record into the QC
+//     per-query accumulators held in registers (TaskletXOR), folds lanes with warp shuffles (MasterXOR),
+//     and XORs the result into the per-query answer in global memory with 64-bit atomic XOR
+//     (AggregateSubresults; XOR is order-independent, so the result is bit-exact whatever the order).
+//   * Batches of many queries take the tensor-core form of the same computation (fused_tc.cu).
 //   * MODE 1, the additive answer over Z_2^32: one or two queries per unit, 32-bit shares
 //     instead of bits, the queries' walks advanced in turn by chunks of leaves and each chunk's
 //     records scanned once for all of them with integer multiply-adds.
-//   * A persistent grid, one CTA of 16 or 20 warps per SM: warps take work units from a global
-//     counter, units ordered tile-major so that concurrently running warps read the same DB
-//     tile (served from L2).
+//   * A persistent grid, one CTA of 16 or 20 warps per SM: each warp's first unit is fixed, the
+//     others come from a global counter, units ordered tile-major so that concurrently running warps
+//     read the same DB tile (served from L2).
 //
 // AES: 32-bit T-tables (Te0..Te3) replicated per lane in shared memory. Row x of a 64 KiB
 // region holds [Te_a[x] for lanes 0..31 | Te_b[x] for lanes 0..31] (256 bytes), so the byte
@@ -103,7 +105,9 @@ __device__ __forceinline__ bool slice_ok(const void* p, uint32_t n, uint32_t war
 }
 
 // A 32-bit word of the warp's bit / share buffer (zero if a debug-build check fails).
-__device__ __forceinline__ uint32_t ld_slice(const uint32_t* p) { return slice_ok(p, 4) ? *p : 0u; }
+__device__ __forceinline__ uint32_t ld_slice(const uint32_t* p) {
+    return slice_ok(p, 4) ? *p : 0u;
+}
 
 struct Blk {
     uint32_t x, y, z, w;
@@ -749,13 +753,10 @@ struct AddWalk {
 
 // Advances the walk by ch leaves (ch >= 2, even): the shares (-1)^party low32(R(m, j)) of the
 // lane's next ch leaves go to shares[lane * ch + 0 .. ch - 1].
-// A function of its own: inlined, each query of a unit and each PRF had a copy of the AES rounds, and
-// a batch that mixes the PRFs fetched instructions half the time (198 mixed queries on 2^22 records
-// of 128 bytes: 64.3 ms inlined, 33.3 ms so; 64 keyed ones on 2^20 x 256 bytes 3654 and 3619 us).
 template <int PRF>
-__device__ __noinline__ void add_walk_chunk(const uint8_t* kq, uint32_t m, uint32_t D,
-                                               uint32_t sq, AddWalk& w, uint32_t ch, uint32_t* shares, uint32_t lane,
-                                               uint32_t L, uint32_t neg) {
+__device__ __forceinline__ void add_walk_chunk_inline(const uint8_t* kq, uint32_t m, uint32_t D, uint32_t sq, AddWalk& w,
+                                                      uint32_t ch, uint32_t* shares, uint32_t lane, uint32_t L,
+                                                      uint32_t neg) {
     Blk node = w.node;
     uint32_t depth = w.depth, p = w.p;
     const uint32_t npairs = 1u << (sq - 1), end = p + ch / 2;
@@ -799,6 +800,16 @@ __device__ __noinline__ void add_walk_chunk(const uint8_t* kq, uint32_t m, uint3
     w.node = node;
     w.depth = depth;
     w.p = p;
+}
+
+// The same as a function of its own: inlined, each query of a unit and each PRF has a copy of the AES
+// rounds, and a batch that mixes the PRFs fetched instructions half the time (198 mixed queries on 2^22
+// records of 128 bytes: 64.3 ms inlined, 33.3 ms so). Records above 1 KiB, whose accumulators fill the
+// registers, keep it inlined (16 queries on 2^19 x 2 KiB: 1290 us inlined, 1400 with calls).
+template <int PRF>
+__device__ __noinline__ void add_walk_chunk(const uint8_t* kq, uint32_t m, uint32_t D, uint32_t sq, AddWalk& w,
+                                            uint32_t ch, uint32_t* shares, uint32_t lane, uint32_t L, uint32_t neg) {
+    add_walk_chunk_inline<PRF>(kq, m, D, sq, w, ch, shares, lane, L, neg);
 }
 
 // One work unit of the additive answer: the group's queries over one warp tile. Every lane
@@ -847,10 +858,16 @@ __device__ __forceinline__ void unit_add(const FusedParams& P, const GroupDesc& 
         for (int q = 0; q < QC; ++q)
             if (uint32_t(q) < count) {
                 const uint8_t* kq = query_key(P, query_at(P, qidx, q));
-                if (kq[1] == 0)
+                if constexpr (NK >= 4) {
+                    if (kq[1] == 0)
+                        add_walk_chunk_inline<0>(kq, m, D, sq, w[q], ch, shares + q * qstride, lane, L, neg[q]);
+                    else
+                        add_walk_chunk_inline<1>(kq, m, D, sq, w[q], ch, shares + q * qstride, lane, L, neg[q]);
+                } else if (kq[1] == 0) {
                     add_walk_chunk<0>(kq, m, D, sq, w[q], ch, shares + q * qstride, lane, L, neg[q]);
-                else
+                } else {
                     add_walk_chunk<1>(kq, m, D, sq, w[q], ch, shares + q * qstride, lane, L, neg[q]);
+                }
             }
         __syncwarp();
         scan_chunk_add<QC, NK>(P, tile_base, nrec, shares, qstride, count, qidx, runs, run_len, sq, c * ch, acc_out,

@@ -246,15 +246,14 @@ impir_config default_add_config(uint64_t n_records, uint32_t words, uint32_t n_q
     impir_config best{};
     double best_t = 0;
     for (uint32_t qpw = 1; qpw <= std::min(max_add_qpw(words), n_queries); qpw *= 2)
-        for (uint32_t w = 16; w <= (nk_need(words) == 1 ? 20u : 16u); w += 4)
-            for (uint32_t b = 0; b <= 8; ++b) {
-                const impir_config c{b, qpw, w, 0};
-                const double t = shape_clocks(c, n_records, words, n_queries, sms, true);
-                if (best_t == 0 || t < best_t) {
-                    best_t = t;
-                    best = c;
-                }
+        for (uint32_t b = 0; b <= 8; ++b) {
+            const impir_config c{b, qpw, nk_need(words) == 1 ? 20u : 16u, 0};
+            const double t = shape_clocks(c, n_records, words, n_queries, sms, true);
+            if (best_t == 0 || t < best_t) {
+                best_t = t;
+                best = c;
             }
+        }
     return best;
 }
 
@@ -358,7 +357,7 @@ impir_status launch_batch(const DeviceState& dev, const Db& db, const impir_conf
     zp.record_bytes = db.bytes;
     zp.stride = db.stride;
     zp.bounds = sp.bounds;
-    CK(launch_finalize(zp, st), "finalize kernel launch");
+    CK(launch_finalize(zp, st, !timed), "finalize kernel launch");
     return IMPIR_OK;
 }
 
@@ -979,7 +978,7 @@ impir_status impir_answer_streamed(const void* records, uint64_t N, uint32_t B, 
         zp.record_bytes = B;
         zp.stride = stride;
         zp.bounds = bounds_record();
-        e = launch_finalize(zp, ks[0]);
+        e = launch_finalize(zp, ks[0], false);
         count_launches(1);
     }
     WsHeader hdr[2] = {};

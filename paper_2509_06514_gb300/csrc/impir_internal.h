@@ -180,9 +180,9 @@ inline SmemSplit split_smem(uint32_t warps, size_t slice) {
 // costs a warp the walk to the tile, four cooperative levels, the lanes' subtrees and the scan's share
 // of the ALU pipe, counted in node pairs. A pair takes a warp 2000 clocks by itself (a single child
 // 1750), and an SM's warps together 330 each (the lookups' shared-memory port); a round of record
-// loads 900. Where every unit finds
-// a warp at once, the block's warps share the walk and the cooperative levels if it has more than four
-// units (fused.cuh); else units go to the warps whole, so the last, partly filled round counts in full.
+// loads 900. Where every unit finds a warp at once, the block's warps share the walk and the
+// cooperative levels if it has more than four units (fused.cuh); else the port is busy throughout, and
+// the last units add their latency.
 // The scan's reads: every group reads the tiles it covers, the first from HBM, the others from L2 if
 // the tiles in work at a time fit there.
 // The additive answer (add): every lane walks the last five levels by itself, for each query.
@@ -211,10 +211,10 @@ inline double shape_clocks(const impir_config& c, uint64_t n_records, uint32_t w
     } else {
         double coop = 0;
         for (int k = 0; k < 4 && !add; ++k) coop += 1.3 * std::ceil(q * double(1 << k) / 32);
-        const double full = std::floor(units / (sms * w)), left = std::ceil((units - full * sms * w) / sms);
-        clocks = (1.3 * (top + coop) + lanes + scan) * slow * (full * (330 * w + 700) + (left > 0 ? 330 * left + 1400 : 0));
+        clocks = (1.3 * (top + coop) + lanes + scan) * slow * (1.04 - 0.005 * s) * (320 * (1 + 0.4 / w) * units / sms + 2000);
+        hbm *= 2;  // (reads of one unit pass under another's lookups)
     }
-    const double record = words * 16.0 * (c.queries_per_warp == 1 ? 0.5 : 1.0), pass = double(n_records) * record;
+    const double record = words * 16.0 * (c.queries_per_warp == 1 && !add ? 0.5 : 1.0), pass = double(n_records) * record;
     const double live = std::min(units, sms * w) / groups * double(32ull << c.lane_bits) * record;
     const double passes = 1 + (groups - 1) * std::min(1.0, std::max(0.0, (live - 64e6) / 192e6));
     return clocks + pass * passes / hbm + pass * groups / 5000;
@@ -226,20 +226,21 @@ inline impir_config default_config(uint64_t n_records, uint32_t words, uint32_t 
     double best_t = 0;
     for (uint32_t qpw = 1; qpw <= 8; qpw *= 2) {
         if (qpw * nk_xor(words, qpw) > 16 || (qpw > 1 && qpw / 2 >= n_queries)) continue;
-        for (uint32_t w = 16; w <= max_warps(qpw, words); w += 4)
-            for (uint32_t b = 0; b <= 8; ++b) {
-                const impir_config c{b, qpw, w, 0};
-                if (smem_for(c) > kSmemMax) continue;
-                // groups that share a database above L2's size: tiles of at most 512 KiB, read again while
-                // they are there (18 queries on 2^21 x 256 B: 1395 us with tiles of 1 MiB, 1086 with 256 KiB)
-                if (b > 0 && n_queries > qpw && uint64_t(n_records) * words > (64u << 20) / 16 && (uint64_t(words) << (b + 9)) > (512u << 10))
-                    continue;
-                const double t = shape_clocks(c, n_records, words, n_queries, sms);
-                if (best_t == 0 || t < best_t) {
-                    best_t = t;
-                    best = c;
-                }
+        // as many warps as the kernel is built for (16 were never more than 1 % faster than 20, and 50 %
+        // slower where the units just fill 20)
+        for (uint32_t b = 0; b <= 8; ++b) {
+            const impir_config c{b, qpw, max_warps(qpw, words), 0};
+            if (smem_for(c) > kSmemMax) continue;
+            // groups that share a database above L2's size: tiles of at most 512 KiB, read again while
+            // they are there (18 queries on 2^21 x 256 B: 1395 us with tiles of 1 MiB, 1086 with 256 KiB)
+            if (b > 0 && n_queries > qpw && uint64_t(n_records) * words > (64u << 20) / 16 && (uint64_t(words) << (b + 9)) > (512u << 10))
+                continue;
+            const double t = shape_clocks(c, n_records, words, n_queries, sms);
+            if (best_t == 0 || t < best_t) {
+                best_t = t;
+                best = c;
             }
+        }
     }
     return best;
 }
@@ -358,7 +359,8 @@ BoundsRecord* bounds_record();
 // uint4 words of a database the index checks allow the kernels to read: n_words, less the
 // records a debug-build test withholds (IMPIR_BOUNDS_TEST_WITHHOLD_RECORDS) to see a check fire.
 unsigned long long bounds_db_words(unsigned long long n_words, uint32_t words_per_record);
-cudaError_t launch_finalize(const FinalizeParams& p, cudaStream_t s);
+// follows: nothing but the fused kernel's launch came before it in the stream (a dependent launch).
+cudaError_t launch_finalize(const FinalizeParams& p, cudaStream_t s, bool follows);
 // The XOR answer's fused launch in the given shape: sets the shape's fields of the setup
 // parameters (before launch_setup) and launches the kernel it names.
 void apply_shape(const XorShape& s, int sms, SetupParams* sp);

@@ -151,7 +151,7 @@ extern "C" impir_status impir_answer_noalloc(const void* d_records, uint64_t n_r
     zp.record_bytes = record_bytes;
     zp.stride = stride_bytes;
     zp.bounds = dev->bounds;
-    if (launch_finalize(zp, st) != cudaSuccess) {
+    if (launch_finalize(zp, st, true) != cudaSuccess) {
         cudaGetLastError();
         return set_error(IMPIR_ECUDA, "finalize kernel launch failed");
     }

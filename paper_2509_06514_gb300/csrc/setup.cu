@@ -1,14 +1,15 @@
 // setup.cu — per-batch scheduling and answer write-out kernels.
 //
 // setup_kernel (one CTA) reads the key headers on the device, validates them, sorts the
-// queries by domain size (largest first), forms query groups of one domain size (the
-// paper's queries handled together, §3.4), and builds the tile-major work-unit schedule the
-// fused kernel walks: warp tile i is covered by every group whose DB prefix min(N, 2^m)
-// reaches it, so the schedule is a handful of segments (one per distinct domain size). It
-// also zeroes the per-query accumulators and the work counter.
+// queries by domain size (largest first), forms query groups (the paper's queries handled
+// together, §3.4), and builds the tile-major work-unit schedule the fused kernels walk: a tile is
+// covered by every group whose DB prefix min(N, 2^m) reaches it, so the schedule is a handful of
+// segments (one per distinct domain size). Tiles that enough queries reach are scheduled for the
+// tensor-core kernel, the rest for the warp kernels. It also zeroes the per-query accumulators
+// and the work counters.
 //
 // finalize_kernel copies each query's accumulator (record stride) into the caller's
-// answer buffer (record_bytes per query).
+// answer buffer (record_bytes per query) where the answers were not accumulated there.
 #include <algorithm>
 #include <cstdlib>
 
@@ -301,10 +302,12 @@ cudaError_t launch_setup(const SetupParams& p, cudaStream_t s) {
     return cudaGetLastError();
 }
 
-cudaError_t launch_finalize(const FinalizeParams& p, cudaStream_t s) {
+cudaError_t launch_finalize(const FinalizeParams& p, cudaStream_t s, bool follows) {
     const size_t n = size_t(p.n_queries) * p.record_bytes;
     const unsigned blocks = unsigned(n / 256 + 1 < 1024 ? n / 256 + 1 : 1024);
-    return launch_after(finalize_kernel, dim3(blocks), dim3(256), 0, s, p);
+    if (follows) return launch_after(finalize_kernel, dim3(blocks), dim3(256), 0, s, p);
+    finalize_kernel<<<blocks, 256, 0, s>>>(p);
+    return cudaGetLastError();
 }
 
 cudaError_t launch_fused(uint32_t qpw, uint32_t nk, dim3 grid, dim3 block, size_t smem, cudaStream_t s,
