@@ -1135,10 +1135,9 @@ __global__ void __launch_bounds__((NK == 1 && QC <= 8) ? 640 : 512, 1)
     const uint32_t lane = tid & 31, warp = tid >> 5;
 
     WsHeader* hdr = reinterpret_cast<WsHeader*>(P.ws);
-    // behind the setup kernel the tables are filled while it runs; behind the tensor-core kernel there
-    // may be nothing left to do
-    if (P.after_tc) grid_wait();
-    if (P.after_tc && hdr->n_units == 0) return;
+    // the tables are filled while the setup kernel runs, unless there may be nothing to do
+    if (P.with_tc) grid_wait();
+    if (P.with_tc && hdr->n_units == 0) return;
     const bool tables = fill_tables(P.te0, tid, nthr);
     grid_wait();
     if (!tables) {

@@ -331,7 +331,7 @@ struct FusedParams {
     uint32_t n_queries;
     uint32_t words;          // uint4 words per record (stride / 16)
     uint32_t bits_words;     // 32-bit words of selection bits (additive: shares) per (warp, query slot)
-    uint32_t after_tc;       // the tensor-core kernel is the one before this in the stream
+    uint32_t with_tc;        // the tensor-core kernel takes part of the batch: nothing may be left here
     uint32_t slices_low;     // warps whose slice of those lies below the tables
     unsigned long long rec_lo;  // global index of the record at db[0] (0 unless a chunk or a row shard)
     // extents for the debug build's index checks

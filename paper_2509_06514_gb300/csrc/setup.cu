@@ -333,18 +333,20 @@ void apply_shape(const XorShape& s, int sms, SetupParams* sp) {
 }
 
 cudaError_t launch_xor(const XorShape& s, int sms, cudaStream_t st, FusedParams& fp) {
-    if (s.tc) {
-        fp.smem_bytes = tc_smem_bytes();
-        const cudaError_t e = launch_fused_tc(sms, st, fp);
-        if (e != cudaSuccess) return e;
-    }
-    fp.after_tc = s.tc ? 1u : 0u;
+    // The warp kernel's share, often none, goes first: behind the tensor-core kernel it would wait for an
+    // SM while another stream's launch fills the chip (a streamed database's next chunk, another batch of
+    // a server), and with it everything that waits for this batch: 416 uneven queries on 8 GiB streamed
+    // in 2 GiB chunks 302-308 ms behind it, 286 before it.
+    fp.with_tc = s.tc ? 1u : 0u;
     fp.bits_words = bits_words(s.c);
     const SmemSplit sp = split_smem(s.c.warps_per_cta, size_t(s.c.queries_per_warp) * fp.bits_words * 4);
     fp.slices_low = sp.low;
     fp.smem_bytes = sp.bytes;
-    return launch_fused(s.c.queries_per_warp, nk_xor(fp.words, s.c.queries_per_warp), dim3(sms), dim3(sp.warps * 32),
-                        sp.bytes, st, fp);
+    const cudaError_t e = launch_fused(s.c.queries_per_warp, nk_xor(fp.words, s.c.queries_per_warp), dim3(sms),
+                                       dim3(sp.warps * 32), sp.bytes, st, fp);
+    if (e != cudaSuccess || !s.tc) return e;
+    fp.smem_bytes = tc_smem_bytes();
+    return launch_fused_tc(sms, st, fp);
 }
 
 cudaError_t prepare_xor_kernels() {

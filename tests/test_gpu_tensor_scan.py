@@ -45,14 +45,14 @@ def check(orc, N, B, keys, sample):
 
 
 @pytest.mark.parametrize("N,B,ms", [
-    (623_617, 16, [20] * 48),                                # 609 tiles, one record in the last; one column pass
+    (623_617, 16, [20] * 64),                                # 609 tiles, one record in the last; one column pass
     (640_000, 40, [20] * 65),                                # three words: a one-word last pass
     (78_000, 256, [17] * 1024),                              # eight full groups of 128 rows
     (80_001, 100, [17, 16, 13, 11, 10, 9, 6, 1, 40] * 115),  # domains below a tile, groups that shrink
     (700_000, 64, [20] * 5 + [19] * 130),                    # 5 queries past 2^19: the warp kernel's share
     (700_000, 64, [20] * 5 + [12] * 300 + [3] * 9),          # too few units: all the warp kernel's
     (120_065, 528, [17, 30] * 100),                          # 33 words, more than 512 bytes
-    (235_000, 512, [18] * 48),
+    (235_000, 512, [18] * 64),
     (60_000, 1040, [16, 15] * 256),
 ])
 def test_tensor_scan_matches_the_warp_kernels(orc, N, B, ms):
