@@ -175,7 +175,7 @@ def kernel_source_hash() -> str:
     import re
     h = hashlib.sha256()
     for f in ("fused.cuh", "fused_tc.cu", "launch.cuh", "bounds.cuh", "impir_internal.h", "fused_q1.cu", "fused_q2.cu", "fused_q4.cu", "fused_q8.cu",
-              "fused_q16.cu", "setup.cu"):
+              "fused_q16.cu", "setup.cu", "schedule.h"):
         with open(os.path.join(ROOT, "paper_2509_06514_gb300", "csrc", f)) as fh:
             src = fh.read()
         src = re.sub(r"/\*.*?\*/", " ", src, flags=re.S)

@@ -319,6 +319,17 @@ struct SetupParams {
     unsigned long long keys_bytes;    // size of the key buffer (0: unknown)
 };
 
+// Sets the launch shape's fields of the setup parameters.
+inline void apply_shape(const XorShape& s, int sms, SetupParams* sp) {
+    sp->lane_bits = s.c.lane_bits;
+    sp->qpw = s.c.queries_per_warp;
+    sp->mixed = 1;
+    sp->want_units = s.want_units;
+    sp->group_cap = s.tc ? s.tc_cap : 0;
+    sp->tc_min_queries = tc_min_queries(sp->words);
+    sp->tc_min_units = tc_min_units(sp->words, sms);
+}
+
 struct FusedParams {
     const uint4* db;
     const uint8_t* keys;
@@ -361,9 +372,7 @@ BoundsRecord* bounds_record();
 unsigned long long bounds_db_words(unsigned long long n_words, uint32_t words_per_record);
 // follows: nothing but the fused kernel's launch came before it in the stream (a dependent launch).
 cudaError_t launch_finalize(const FinalizeParams& p, cudaStream_t s, bool follows);
-// The XOR answer's fused launch in the given shape: sets the shape's fields of the setup
-// parameters (before launch_setup) and launches the kernel it names.
-void apply_shape(const XorShape& s, int sms, SetupParams* sp);
+// The XOR answer's fused launch in the given shape.
 cudaError_t launch_xor(const XorShape& s, int sms, cudaStream_t st, FusedParams& fp);
 cudaError_t launch_fused_tc(int sms, cudaStream_t s, const FusedParams& p);
 cudaError_t prepare_fused_tc();

@@ -1,0 +1,103 @@
+"""The work schedule of a batch, built on the host by the code the setup kernel runs: every query gets
+each record of its domain exactly once, whichever kernel takes a tile, for whole databases, row shards
+and the chunks of a streamed database, and no launch reads past its records."""
+import ctypes
+import os
+import random
+import subprocess
+
+import pytest
+
+ROOT = os.path.dirname(os.path.dirname(os.path.abspath(__file__)))
+SHARD_ALIGN = 32768
+
+
+class Result(ctypes.Structure):
+    _fields_ = [("tc_units", ctypes.c_uint64), ("n_units", ctypes.c_uint64), ("lane_bits", ctypes.c_uint32),
+                ("shape_lane_bits", ctypes.c_uint32), ("qpw", ctypes.c_uint32), ("tc_min_active", ctypes.c_uint32),
+                ("tc_shape", ctypes.c_uint32), ("pad", ctypes.c_uint32)]
+
+
+@pytest.fixture(scope="module")
+def sched(tmp_path_factory):
+    so = str(tmp_path_factory.mktemp("schedule") / "schedule.so")
+    subprocess.run(["g++", "-std=c++17", "-O2", "-shared", "-fPIC", "-I", "/usr/local/cuda/include",
+                    os.path.join(ROOT, "tests", "schedule_host.cpp"), "-o", so], check=True)
+    L = ctypes.CDLL(so)
+    L.schedule_what.restype = ctypes.c_char_p
+    L.schedule_check.argtypes = [ctypes.c_uint64, ctypes.c_uint64, ctypes.c_uint32, ctypes.c_void_p, ctypes.c_int,
+                                 ctypes.c_uint64, ctypes.c_uint64, ctypes.c_int, ctypes.c_void_p]
+    L.schedule_tile_bits.argtypes = [ctypes.c_uint64, ctypes.c_uint32, ctypes.c_uint32, ctypes.c_int]
+
+    def check(N, B, counts, sms=152, lo=0, hi=0, n_launch=None, add=0):
+        hist = (ctypes.c_uint32 * 41)()
+        for m, k in counts.items():
+            hist[m] += k
+        r = Result()
+        st = L.schedule_check(N, n_launch or N, (B + 15) // 16, hist, sms, lo, hi, add, ctypes.byref(r))
+        assert st == 0, (L.schedule_what().decode(), N, B, dict(counts), sms, lo, hi)
+        return r
+
+    check.tile_bits = lambda N, B, n, sms=152: L.schedule_tile_bits(N, (B + 15) // 16, n, sms)
+    return check
+
+
+# many queries of domains below one tensor-core tile, a few above: a warp kernel's tile can be smaller
+# than a tensor-core tile, and the line between the two kernels may not fall inside the latter
+@pytest.mark.parametrize("N,B,counts", [
+    (544, 272, {9: 29970, 10: 30}),
+    (600, 512, {9: 30000, 10: 30}),
+    (1000, 512, {9: 30000, 10: 30}),
+    (1100, 512, {8: 30000, 11: 40}),
+    (1500, 512, {9: 30000, 11: 40}),
+    (5000, 4096, {7: 30000, 13: 30}),
+    (1 << 20, 4096, {9: 30000, 20: 95}),
+    (700, 16, {9: 80000, 10: 63}),
+])
+def test_the_line_between_the_kernels(sched, N, B, counts):
+    sched(N, B, counts)
+
+
+def batch(r, N, top):
+    """Domain sizes of a batch: one to four sizes, one of them often far more frequent."""
+    cover = max(1, (N - 1).bit_length())
+    ms = [min(40, max(1, r.choice([cover, cover - r.randint(0, 12), r.randint(1, cover), r.randint(1, 14), 40])))
+          for _ in range(r.randint(1, 4))]
+    return {m: max(1, int(2 ** r.uniform(0, top))) for m in ms}
+
+
+def size(r):
+    B = r.choice([1, 16, 40, 64, 256, 272, 512, 528, 1024, 2048, 4096, 20000])
+    return int(2 ** r.uniform(0, 15)) if r.random() < 0.6 else int(2 ** r.uniform(10, 25)), B
+
+
+@pytest.mark.parametrize("seed", range(4))
+def test_random_databases(sched, seed):
+    r = random.Random(seed)
+    took = 0
+    for _ in range(2000):
+        N, B = size(r)
+        counts = batch(r, N, 17)
+        took += sched(N, B, counts, sms=r.choice([148, 152])).tc_units > 0
+        sched(N, B, counts, add=1)
+    assert took > 50        # the tensor-core kernel is among what was checked
+
+
+@pytest.mark.parametrize("seed", range(2))
+def test_random_shards_and_chunks(sched, seed):
+    r = random.Random(1000 + seed)
+    took = 0
+    for _ in range(700):
+        N, B = size(r)
+        counts = batch(r, N, 12)
+        n = sum(counts.values())
+        cuts = sorted({0, N, *(r.randrange(0, N, SHARD_ALIGN) for _ in range(r.randint(0, 3)))})
+        for lo, hi in zip(cuts, cuts[1:]):
+            took += sched(N, B, counts, lo=lo, hi=hi, n_launch=hi - lo).tc_units > 0
+        # chunks of a streamed database: whole tiles of both kernels
+        T = 32 << sched.tile_bits(N, B, n)
+        chunk = T * r.randint(1, 1 + N // T)
+        for lo in range(0, N, max(chunk, (N // 8 + T - 1) // T * T)):
+            hi = min(N, lo + max(chunk, (N // 8 + T - 1) // T * T))
+            took += sched(N, B, counts, lo=lo, hi=hi).tc_units > 0
+    assert took > 50
