@@ -46,9 +46,6 @@ constexpr uint32_t K = 32u << S;        // records of a tile
 constexpr uint32_t LG = S + 5;          // its levels
 constexpr uint32_t kStages = 2;         // operand tiles in flight
 constexpr uint32_t kStageBytes = 64 * 256;
-// a wait that outlasts this is an error (nanoseconds): units take milliseconds
-constexpr unsigned long long kWaitLimitNs = 20ull * 1000 * 1000 * 1000;
-
 struct UnitDesc {
     unsigned long long tile;
     uint32_t first, count;  // its queries: sorted positions [first, first + count)
@@ -60,6 +57,7 @@ struct Ctl {
     unsigned long long full[2];          // unit's selection bits are there (AES warps -> scan warps)
     unsigned long long empty[kStages];   // operand tile read by its MMAs
     unsigned long long dfull;            // accumulators of a pass complete
+    unsigned long long wait_ns;          // a wait that outlasts this is an error
     UnitDesc unit[2];
     uint32_t done[2];        // finished tasks of the unit
     uint32_t task;           // next AES task
@@ -115,7 +113,7 @@ __device__ __forceinline__ bool mbar_wait(unsigned long long* b, uint32_t parity
         if (nap) __nanosleep(nap);
         if (mbar_try(b, parity)) return true;
         if (*reinterpret_cast<volatile uint32_t*>(&ctl->abort)) return false;
-        if (now_ns() - t0 > kWaitLimitNs) {
+        if (now_ns() - t0 > ctl->wait_ns) {
             *reinterpret_cast<volatile uint32_t*>(&ctl->abort) = 1;
             return false;
         }
@@ -505,6 +503,7 @@ __global__ void __launch_bounds__(kTcThreads, 1) fused_tc_kernel(const __grid_co
         mbar_init(&ctl->dfull, 1);
         ctl->task = 0;
         ctl->abort = 0;
+        ctl->wait_ns = P.wait_ns;
         asm volatile("fence.mbarrier_init.release.cluster;" ::: "memory");
     }
     asm volatile("tcgen05.fence::before_thread_sync;" ::: "memory");

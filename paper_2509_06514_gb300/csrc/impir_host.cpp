@@ -942,6 +942,7 @@ impir_status impir_answer_streamed(const void* records, uint64_t N, uint32_t B, 
         sp.rec_lo = lo;
         sp.rec_hi = lo + cnt;
         sp.keep_acc = c > 0;
+        sp.keep_status = c >= 2;  // each schedule's header is read once, after its last chunk
         sp.bounds = bounds_record();
         sp.keys_bytes = total;
         e = launch_setup(sp, ks[b]);

@@ -315,6 +315,7 @@ struct SetupParams {
     // launch.
     unsigned long long rec_lo, rec_hi;
     uint32_t keep_acc;
+    uint32_t keep_status;             // keeps the header's timed_out too: its earlier launches belong to the call
     BoundsRecord* bounds;             // debug build: where failed checks are recorded
     unsigned long long keys_bytes;    // size of the key buffer (0: unknown)
 };
@@ -343,6 +344,7 @@ struct FusedParams {
     uint32_t words;          // uint4 words per record (stride / 16)
     uint32_t bits_words;     // 32-bit words of selection bits (additive: shares) per (warp, query slot)
     uint32_t with_tc;        // the tensor-core kernel takes part of the batch: nothing may be left here
+    unsigned long long wait_ns;  // limit of the tensor-core kernel's waits
     uint32_t slices_low;     // warps whose slice of those lies below the tables
     unsigned long long rec_lo;  // global index of the record at db[0] (0 unless a chunk or a row shard)
     // extents for the debug build's index checks
@@ -370,6 +372,9 @@ BoundsRecord* bounds_record();
 // uint4 words of a database the index checks allow the kernels to read: n_words, less the
 // records a debug-build test withholds (IMPIR_BOUNDS_TEST_WITHHOLD_RECORDS) to see a check fire.
 unsigned long long bounds_db_words(unsigned long long n_words, uint32_t words_per_record);
+// Nanoseconds after which a wait between the tensor-core kernel's warps gives up: 20 s, where a unit takes
+// milliseconds. A debug-build test shortens it (IMPIR_BOUNDS_TEST_WAIT_NS) to see a wait run out.
+unsigned long long wait_limit_ns();
 // follows: nothing but the fused kernel's launch came before it in the stream (a dependent launch).
 cudaError_t launch_finalize(const FinalizeParams& p, cudaStream_t s, bool follows);
 // The XOR answer's fused launch in the given shape.

@@ -41,7 +41,7 @@ __global__ void __launch_bounds__(1024) setup_kernel(const SetupParams S) {
         s_nbad = 0;
         s_first_bad = 0xffffffffu;
         hdr->bounds_failed = 0;
-        hdr->timed_out = 0;
+        if (!S.keep_status) hdr->timed_out = 0;
 #ifdef IMPIR_BOUNDS
         s_bctx = BoundsCtx{S.bounds, hdr, S.keys, S.keys_bytes, nullptr, 0, 0, 0, 0};
 #endif
@@ -171,6 +171,13 @@ unsigned long long bounds_db_words(unsigned long long n_words, uint32_t words_pe
     return n_words;
 }
 
+unsigned long long wait_limit_ns() {
+#ifdef IMPIR_BOUNDS
+    if (const char* w = std::getenv("IMPIR_BOUNDS_TEST_WAIT_NS")) return std::strtoull(w, nullptr, 10);
+#endif
+    return 20ull * 1000 * 1000 * 1000;
+}
+
 cudaError_t launch_setup(const SetupParams& p, cudaStream_t s) {
     // one CTA, no larger than the queries and accumulator words it has to pass over
     const size_t work = std::max(size_t(p.n_queries), p.keep_acc ? size_t(0) : size_t(p.n_queries) * p.words / 4);
@@ -212,6 +219,7 @@ cudaError_t launch_xor(const XorShape& s, int sms, cudaStream_t st, FusedParams&
                                        dim3(sp.warps * 32), sp.bytes, st, fp);
     if (e != cudaSuccess || !s.tc) return e;
     fp.smem_bytes = tc_smem_bytes();
+    fp.wait_ns = wait_limit_ns();
     return launch_fused_tc(sms, st, fp);
 }
 
