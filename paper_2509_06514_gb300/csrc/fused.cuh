@@ -64,7 +64,7 @@ __device__ __forceinline__ uint8_t* smem_at(uint32_t addr) { return g_smem + (ad
 __device__ __forceinline__ bool fill_tables(const uint32_t* te0, uint32_t tid, uint32_t nthr) {
     const uint32_t base = smem32(g_smem);
 #ifdef IMPIR_BOUNDS
-    if (base < kSmemBase || base > kSmemBase + kSmemStatic) return false;
+    if (base < kSmemBase || base > kSmemBase + kSmemStatic || !te0) return false;
 #else
     if (base != kSmemBase) return false;
 #endif

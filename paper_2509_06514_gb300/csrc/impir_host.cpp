@@ -280,7 +280,7 @@ bool answers_fit(const Db& db, const uint8_t* d_out) {
 // build's index checks use it)
 impir_status launch_batch(const DeviceState& dev, const Db& db, const impir_config& cfg, const uint8_t* d_keys,
                           const uint32_t* d_off, uint32_t n, uint8_t* d_out, uint8_t* d_ws, cudaStream_t st,
-                          int mode = 0, size_t keys_bytes = 0, bool free_shape = false) {
+                          int mode = 0, size_t keys_bytes = 0, bool free_shape = false, bool keep_status = false) {
     const WsLayout lay = ws_layout(n, db.stride);
     // a row shard covers the warp tiles of its rows (shard bounds are whole tiles) of a
     // database of n_total records; its device rows start at global row row_lo
@@ -300,6 +300,7 @@ impir_status launch_batch(const DeviceState& dev, const Db& db, const impir_conf
     sp.mixed = mode == 0;
     sp.rec_lo = shard ? db.row_lo : 0;
     sp.rec_hi = shard ? db.row_lo + db.n : 0;
+    sp.keep_status = keep_status;
     sp.bounds = bounds_record();
     sp.keys_bytes = keys_bytes;
     CK(launch_setup(sp, st), "setup kernel launch");
@@ -310,7 +311,7 @@ impir_status launch_batch(const DeviceState& dev, const Db& db, const impir_conf
     fp.key_off = d_off;
     fp.ws = d_ws;
     fp.acc = sp.acc;
-    fp.te0 = dev.d_te0;
+    fp.te0 = bounds_te0(dev.d_te0);
     fp.lay = lay;
     fp.n_records = db.n_total;
     fp.n_queries = n;
@@ -387,7 +388,7 @@ impir_status answer_async_impl(const Db& db, const impir_config* cfg_in, const u
         if (ws_bytes < ws_layout(1, db.stride).total) return fail(IMPIR_ENOMEM, "workspace too small");
         for (uint32_t q = 0; q < n; ++q)
             if (impir_status s = launch_batch(*dev, db, cfg, d_keys, d_off + q, 1, d_out + size_t(q) * db.bytes,
-                                              static_cast<uint8_t*>(d_ws), st, mode, keys_bytes))
+                                              static_cast<uint8_t*>(d_ws), st, mode, keys_bytes, false, q > 0))
                 return s;
         return IMPIR_OK;
     }
@@ -402,8 +403,8 @@ impir_status answer_async_impl(const Db& db, const impir_config* cfg_in, const u
 struct SyncCtx {
     std::mutex mu;
     cudaStream_t stream = nullptr;
-    void *d_keys = nullptr, *d_ws = nullptr, *d_out = nullptr;  // d_keys: keys, then their offsets
-    size_t c_keys = 0, c_ws = 0, c_out = 0;
+    void *d_keys = nullptr, *d_ws = nullptr;  // keys, then their offsets; workspace, then the answers if not in it
+    size_t c_keys = 0, c_ws = 0;
     uint8_t* h_stage = nullptr;
     size_t c_stage = 0;
 };
@@ -699,12 +700,14 @@ static impir_status answer_sync(int32_t h, const uint8_t* keys, uint32_t n, uint
     const WsLayout lay = ws_layout(cfg.queries_per_launch == 1 ? 1 : n, db.stride);
     const size_t out_bytes = size_t(n) * db.bytes;
     const size_t koff = (total + 15) & ~size_t(15), up = koff + size_t(n) * 4;
-    const size_t hdr_at = (out_bytes + 15) & ~size_t(15);  // the workspace header comes back behind the answers
-    const size_t stage = std::max(up, hdr_at + sizeof(WsHeader));
+    // The workspace's header comes back with the answers, in one copy unless what lies between them
+    // (schedule, and for padded records the accumulators) would cost more than a second one.
+    const size_t ans_at = direct ? lay.off_acc : lay.total;
+    const bool one_copy = ans_at <= (64u << 10);
+    const size_t back_at = one_copy ? ans_at : sizeof(WsHeader);  // the answers' place in the staging buffer
+    const size_t stage = std::max(up, back_at + out_bytes);
     if (impir_status s = grow(&g_sync.d_keys, &g_sync.c_keys, up)) return s;
-    if (impir_status s = grow(&g_sync.d_ws, &g_sync.c_ws, lay.total)) return s;
-    if (!direct)
-        if (impir_status s = grow(&g_sync.d_out, &g_sync.c_out, out_bytes)) return s;
+    if (impir_status s = grow(&g_sync.d_ws, &g_sync.c_ws, ans_at + out_bytes)) return s;
     if (impir_status s = grow(reinterpret_cast<void**>(&g_sync.h_stage), &g_sync.c_stage, stage, true)) return s;
     std::memcpy(g_sync.h_stage, keys, total);
     std::memcpy(g_sync.h_stage + koff, offs.data(), size_t(n) * 4);
@@ -712,18 +715,18 @@ static impir_status answer_sync(int32_t h, const uint8_t* keys, uint32_t n, uint
     uint8_t* d_keys = static_cast<uint8_t*>(g_sync.d_keys);
     CK(cudaMemcpyAsync(d_keys, g_sync.h_stage, up, cudaMemcpyHostToDevice, st), "key upload");
     if (impir_status s = answer_async_impl(db, nullptr, d_keys, reinterpret_cast<const uint32_t*>(d_keys + koff), n,
-                                           static_cast<uint8_t*>(g_sync.d_out), g_sync.d_ws, g_sync.c_ws, st, mode,
+                                           static_cast<uint8_t*>(g_sync.d_ws) + ans_at, g_sync.d_ws, lay.total, st, mode,
                                            direct, total))
         return s;
-    const void* src = direct ? static_cast<const void*>(static_cast<uint8_t*>(g_sync.d_ws) + lay.off_acc) : g_sync.d_out;
-    CK(cudaMemcpyAsync(g_sync.h_stage, src, out_bytes, cudaMemcpyDeviceToHost, st), "answer download");
-    const bool waits = mode == 0 && n >= tc_min_queries(db.stride / 16);  // batches the tensor-core kernel may have taken
-    if (waits)
-        CK(cudaMemcpyAsync(g_sync.h_stage + hdr_at, g_sync.d_ws, sizeof(WsHeader), cudaMemcpyDeviceToHost, st), "status download");
+    const uint8_t* d_ws = static_cast<const uint8_t*>(g_sync.d_ws);
+    CK(cudaMemcpyAsync(g_sync.h_stage, d_ws, one_copy ? ans_at + out_bytes : sizeof(WsHeader), cudaMemcpyDeviceToHost, st),
+       "answer download");
+    if (!one_copy)
+        CK(cudaMemcpyAsync(g_sync.h_stage + back_at, d_ws + ans_at, out_bytes, cudaMemcpyDeviceToHost, st), "answer download");
     CK(cudaStreamSynchronize(st), "answer");
-    if (waits && reinterpret_cast<const WsHeader*>(g_sync.h_stage + hdr_at)->timed_out)
-        return fail(IMPIR_ECUDA, "a wait inside the kernel ran out");
-    std::memcpy(out, g_sync.h_stage, out_bytes);
+    if (reinterpret_cast<const WsHeader*>(g_sync.h_stage)->timed_out)
+        return fail(IMPIR_ECUDA, "a wait inside the kernel ran out, or its tables had no place: the answers are not valid");
+    std::memcpy(out, g_sync.h_stage + back_at, out_bytes);
     return bounds_verdict();
 }
 
@@ -953,7 +956,7 @@ impir_status impir_answer_streamed(const void* records, uint64_t N, uint32_t B, 
         fp.key_off = d_off;
         fp.ws = ws_of[b];
         fp.acc = sp.acc;
-        fp.te0 = dev->d_te0;
+        fp.te0 = bounds_te0(dev->d_te0);
         fp.lay = *lay_of[b];
         fp.n_records = N;
         fp.n_queries = n;

@@ -37,7 +37,7 @@ struct WsHeader {
     uint32_t n_groups;
     uint32_t n_segs;
     uint32_t bounds_failed;       // failed index checks of this launch (debug build only)
-    uint32_t timed_out;           // a wait inside the kernel ran out: the answers are not valid
+    uint32_t timed_out;           // a wait ran out or the tables had no place: the answers are not valid
     // the tensor-core kernel's share of the batch (fused_tc.cu): its segments come first
     unsigned long long tc_counter, tc_units;
     uint32_t tc_segs;
@@ -372,6 +372,9 @@ BoundsRecord* bounds_record();
 // uint4 words of a database the index checks allow the kernels to read: n_words, less the
 // records a debug-build test withholds (IMPIR_BOUNDS_TEST_WITHHOLD_RECORDS) to see a check fire.
 unsigned long long bounds_db_words(unsigned long long n_words, uint32_t words_per_record);
+// The T-table as the kernels get it: a debug-build test (IMPIR_BOUNDS_TEST_NO_TABLES) has them refuse to run,
+// as they do where their shared memory does not begin at the address that the tables' place assumes.
+const uint32_t* bounds_te0(const uint32_t* te0);
 // Nanoseconds after which a wait between the tensor-core kernel's warps gives up: 20 s, where a unit takes
 // milliseconds. A debug-build test shortens it (IMPIR_BOUNDS_TEST_WAIT_NS) to see a wait run out.
 unsigned long long wait_limit_ns();

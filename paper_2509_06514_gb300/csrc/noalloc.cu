@@ -131,7 +131,7 @@ extern "C" impir_status impir_answer_noalloc(const void* d_records, uint64_t n_r
     fp.key_off = d_key_offsets;
     fp.ws = dev->scratch;
     fp.acc = sp.acc;
-    fp.te0 = dev->te0;
+    fp.te0 = bounds_te0(dev->te0);
     fp.lay = lay;
     fp.n_records = n_records;
     fp.n_queries = n_queries;

@@ -171,6 +171,13 @@ unsigned long long bounds_db_words(unsigned long long n_words, uint32_t words_pe
     return n_words;
 }
 
+const uint32_t* bounds_te0(const uint32_t* te0) {
+#ifdef IMPIR_BOUNDS
+    if (std::getenv("IMPIR_BOUNDS_TEST_NO_TABLES")) return nullptr;
+#endif
+    return te0;
+}
+
 unsigned long long wait_limit_ns() {
 #ifdef IMPIR_BOUNDS
     if (const char* w = std::getenv("IMPIR_BOUNDS_TEST_WAIT_NS")) return std::strtoull(w, nullptr, 10);

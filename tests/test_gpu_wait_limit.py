@@ -73,5 +73,38 @@ def run(code):
     assert r.returncode == 0 and "REPORTED" in r.stdout, r.stdout[-3000:] + r.stderr[-3000:]
 
 
+SMALL = r"""
+def no_tables(f):
+    os.environ["IMPIR_BOUNDS_TEST_NO_TABLES"] = "1"
+    try:
+        f()
+    except impir.ImpirError as e:
+        assert e.status == impir.IMPIR_ECUDA and "not valid" in str(e), e
+    else:
+        raise SystemExit("the kernel that did not run was not reported")
+    del os.environ["IMPIR_BOUNDS_TEST_NO_TABLES"]
+
+
+# one query, three, and enough that the header comes back in a copy of its own; padded records too
+for B in (64, 40):
+    d = np.ascontiguousarray(db[: 1 << 18, :B])
+    h = impir.impir_db_load(d, 1 << 18, B)
+    for n in (1, 3, 63, 4000):
+        blob, _ = impir.pack_keys([key] * n)
+        for call in (impir.impir_answer, impir.impir_answer_add32):
+            no_tables(lambda: call(h, blob, n, B))
+            got = call(h, blob, n, B)
+            assert (got == got[0]).all() and got.any()
+    blob, _ = impir.pack_keys([key] * 3)
+    impir.impir_set_config(h, lane_bits=4, queries_per_warp=1, queries_per_launch=1)
+    no_tables(lambda: impir.impir_answer(h, blob, 3, B))
+    impir.impir_db_free(h)
+"""
+
+
+def test_every_synchronous_call_reports_a_kernel_that_did_not_run(bounds_lib):
+    run(SMALL)
+
+
 def test_streamed_answers_report_a_wait_of_any_chunk(bounds_lib):
     run(STREAMED)
