@@ -353,11 +353,16 @@ const char* impir_last_error(void);
  *     it: issue them on one stream, or otherwise order them.
  * d_records: n_records records, record j at d_records + j * stride_bytes (stride a multiple
  * of 16, >= record_bytes, padding bytes zero, 16-byte aligned). Malformed keys give zero
- * answers, as in impir_answer_async (their status is not reported here). */
+ * answers, as in impir_answer_async; impir_noalloc_status reports them. */
 #define IMPIR_NOALLOC_SCRATCH_BYTES (8u << 20)
 impir_status impir_answer_noalloc(const void* d_records, uint64_t n_records, uint32_t record_bytes,
                                   uint32_t stride_bytes, const uint8_t* d_keys, const uint32_t* d_key_offsets,
                                   uint32_t n_queries, uint8_t* d_out, void* cuda_stream);
+
+/* impir_workspace_status for the last impir_answer_noalloc on the current device, read from the
+ * scratch array (synchronizes with the device, allocates nothing): malformed keys, and ECUDA when its
+ * answers are not valid because a wait inside the kernel ran out. EINVAL: no such call was made there. */
+impir_status impir_noalloc_status(uint32_t* n_bad, uint32_t* first_bad);
 
 /* ---- Kernel timing (measurement support; off by default) ----
  * While enabled, each fused EvalAll + dpXOR launch is bracketed by two CUDA events recorded

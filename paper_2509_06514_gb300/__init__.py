@@ -37,7 +37,7 @@ EXPORTS = [
     "impir_aes_calibrate", "impir_db_update", "impir_db_update_async", "impir_db_version", "impir_server_update",
     "impir_answer_streamed", "impir_answer_add32", "impir_answer_add32_async", "impir_tune_cache_save",
     "impir_tune_cache_load", "impir_db_load_rows", "impir_db_rows", "impir_combine_partials",
-    "impir_get_config_add32", "impir_bounds_status", "impir_aes_calibrate_bitsliced",
+    "impir_get_config_add32", "impir_bounds_status", "impir_aes_calibrate_bitsliced", "impir_noalloc_status",
 ]
 
 
@@ -125,6 +125,7 @@ def lib():
                 "impir_server_destroy": (ctypes.c_int, [vp]),
                 "impir_answer_noalloc": (ctypes.c_int, [vp, ctypes.c_uint64, ctypes.c_uint32, ctypes.c_uint32, vp, vp,
                                                         ctypes.c_uint32, vp, vp]),
+                "impir_noalloc_status": (ctypes.c_int, [ctypes.POINTER(ctypes.c_uint32), ctypes.POINTER(ctypes.c_uint32)]),
                 "impir_timing_read": (ctypes.c_int, [ctypes.POINTER(ctypes.c_double), ctypes.POINTER(ctypes.c_uint64),
                                                      ctypes.POINTER(ctypes.c_uint64)]),
                 "impir_db_load_rows": (ctypes.c_int, [vp, ctypes.c_uint64, ctypes.c_uint32, ctypes.c_uint64,
@@ -423,6 +424,12 @@ def impir_answer_noalloc(d_records, n_records: int, record_bytes: int, stride_by
     _check(lib().impir_answer_noalloc(_dev(d_records), n_records, record_bytes, stride_bytes, _dev(d_keys),
                                       _dev(d_key_offsets), n_queries, _dev(d_out), _stream(stream)),
            "impir_answer_noalloc")
+
+
+def impir_noalloc_status() -> tuple[int, int]:
+    nb, fb = ctypes.c_uint32(), ctypes.c_uint32()
+    _check(lib().impir_noalloc_status(ctypes.byref(nb), ctypes.byref(fb)), "impir_noalloc_status")
+    return nb.value, fb.value
 
 
 def impir_aes_calibrate(prf: int, iters: int, seeds: np.ndarray, threads_per_cta: int = 512):

@@ -464,6 +464,19 @@ std::map<std::tuple<int, uint64_t, uint32_t, uint32_t>, impir_config> g_tune;
 
 }  // namespace
 
+namespace impir {
+// The status that the last batch left in the header of its workspace (or of the no-alloc scratch).
+impir_status header_status(const void* d_ws, uint32_t* n_bad, uint32_t* first_bad) {
+    WsHeader h;
+    CK(cudaDeviceSynchronize(), "synchronize");
+    CK(cudaMemcpy(&h, d_ws, sizeof h, cudaMemcpyDeviceToHost), "workspace status copy");
+    if (n_bad) *n_bad = h.n_bad;
+    if (first_bad) *first_bad = h.first_bad;
+    if (h.timed_out) return fail(IMPIR_ECUDA, "a wait inside the kernel ran out: the answers are not valid");
+    return IMPIR_OK;
+}
+}  // namespace impir
+
 extern "C" {
 
 size_t impir_key_bytes(uint32_t m) { return 8 + size_t(64) * (m + 1); }
@@ -671,13 +684,7 @@ impir_status impir_answer_async(int32_t h, const uint8_t* d_keys, const uint32_t
 
 impir_status impir_workspace_status(const void* d_ws, uint32_t* n_bad, uint32_t* first_bad) {
     if (!d_ws) return fail(IMPIR_EINVAL, "NULL workspace");
-    WsHeader h;
-    CK(cudaDeviceSynchronize(), "synchronize");
-    CK(cudaMemcpy(&h, d_ws, sizeof h, cudaMemcpyDeviceToHost), "workspace status copy");
-    if (n_bad) *n_bad = h.n_bad;
-    if (first_bad) *first_bad = h.first_bad;
-    if (h.timed_out) return fail(IMPIR_ECUDA, "a wait inside the kernel ran out: the answers are not valid");
-    return IMPIR_OK;
+    return header_status(d_ws, n_bad, first_bad);
 }
 
 static impir_status answer_sync(int32_t h, const uint8_t* keys, uint32_t n, uint8_t* out, int mode) {

@@ -25,6 +25,7 @@ static __device__ __align__(256) uint8_t g_noalloc_scratch[IMPIR_NOALLOC_SCRATCH
 static __device__ __align__(16) uint32_t g_noalloc_te0[256];
 
 impir_status set_error(impir_status st, const char* msg);
+impir_status header_status(const void* d_ws, uint32_t* n_bad, uint32_t* first_bad);
 
 namespace {
 
@@ -156,4 +157,16 @@ extern "C" impir_status impir_answer_noalloc(const void* d_records, uint64_t n_r
         return set_error(IMPIR_ECUDA, "finalize kernel launch failed");
     }
     return IMPIR_OK;
+}
+
+extern "C" impir_status impir_noalloc_status(uint32_t* n_bad, uint32_t* first_bad) {
+    int dev = -1;
+    if (cudaGetDevice(&dev) != cudaSuccess || dev < 0) return set_error(IMPIR_ECUDA, "no current CUDA device");
+    const uint8_t* scratch = nullptr;
+    if (dev < kMaxDevices) {
+        std::lock_guard<std::mutex> lk(g_mu);
+        if (g_dev[dev].ready) scratch = g_dev[dev].scratch;
+    }
+    if (!scratch) return set_error(IMPIR_EINVAL, "no no-alloc answer was made on this device");
+    return header_status(scratch, n_bad, first_bad);
 }

@@ -102,6 +102,52 @@ for B in (64, 40):
 """
 
 
+ASYNC = r"""
+d_db = torch.from_numpy(db).cuda()
+d_keys = torch.from_numpy(np.frombuffer(blob, np.uint8).copy()).cuda()
+d_off = torch.from_numpy(offs.view(np.int32).copy()).cuda()
+out = torch.zeros((n, B), dtype=torch.uint8, device="cuda")
+
+
+def noalloc():
+    impir.impir_answer_noalloc(d_db, N, B, B, d_keys, d_off, n, out, None)
+    assert impir.impir_noalloc_status() == (0, 0xFFFFFFFF)
+
+
+try:
+    impir.impir_noalloc_status()
+    raise SystemExit("a status without a call")
+except impir.ImpirError as e:
+    assert e.status == impir.IMPIR_EINVAL
+noalloc()
+want = out.clone()
+refused(noalloc)
+noalloc()
+assert torch.equal(out, want)
+
+h = impir.impir_db_attach(d_db, N, B, B)
+wsb = impir.impir_workspace_bytes(n, B)
+ws = torch.empty(wsb, dtype=torch.uint8, device="cuda")
+
+
+def resident():
+    impir.impir_answer_async(h, d_keys, d_off, n, out, ws, wsb, None)
+    impir.impir_workspace_status(ws)
+
+
+refused(resident)
+resident()
+assert torch.equal(out, want)
+refused(lambda: impir.impir_answer(h, blob, n, B))
+assert np.array_equal(impir.impir_answer(h, blob, n, B), want.cpu().numpy())
+impir.impir_db_free(h)
+"""
+
+
+def test_noalloc_and_workspace_status_report_it(bounds_lib):
+    run(ASYNC)
+
+
 def test_every_synchronous_call_reports_a_kernel_that_did_not_run(bounds_lib):
     run(SMALL)
 
