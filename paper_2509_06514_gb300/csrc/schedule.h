@@ -72,19 +72,19 @@ IMPIR_HD uint32_t make_schedule(const SetupParams& S, unsigned long long present
     const auto covered = [&](uint32_t m) { return S.n_records < (1ull << m) ? S.n_records : 1ull << m; };
     if (S.group_cap) {
         unsigned long long prev = 0, units = 0;
-        bool whole = true;  // prev is a place to split at
         ascending([&](uint32_t m) {
             const unsigned long long end = covered(m);
             const uint32_t active = bstart[m] + hist[m];  // queries with domain bits >= m
-            if (active < S.tc_min_queries && whole) return false;
+            if (active < S.tc_min_queries) return false;
             const unsigned long long lo = (prev > S.rec_lo ? prev : S.rec_lo) / tc_tile;
             const unsigned long long hi = ((S.rec_hi && S.rec_hi < end ? S.rec_hi : end) + tc_tile - 1) / tc_tile;
             if (hi > lo) units += (hi - lo) * ((active + S.group_cap - 1) / S.group_cap);
             if (end > prev) prev = end;
-            whole = prev % tmax == 0 || prev == S.n_records;
+            // (a domain that ends inside a tile is no place to split at; if too few queries go on from
+            // there, the line stays at the last one that is)
+            if (units >= S.tc_min_units && (prev % tmax == 0 || prev == S.n_records)) split = prev;
             return true;
         });
-        if (whole && units >= S.tc_min_units) split = prev;
     }
     // segs[nseg ...]: tiles of `tile` records from tile `prev` on (clipped to the records of this
     // launch), for each domain size the tiles it adds; groups(m) of them cover such a tile

@@ -101,3 +101,32 @@ def test_random_shards_and_chunks(sched, seed):
             hi = min(N, lo + max(chunk, (N // 8 + T - 1) // T * T))
             took += sched(N, B, counts, lo=lo, hi=hi).tc_units > 0
     assert took > 50
+
+
+def fewest(B):
+    return 64 if (B + 15) // 16 <= 32 else 96
+
+
+# (queries of a small domain, the large domain, its queries): a domain that ends inside a warp tile is no
+# place to draw the line, but does not hand the tiles behind it to the tensor-core kernel either
+@pytest.mark.parametrize("N,B,counts", [
+    (1 << 24, 512, {10: 64, 24: 8}),
+    (1 << 25, 256, {12: 200, 25: 1}),
+    (1 << 20, 4096, {9: 30000, 20: 95}),
+    (1 << 22, 64, {3: 100, 14: 20, 22: 40}),
+])
+def test_tiles_that_few_queries_reach_stay_with_the_warp_kernels(sched, N, B, counts):
+    assert sched(N, B, counts).tc_units == 0
+
+
+@pytest.mark.parametrize("seed", range(4))
+def test_every_tensor_core_tile_has_enough_queries(sched, seed):
+    r = random.Random(2000 + seed)
+    took = 0
+    for _ in range(2000):
+        N, B = size(r)
+        got = sched(N, B, batch(r, N, 13))
+        if got.tc_units:
+            took += 1
+            assert got.tc_min_active >= fewest(B), (N, B)
+    assert took > 50
