@@ -249,8 +249,12 @@ __device__ __forceinline__ void aes_role(const FusedParams& P, Ctl* ctl, uint32_
         if (q0 < u.count) aes_task(P, b, q0, min(kTaskQ, u.count - q0), u.tile, lane, L);
         __syncwarp();
         if (lane == 0) {
+            // the fences order the words of all the unit's tasks, through the count, before the one arrival
             __threadfence_block();
-            if (atomicAdd(&ctl->done[b], 1u) + 1 == kTcTasks) mbar_arrive(&ctl->full[b]);
+            if (atomicAdd(&ctl->done[b], 1u) + 1 == kTcTasks) {
+                __threadfence_block();
+                mbar_arrive(&ctl->full[b]);
+            }
         }
     }
 }
