@@ -97,7 +97,8 @@ struct Db {
     bool owned = false;
     bool live = false;
     bool cfg_set = false;
-    bool cfg_tuned = false;  // cfg came from the autotuner: the tensor-core kernel may still take a batch
+    bool cfg_tuned = false;  // cfg came from the autotuner, with warps_only
+    bool warps_only = false; // the tuner found the warp kernels alone faster
     impir_config cfg{};
     uint64_t version = 0;  // bumped by every bulk update
     uint64_t row_lo = 0;   // a row shard: global index of its first row
@@ -257,6 +258,22 @@ impir_config default_add_config(uint64_t n_records, uint32_t words, uint32_t n_q
     return best;
 }
 
+// How a batch is launched: the configuration, and whether the library may deviate from it (smaller tiles
+// for uneven domains, and the tensor-core kernel unless warps_only): a shape that the caller set is
+// launched as it is.
+struct BatchShape {
+    impir_config c;
+    bool free_shape;
+    bool warps_only;
+};
+
+BatchShape shape_for(const Db& db, uint32_t n_queries, int sms, int mode) {
+    const bool free_shape = !db.cfg_set || db.cfg_tuned;
+    if (mode == 0) return {config_for(db, n_queries, sms), free_shape, db.warps_only};
+    const uint32_t words = db.stride / 16;
+    return {add_config(db.cfg_set ? db.cfg : default_add_config(db.n, words, n_queries, sms), words), free_shape, true};
+}
+
 size_t smem_add(const impir_config& c) {
     return kTableBytes + kSegSmemBytes + size_t(c.warps_per_cta) * c.queries_per_warp * add_share_words(c) * 4;
 }
@@ -278,13 +295,14 @@ bool answers_fit(const Db& db, const uint8_t* d_out) {
 
 // keys_bytes: size of the key buffer when the library knows it (0: unknown; only the debug
 // build's index checks use it)
-impir_status launch_batch(const DeviceState& dev, const Db& db, const impir_config& cfg, const uint8_t* d_keys,
+impir_status launch_batch(const DeviceState& dev, const Db& db, const BatchShape& bs, const uint8_t* d_keys,
                           const uint32_t* d_off, uint32_t n, uint8_t* d_out, uint8_t* d_ws, cudaStream_t st,
-                          int mode = 0, size_t keys_bytes = 0, bool free_shape = false, bool keep_status = false) {
+                          int mode, size_t keys_bytes, bool keep_status = false) {
+    const impir_config& cfg = bs.c;
     const WsLayout lay = ws_layout(n, db.stride);
     // a row shard covers the warp tiles of its rows (shard bounds are whole tiles) of a
     // database of n_total records; its device rows start at global row row_lo
-    const XorShape shape = xor_shape(cfg, free_shape, db.n, db.stride / 16, n, dev.sms, mode == 1);
+    const XorShape shape = xor_shape(cfg, bs.free_shape, db.n, db.stride / 16, n, dev.sms, bs.warps_only);
     const bool shard = db.row_lo != 0 || db.n_total != db.n;
     SetupParams sp{};
     sp.keys = d_keys;
@@ -363,8 +381,9 @@ impir_status launch_batch(const DeviceState& dev, const Db& db, const impir_conf
 }
 
 // direct_out: no finalize kernel; the answers stay in the workspace's accumulators (one
-// launch for the batch only), where the synchronous path downloads them from
-impir_status answer_async_impl(const Db& db, const impir_config* cfg_in, const uint8_t* d_keys, const uint32_t* d_off,
+// launch for the batch only), where the synchronous path downloads them from.
+// shape: of the batch if the caller has it already, else nullptr
+impir_status answer_async_impl(const Db& db, const BatchShape* shape, const uint8_t* d_keys, const uint32_t* d_off,
                                uint32_t n, uint8_t* d_out, void* d_ws, size_t ws_bytes, cudaStream_t st, int mode = 0,
                                bool direct_out = false, size_t keys_bytes = 0) {
     DeviceState* dev = nullptr;
@@ -373,30 +392,24 @@ impir_status answer_async_impl(const Db& db, const impir_config* cfg_in, const u
     if (!d_keys || !d_off || (!d_out && !direct_out) || !d_ws) return fail(IMPIR_EINVAL, "NULL device buffer");
     if (!bytes_ok(n, db.stride)) return fail(IMPIR_EINVAL, "batch too large: %u answers of %u bytes", n, db.stride);
     if (reinterpret_cast<uintptr_t>(d_ws) & 255) return fail(IMPIR_EINVAL, "workspace must be 256-byte aligned");
-    impir_config cfg = cfg_in                      ? *cfg_in
-                       : (mode == 1 && !db.cfg_set) ? default_add_config(db.n, db.stride / 16, n, dev->sms)
-                                                    : config_for(db, n, dev->sms);
-    if (mode == 1) {
-        if (db.bytes % 4) return fail(IMPIR_EINVAL, "the additive answer needs records of a multiple of 4 bytes");
-        cfg = add_config(cfg, db.stride / 16);
-    }
+    if (mode == 1 && db.bytes % 4) return fail(IMPIR_EINVAL, "the additive answer needs records of a multiple of 4 bytes");
+    const BatchShape bs = shape ? *shape : shape_for(db, n, dev->sms, mode);
+    const impir_config& cfg = bs.c;
     if (impir_status s = check_config(cfg, db.stride / 16, mode)) return s;
-    // a shape that the caller set is launched as it is
-    const bool free_shape = !cfg_in && (!db.cfg_set || db.cfg_tuned);
     if (cfg.queries_per_launch == 1) {
         if (direct_out) return fail(IMPIR_EINVAL, "direct answers need one launch for the batch");
         if (ws_bytes < ws_layout(1, db.stride).total) return fail(IMPIR_ENOMEM, "workspace too small");
         for (uint32_t q = 0; q < n; ++q)
-            if (impir_status s = launch_batch(*dev, db, cfg, d_keys, d_off + q, 1, d_out + size_t(q) * db.bytes,
-                                              static_cast<uint8_t*>(d_ws), st, mode, keys_bytes, false, q > 0))
+            if (impir_status s = launch_batch(*dev, db, bs, d_keys, d_off + q, 1, d_out + size_t(q) * db.bytes,
+                                              static_cast<uint8_t*>(d_ws), st, mode, keys_bytes, q > 0))
                 return s;
         return IMPIR_OK;
     }
     if (ws_bytes < ws_layout(n, db.stride).total)
         return fail(IMPIR_ENOMEM, "workspace of %zu bytes is smaller than the %zu needed", ws_bytes,
                     ws_layout(n, db.stride).total);
-    return launch_batch(*dev, db, cfg, d_keys, d_off, n, direct_out ? nullptr : d_out, static_cast<uint8_t*>(d_ws), st,
-                        mode, keys_bytes, free_shape);
+    return launch_batch(*dev, db, bs, d_keys, d_off, n, direct_out ? nullptr : d_out, static_cast<uint8_t*>(d_ws), st,
+                        mode, keys_bytes);
 }
 
 // ---- synchronous path context: cached device and pinned buffers ----
@@ -458,9 +471,13 @@ impir_status grow(void** p, size_t* cap, size_t need, bool pinned = false) {
     return IMPIR_OK;
 }
 
-// ---- tuning cache: (SMs, N, stride, batch, config hint) -> best configuration ----
+// ---- tuning cache: (SMs, N, stride, batch) -> best configuration ----
+struct Tuned {
+    impir_config c;
+    bool warps_only;  // the warp kernels alone were faster than with the tensor-core kernel
+};
 std::mutex g_tune_mu;
-std::map<std::tuple<int, uint64_t, uint32_t, uint32_t>, impir_config> g_tune;
+std::map<std::tuple<int, uint64_t, uint32_t, uint32_t>, Tuned> g_tune;
 
 }  // namespace
 
@@ -700,11 +717,11 @@ static impir_status answer_sync(int32_t h, const uint8_t* keys, uint32_t n, uint
     if (impir_status s = parse_host_keys(keys, n, offs, total)) return s;
     std::lock_guard<std::mutex> lk(g_sync.mu);
     if (!g_sync.stream) CK(cudaStreamCreateWithFlags(&g_sync.stream, cudaStreamNonBlocking), "stream create");
-    const impir_config cfg = config_for(db, n, dev->sms);
+    const BatchShape shape = shape_for(db, n, dev->sms, mode);
     // records without padding and one launch for the batch: the answers are downloaded straight
     // from the accumulators (no finalize kernel); keys and their offsets go up in one copy
-    const bool direct = cfg.queries_per_launch == 0 && db.stride == db.bytes;
-    const WsLayout lay = ws_layout(cfg.queries_per_launch == 1 ? 1 : n, db.stride);
+    const bool direct = shape.c.queries_per_launch == 0 && db.stride == db.bytes;
+    const WsLayout lay = ws_layout(shape.c.queries_per_launch == 1 ? 1 : n, db.stride);
     const size_t out_bytes = size_t(n) * db.bytes;
     const size_t koff = (total + 15) & ~size_t(15), up = koff + size_t(n) * 4;
     // The workspace's header comes back with the answers, in one copy unless what lies between them
@@ -721,7 +738,7 @@ static impir_status answer_sync(int32_t h, const uint8_t* keys, uint32_t n, uint
     cudaStream_t st = g_sync.stream;
     uint8_t* d_keys = static_cast<uint8_t*>(g_sync.d_keys);
     CK(cudaMemcpyAsync(d_keys, g_sync.h_stage, up, cudaMemcpyHostToDevice, st), "key upload");
-    if (impir_status s = answer_async_impl(db, nullptr, d_keys, reinterpret_cast<const uint32_t*>(d_keys + koff), n,
+    if (impir_status s = answer_async_impl(db, &shape, d_keys, reinterpret_cast<const uint32_t*>(d_keys + koff), n,
                                            static_cast<uint8_t*>(g_sync.d_ws) + ans_at, g_sync.d_ws, lay.total, st, mode,
                                            direct, total))
         return s;
@@ -768,12 +785,11 @@ impir_status impir_get_config_add32(int32_t h, uint32_t n_queries, impir_config*
     if (impir_status s = get_db(h, &db)) return s;
     DeviceState* dev = nullptr;
     if (impir_status s = need_device(&dev)) return s;
-    const uint32_t n = n_queries ? n_queries : 1;
-    *cfg = add_config(db.cfg_set ? db.cfg : default_add_config(db.n, db.stride / 16, n, dev->sms), db.stride / 16);
+    *cfg = shape_for(db, n_queries ? n_queries : 1, dev->sms, 1).c;
     return IMPIR_OK;
 }
 
-static impir_status set_config(int32_t h, const impir_config* cfg, bool tuned) {
+static impir_status set_config(int32_t h, const impir_config* cfg, bool tuned, bool warps_only = false) {
     if (!cfg) return fail(IMPIR_EINVAL, "NULL argument");
     std::lock_guard<std::mutex> lk(g_db_mu);
     if (h < 1 || size_t(h) > g_dbs.size() || !g_dbs[h - 1].live) return fail(IMPIR_EINVAL, "unknown database handle %d", h);
@@ -781,6 +797,7 @@ static impir_status set_config(int32_t h, const impir_config* cfg, bool tuned) {
     g_dbs[h - 1].cfg = *cfg;
     g_dbs[h - 1].cfg_set = true;
     g_dbs[h - 1].cfg_tuned = tuned;
+    g_dbs[h - 1].warps_only = warps_only;
     return IMPIR_OK;
 }
 
@@ -798,8 +815,8 @@ impir_status impir_autotune(int32_t h, const uint8_t* d_keys, const uint32_t* d_
         std::lock_guard<std::mutex> lk(g_tune_mu);
         auto it = g_tune.find(key);
         if (it != g_tune.end()) {
-            if (best) *best = it->second;
-            return set_config(h, &it->second, true);
+            if (best) *best = it->second.c;
+            return set_config(h, &it->second.c, true, it->second.warps_only);
         }
     }
     const impir_config base = default_config(db.n, db.stride / 16, n, dev->sms);
@@ -822,29 +839,47 @@ impir_status impir_autotune(int32_t h, const uint8_t* d_keys, const uint32_t* d_
     cudaEvent_t e0, e1;
     CK(cudaEventCreate(&e0), "event");
     CK(cudaEventCreate(&e1), "event");
-    float best_ms = 1e30f;
-    impir_config best_c = base;
-    for (const impir_config& c : cands) {
-        if (impir_status s = answer_async_impl(db, &c, d_keys, d_off, n, d_out, d_ws, ws_bytes, st)) return s;
-        CK(cudaEventRecord(e0, st), "event record");
-        if (impir_status s = answer_async_impl(db, &c, d_keys, d_off, n, d_out, d_ws, ws_bytes, st)) return s;
+    // device time of the batch launched as a tuned shape is, with or without the tensor-core kernel
+    const auto time_ms = [&](const impir_config& c, bool warps_only, float* ms) {
+        const BatchShape shape{c, true, warps_only};
+        for (int i = 0; i < 2; ++i) {
+            if (i == 1) CK(cudaEventRecord(e0, st), "event record");
+            if (impir_status s = answer_async_impl(db, &shape, d_keys, d_off, n, d_out, d_ws, ws_bytes, st)) return s;
+        }
         CK(cudaEventRecord(e1, st), "event record");
         CK(cudaEventSynchronize(e1), "event sync");
-        float ms = 0;
-        CK(cudaEventElapsedTime(&ms, e0, e1), "event time");
+        CK(cudaEventElapsedTime(ms, e0, e1), "event time");
+        return IMPIR_OK;
+    };
+    float best_ms = 1e30f, ms = 0;
+    Tuned found{base, false};
+    for (const impir_config& c : cands) {
+        if (impir_status s = time_ms(c, true, &ms)) return s;
         if (ms < best_ms) {
             best_ms = ms;
-            best_c = c;
+            found.c = c;
+        }
+    }
+    // Where the tensor-core kernel may take tiles of the batch it stays only if that is faster than the
+    // fastest warp shape; the shape beside it (the tiles that few queries reach) is that one or the default.
+    if (xor_shape(found.c, true, db.n, db.stride / 16, n, dev->sms).tc) {
+        found.warps_only = true;
+        for (const impir_config& c : {found.c, base}) {
+            if (impir_status s = time_ms(c, false, &ms)) return s;
+            if (ms < best_ms) {
+                best_ms = ms;
+                found = {c, false};
+            }
         }
     }
     cudaEventDestroy(e0);
     cudaEventDestroy(e1);
     {
         std::lock_guard<std::mutex> lk(g_tune_mu);
-        g_tune[key] = best_c;
+        g_tune[key] = found;
     }
-    if (best) *best = best_c;
-    return set_config(h, &best_c, true);
+    if (best) *best = found.c;
+    return set_config(h, &found.c, true, found.warps_only);
 }
 
 // ---- databases larger than HBM: streamed in chunks (§3.3) ----
@@ -1017,14 +1052,14 @@ impir_status impir_tune_cache_save(const char* path) {
     FILE* f = std::fopen(path, "w");
     if (!f) return fail(IMPIR_EINVAL, "cannot write %s", path);
     std::fprintf(f, "# impir tuning cache: sms n_records stride_bytes n_queries lane_bits queries_per_warp "
-                    "warps_per_cta queries_per_launch\n");
+                    "warps_per_cta queries_per_launch [1: no tensor-core kernel]\n");
     {
         std::lock_guard<std::mutex> lk(g_tune_mu);
         for (const auto& kv : g_tune)
-            std::fprintf(f, "%d %llu %u %u %u %u %u %u\n", std::get<0>(kv.first),
+            std::fprintf(f, "%d %llu %u %u %u %u %u %u%s\n", std::get<0>(kv.first),
                          (unsigned long long)std::get<1>(kv.first), std::get<2>(kv.first), std::get<3>(kv.first),
-                         kv.second.lane_bits, kv.second.queries_per_warp, kv.second.warps_per_cta,
-                         kv.second.queries_per_launch);
+                         kv.second.c.lane_bits, kv.second.c.queries_per_warp, kv.second.c.warps_per_cta,
+                         kv.second.c.queries_per_launch, kv.second.warps_only ? " 1" : "");
     }
     std::fclose(f);
     return IMPIR_OK;
@@ -1040,14 +1075,14 @@ impir_status impir_tune_cache_load(const char* path, uint32_t* n_loaded) {
         if (line[0] == '#') continue;
         int sms;
         unsigned long long nrec;
-        unsigned stride, nq;
+        unsigned stride, nq, warps_only = 0;
         impir_config c{};
-        if (std::sscanf(line, "%d %llu %u %u %u %u %u %u", &sms, &nrec, &stride, &nq, &c.lane_bits,
-                        &c.queries_per_warp, &c.warps_per_cta, &c.queries_per_launch) != 8)
+        if (std::sscanf(line, "%d %llu %u %u %u %u %u %u %u", &sms, &nrec, &stride, &nq, &c.lane_bits,
+                        &c.queries_per_warp, &c.warps_per_cta, &c.queries_per_launch, &warps_only) < 8)
             continue;
         if (check_config(c, stride / 16) != IMPIR_OK) continue;  // skip entries this build cannot launch
         std::lock_guard<std::mutex> lk(g_tune_mu);
-        g_tune[std::make_tuple(sms, uint64_t(nrec), uint32_t(stride), uint32_t(nq))] = c;
+        g_tune[std::make_tuple(sms, uint64_t(nrec), uint32_t(stride), uint32_t(nq))] = Tuned{c, warps_only != 0};
         ++n;
     }
     std::fclose(f);

@@ -276,16 +276,17 @@ struct XorShape {
     uint32_t tile_bits() const { return tc ? std::max(kTcLaneBits, c.lane_bits) : c.lane_bits; }
 };
 
-// free_shape: the caller set no launch shape of its own; add: the additive answer (warp kernels only).
+// free_shape: the caller set no launch shape of its own; warps_only: the additive answer, or a tuned shape
+// that was faster without the tensor-core kernel.
 inline XorShape xor_shape(const impir_config& c, bool free_shape, uint64_t n_records, uint32_t words,
-                          uint32_t n_queries, int sms, bool add = false) {
+                          uint32_t n_queries, int sms, bool warps_only = false) {
     XorShape s{c, false, 0, 0};
     // as many units as a batch that covers the database has, but 40 per SM are enough
     const uint64_t T = 32ull << c.lane_bits;
     if (free_shape)
         s.want_units = std::min<uint64_t>(40ull * sms, ((n_records + T - 1) / T) *
                                                            ((n_queries + c.queries_per_warp - 1) / c.queries_per_warp));
-    if (!free_shape || add || c.queries_per_launch != 0 || n_queries < tc_min_queries(words)) return s;
+    if (!free_shape || warps_only || c.queries_per_launch != 0 || n_queries < tc_min_queries(words)) return s;
     const uint64_t groups = (n_queries + kTcQueries - 1) / kTcQueries;
     if (groups * ((n_records + (32u << kTcLaneBits) - 1) >> (kTcLaneBits + 5)) < tc_min_units(words, sms)) return s;
     s.tc = true;
