@@ -254,17 +254,24 @@ constexpr uint32_t kTcLaneBits = 5;    // tiles of 32 << 5 = 1024 records
 
 // Fewest queries that must reach a tile for the tensor-core kernel to take it. Its scan costs the
 // same for 1 query as for 128, the warp kernels' grows with every query: measured on 2^22 records,
-// time of the fastest warp shape over the tensor-core kernel's at 48 / 64 / 96 / 128 queries: 0.95 /
-// 0.99 / 1.02 / 1.01 for 64-byte records, 0.94 / 1.01 / 1.05 / 1.06 for 256 bytes, 0.95 / 1.03 / 1.09 /
-// 1.12 for 512 bytes; for 1 KiB 0.87 / 0.98 / 1.18 / 1.22 (4 KiB on 2^20: 1.06 at 96).
+// time of the default warp shape over the tensor-core kernel's at 64 / 80 / 96 / 128 queries: 1.00 /
+// 1.01 / 1.03 / 1.02 for 64-byte records, 1.02 / 1.04 / 1.06 / 1.06 for 256 bytes, 1.04 / 1.08 / 1.10 /
+// 1.13 for 512 bytes; for 1 KiB 1.21 / 1.28 at 96 / 128 (4 KiB on 2^20: 1.17 / 1.42). At 48 queries it
+// was 0.94 to 0.95 up to 512 bytes, at 64 of 1 KiB 0.98.
 inline uint32_t tc_min_queries(uint32_t words) { return words <= 32 ? 64u : 96u; }
 
-// Fewest units for the tensor-core kernel to take any: units of 1024 records go to SMs whole, and with
-// fewer than four per SM the last round costs more than the scan gains for records up to 256 bytes
-// (0.92 to 0.97 at 2^18 records and 64 or 128 queries); wider ones gain from one and a half on.
-inline uint64_t tc_min_units(uint32_t words, int sms) { return uint64_t(sms) * (words <= 16 ? 8 : 3) / 2; }
+// Fewest units, of at most `rows` queries, for the tensor-core kernel to take any: units of 1024 records
+// go to SMs whole, and with fewer than four per SM the last round costs more than the scan gains for
+// records up to 256 bytes (0.92 to 0.97 at 2^18 records and 64 or 128 queries). Wider ones are taken from
+// one and a half on: full units gain (4 KiB on 2^18, 128 queries 1.13; 512 bytes on 2^18, 96 queries 1.04),
+// units of 64 or 80 rows lose to the default warp shape (512 bytes on 2^19 0.90 and 0.94) though not to
+// the shapes that ran before there was a choice. Above 3 KiB they did lose to those with fewer than 104
+// rows (4 KiB on 2^19, 96 queries 6240 us against 6115): four per SM there too.
+inline uint64_t tc_min_units(uint32_t words, uint32_t rows, int sms) {
+    return uint64_t(sms) * (words <= 16 || (words > 192 && rows < 104) ? 8 : 3) / 2;
+}
 
-// How a batch is launched: the warp kernels of fused.cuh in the shape `c`, with tc after the
+// How a batch is launched: the warp kernels of fused.cuh in the shape `c`, and with tc, behind them, the
 // tensor-core kernel, which takes the tiles that enough queries reach (the setup kernel draws the
 // line: the keys' domains are on the device) in groups of at most tc_cap queries.
 struct XorShape {
@@ -288,9 +295,10 @@ inline XorShape xor_shape(const impir_config& c, bool free_shape, uint64_t n_rec
                                                            ((n_queries + c.queries_per_warp - 1) / c.queries_per_warp));
     if (!free_shape || warps_only || c.queries_per_launch != 0 || n_queries < tc_min_queries(words)) return s;
     const uint64_t groups = (n_queries + kTcQueries - 1) / kTcQueries;
-    if (groups * ((n_records + (32u << kTcLaneBits) - 1) >> (kTcLaneBits + 5)) < tc_min_units(words, sms)) return s;
+    const uint32_t rows = uint32_t((n_queries + groups - 1) / groups);
+    if (groups * ((n_records + (32u << kTcLaneBits) - 1) >> (kTcLaneBits + 5)) < tc_min_units(words, rows, sms)) return s;
     s.tc = true;
-    s.tc_cap = uint32_t((n_queries + groups - 1) / groups);
+    s.tc_cap = rows;
     return s;
 }
 
@@ -329,7 +337,7 @@ inline void apply_shape(const XorShape& s, int sms, SetupParams* sp) {
     sp->want_units = s.want_units;
     sp->group_cap = s.tc ? s.tc_cap : 0;
     sp->tc_min_queries = tc_min_queries(sp->words);
-    sp->tc_min_units = tc_min_units(sp->words, sms);
+    sp->tc_min_units = tc_min_units(sp->words, s.tc_cap, sms);
 }
 
 struct FusedParams {

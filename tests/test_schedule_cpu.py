@@ -130,3 +130,12 @@ def test_every_tensor_core_tile_has_enough_queries(sched, seed):
             took += 1
             assert got.tc_min_active >= fewest(B), (N, B)
     assert took > 50
+
+
+def test_narrow_groups_of_the_widest_records_need_more_units(sched):
+    """96 queries on 2^19 records of 4 KiB (512 units) are faster in the warp kernels, 104 are not, and
+    1024 units gain with either."""
+    assert sched(1 << 19, 4096, {19: 96}).tc_units == 0
+    assert sched(1 << 19, 4096, {19: 104}).tc_units == 512
+    assert sched(1 << 20, 4096, {20: 96}).tc_units == 1024
+    assert sched(1 << 18, 4096, {18: 128}).tc_units == 256
