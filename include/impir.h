@@ -174,7 +174,9 @@ size_t impir_workspace_bytes(uint32_t n_queries, uint32_t stride_bytes);
  * extent of d_keys (the call has no length for it): the caller guarantees that every offset
  * starts a whole key, impir_key_bytes(m) bytes for the m in its header, inside d_keys.
  * Launch errors return ECUDA. Where records carry no padding and d_out is 16-byte aligned memory of
- * the current device, the answers are accumulated in d_out itself while the call's kernels run. */
+ * the current device that lies over none of the call's inputs, the answers are accumulated in d_out
+ * itself while the call's kernels run; else they are written when all inputs have been read, so d_out may
+ * lie over the keys, their offsets or the records. */
 impir_status impir_answer_async(int32_t db_handle, const uint8_t* d_keys, const uint32_t* d_key_offsets,
                                 uint32_t n_queries, uint8_t* d_out, void* d_workspace, size_t workspace_bytes,
                                 void* cuda_stream);

@@ -281,9 +281,24 @@ size_t smem_add(const impir_config& c) {
 // Whether a batch's answers can be accumulated where the caller wants them, with no workspace in
 // between and no finalize kernel (2.5 us of a 22 us batch of one query on 2^15 records): records without
 // padding and 16-byte aligned answers in this device's own memory (atomics on host memory that is
-// mapped into the device's space are another matter).
-bool answers_fit(const Db& db, const uint8_t* d_out) {
+// mapped into the device's space are another matter). Answers that a caller lays over the batch's own
+// inputs are written when those have been read, so not before the finalize kernel. The keys lie back to
+// back; where their buffer's size is not known (keys_bytes 0) they end before the next input, and within
+// the longest keys there are.
+bool answers_fit(const Db& db, const uint8_t* d_out, uint32_t n, const uint8_t* d_keys, size_t keys_bytes,
+                 const uint32_t* d_off, const void* d_ws, size_t ws_bytes) {
     if (db.stride != db.bytes || (reinterpret_cast<uintptr_t>(d_out) & 15)) return false;
+    const auto at = [](const void* p) { return reinterpret_cast<uintptr_t>(p); };
+    const uintptr_t out = at(d_out), end = out + size_t(n) * db.bytes, keys = at(d_keys);
+    const struct {
+        uintptr_t lo, bytes;
+    } in[] = {{at(db.d), size_t(db.n) * db.stride}, {at(d_off), size_t(n) * 4}, {at(d_ws), ws_bytes}};
+    uintptr_t keys_end = keys + (keys_bytes ? keys_bytes : size_t(n) * impir_key_bytes(IMPIR_MAX_DOMAIN_BITS));
+    for (const auto& i : in) {
+        if (out < i.lo + i.bytes && i.lo < end) return false;
+        if (i.lo >= keys) keys_end = std::min(keys_end, i.lo);
+    }
+    if (out < keys_end && keys < end) return false;
     cudaPointerAttributes a{};
     if (cudaPointerGetAttributes(&a, d_out) != cudaSuccess) {
         cudaGetLastError();
@@ -295,9 +310,10 @@ bool answers_fit(const Db& db, const uint8_t* d_out) {
 
 // keys_bytes: size of the key buffer when the library knows it (0: unknown; only the debug
 // build's index checks use it)
+// into_out: the answers are accumulated in d_out (answers_fit)
 impir_status launch_batch(const DeviceState& dev, const Db& db, const BatchShape& bs, const uint8_t* d_keys,
-                          const uint32_t* d_off, uint32_t n, uint8_t* d_out, uint8_t* d_ws, cudaStream_t st,
-                          int mode, size_t keys_bytes, bool keep_status = false) {
+                          const uint32_t* d_off, uint32_t n, uint8_t* d_out, bool into_out, uint8_t* d_ws,
+                          cudaStream_t st, int mode, size_t keys_bytes, bool keep_status = false) {
     const impir_config& cfg = bs.c;
     const WsLayout lay = ws_layout(n, db.stride);
     // a row shard covers the warp tiles of its rows (shard bounds are whole tiles) of a
@@ -308,7 +324,6 @@ impir_status launch_batch(const DeviceState& dev, const Db& db, const BatchShape
     sp.keys = d_keys;
     sp.key_off = d_off;
     sp.ws = d_ws;
-    const bool into_out = d_out && answers_fit(db, d_out);
     sp.acc = reinterpret_cast<uint4*>(into_out ? d_out : d_ws + lay.off_acc);
     sp.lay = lay;
     sp.n_records = db.n_total;
@@ -396,11 +411,14 @@ impir_status answer_async_impl(const Db& db, const BatchShape* shape, const uint
     const BatchShape bs = shape ? *shape : shape_for(db, n, dev->sms, mode);
     const impir_config& cfg = bs.c;
     if (impir_status s = check_config(cfg, db.stride / 16, mode)) return s;
-    if (cfg.queries_per_launch == 1) {
+    const bool one_each = cfg.queries_per_launch == 1;
+    const bool into_out = !direct_out && answers_fit(db, d_out, n, d_keys, keys_bytes, d_off, d_ws,
+                                                     ws_layout(one_each ? 1 : n, db.stride).total);
+    if (one_each) {
         if (direct_out) return fail(IMPIR_EINVAL, "direct answers need one launch for the batch");
         if (ws_bytes < ws_layout(1, db.stride).total) return fail(IMPIR_ENOMEM, "workspace too small");
         for (uint32_t q = 0; q < n; ++q)
-            if (impir_status s = launch_batch(*dev, db, bs, d_keys, d_off + q, 1, d_out + size_t(q) * db.bytes,
+            if (impir_status s = launch_batch(*dev, db, bs, d_keys, d_off + q, 1, d_out + size_t(q) * db.bytes, into_out,
                                               static_cast<uint8_t*>(d_ws), st, mode, keys_bytes, q > 0))
                 return s;
         return IMPIR_OK;
@@ -408,8 +426,8 @@ impir_status answer_async_impl(const Db& db, const BatchShape* shape, const uint
     if (ws_bytes < ws_layout(n, db.stride).total)
         return fail(IMPIR_ENOMEM, "workspace of %zu bytes is smaller than the %zu needed", ws_bytes,
                     ws_layout(n, db.stride).total);
-    return launch_batch(*dev, db, bs, d_keys, d_off, n, direct_out ? nullptr : d_out, static_cast<uint8_t*>(d_ws), st,
-                        mode, keys_bytes);
+    return launch_batch(*dev, db, bs, d_keys, d_off, n, direct_out ? nullptr : d_out, into_out,
+                        static_cast<uint8_t*>(d_ws), st, mode, keys_bytes);
 }
 
 // ---- synchronous path context: cached device and pinned buffers ----
