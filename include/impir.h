@@ -210,7 +210,9 @@ typedef struct {
 
 /* Gets the configuration a batch of n_queries keys would be launched with on this database
  * (the one set or tuned for it, else the built-in default for that batch size), or sets one
- * for all later batches (set validates it: EINVAL). A shape that was set is launched as it is.
+ * for all later batches (set validates it: EINVAL). A shape that was set is launched as it is, but
+ * for two whose warps' shared memory does not all find room beside the AES tables: 12 warps of
+ * queries_per_warp << lane_bits = 2048 run as 11, 6 of 4096 as 5 (the answers are the same).
  * Otherwise tiles that 64 or more queries reach (96 for records above 512 bytes) go to the
  * tensor-core kernel, which has one shape, and the configuration describes the launch for the
  * others; its lane_bits is then an upper limit (queries whose domains end early get smaller tiles). */

@@ -143,3 +143,9 @@ extern "C" int schedule_check(uint64_t n_records, uint64_t n_launch, uint32_t wo
     }
     return 0;
 }
+
+// Warps that a launch in this shape has.
+extern "C" uint32_t launched_warps(uint32_t lane_bits, uint32_t qpw, uint32_t warps) {
+    const impir_config c{lane_bits, qpw, warps, 0};
+    return split_smem(warps, size_t(qpw) * bits_words(c) * 4).warps;
+}

@@ -38,6 +38,7 @@ def sched(tmp_path_factory):
         assert st == 0, (L.schedule_what().decode(), N, B, dict(counts), sms, lo, hi)
         return r
 
+    check.lib = L
     check.tile_bits = lambda N, B, n, sms=152: L.schedule_tile_bits(N, (B + 15) // 16, n, sms)
     return check
 
@@ -139,3 +140,26 @@ def test_narrow_groups_of_the_widest_records_need_more_units(sched):
     assert sched(1 << 19, 4096, {19: 104}).tc_units == 512
     assert sched(1 << 20, 4096, {20: 96}).tc_units == 1024
     assert sched(1 << 18, 4096, {18: 128}).tc_units == 256
+
+
+@pytest.mark.parametrize("B", [16, 512, 528, 4096])
+def test_shapes_that_are_launched_with_fewer_warps(sched, B):
+    """Of all shapes that impir_set_config takes, the two that include/impir.h names."""
+    import paper_2509_06514_gb300 as impir
+    from paper_2509_06514_gb300 import build
+    build.build()
+    h = impir.impir_db_attach(1 << 20, 1 << 20, B, B)      # an address that is never read
+    fewer, taken = set(), 0
+    for lane_bits in range(11):
+        for qpw in (1, 2, 4, 8, 16):
+            for warps in range(4, 21):
+                try:
+                    impir.impir_set_config(h, lane_bits, qpw, warps)
+                except impir.ImpirError:
+                    continue
+                taken += 1
+                got = sched.lib.launched_warps(lane_bits, qpw, warps)
+                if got != warps:
+                    fewer.add((qpw << lane_bits, warps, got))
+    impir.impir_db_free(h)
+    assert taken > 400 and fewer == {(2048, 12, 11), (4096, 6, 5)}
