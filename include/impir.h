@@ -270,7 +270,7 @@ impir_status impir_tune_cache_load(const char* path, uint32_t* n_loaded);
  * within accumulator_budget (a batch of n queries on a database of stride S holds n*S bytes),
  * taking further pending requests for the same database in arrival order; it launches the
  * fused answer on that stream, so batches that arrive while others run overlap on the device.
- * Each result is the same as answering that key alone. No kernel waits on anything; the
+ * Each result is the same as answering that key alone. No kernel waits on another; the
  * dispatcher polls batch completion events on the host. */
 typedef struct impir_server impir_server;
 typedef struct {

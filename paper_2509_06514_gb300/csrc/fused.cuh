@@ -762,7 +762,7 @@ __device__ __forceinline__ void add_walk_chunk_inline(const uint8_t* kq, uint32_
     const uint32_t npairs = 1u << (sq - 1), end = p + ch / 2;
     for (;;) {
         // node and leaf pairs each by their own copy of the rounds: with one copy for both (as in
-        // lane_eval) this walk, whose state fills the registers, measured 11 % slower
+        // subtree_bits) this walk, whose state fills the registers, measured 11 % slower
         const uint32_t t = node.x & 1u;
         Blk a, b;
         if (depth == m - 1) {

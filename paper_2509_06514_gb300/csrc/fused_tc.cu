@@ -16,10 +16,10 @@
 //     accumulators were compared with integer counts up to 2^16 on this GPU). Its parity
 //     is the answer bit: adding 2^23 (scaled) puts the count's lowest bit at a fixed mantissa bit.
 //
-// Structure of a CTA (persistent, one per SM), 16 AES warps and 4 scan warps:
+// Structure of a CTA (persistent, one per SM), 20 AES warps and 4 scan warps:
 //   * unit = (tile of K = 32 << S records, group of at most 128 queries of the sorted batch);
 //     units come from the launch's global counter. Domain sizes mix freely inside a group. Tiles that
-//     few queries reach are left to the warp kernel, which is launched next (see setup.cu).
+//     few queries reach are left to the warp kernel, which is launched before (schedule.h, launch_xor).
 //   * scan warps, thread n for query n: walk the root -> the tile's node and expand 3 levels
 //     below it (8 nodes per query), for the unit after next; all lanes are busy, where a warp of
 //     fused.cuh walks for its 8 queries with 8 lanes.

@@ -176,16 +176,24 @@ inline SmemSplit split_smem(uint32_t warps, size_t slice) {
     return s;
 }
 
-// Estimated time of a batch in the shape c, in SM clocks. A unit (a warp tile for a group of queries)
-// costs a warp the walk to the tile, four cooperative levels, the lanes' subtrees and the scan's share
-// of the ALU pipe, counted in node pairs. A pair takes a warp 2000 clocks by itself (a single child
-// 1750), and an SM's warps together 330 each (the lookups' shared-memory port); a round of record
-// loads 900. Where every unit finds a warp at once, the block's warps share the walk and the
-// cooperative levels if it has more than four units (fused.cuh); else the port is busy throughout, and
-// the last units add their latency.
-// The scan's reads: every group reads the tiles it covers, the first from HBM, the others from L2 if
-// the tiles in work at a time fit there.
-// The additive answer (add): every lane walks the last five levels by itself, for each query.
+// Estimated time of a batch in the shape c, in SM clocks: which shape is best, not how long it takes.
+// The form follows the kernel; the constants, in clocks unless said, are measured where a figure is named
+// here and were else adjusted by hand until the order of timed shapes came out:
+//   pair      2000 alone (a chain of ten rounds of dependent lookups; a single child 1750), 330 of the
+//             lookups' shared-memory port each when an SM's warps share it (329 lookups), and a warp waits
+//             for the port behind the others, at least 700 more than that; in the steady state 320, 40 %
+//             more by a lone warp (1 + 0.4 / w), and 2000 for the last units. 1.04 - 0.005 s: the walk's
+//             loop per subtree; slow: 1 % per query slot (registers)
+//   walk      top levels, 200 for 32 of them that share the port; four cooperative levels of 2500, 330 of
+//             the port for 32 nodes (1.3 pairs' time each in the steady state); the fifth level 0.8 pairs
+//             per query and lane. The additive answer's lanes walk all five (0.65 each for the four more)
+//   scan      per 16-byte word 4.3 operations for each query and 4 (additive: 14, with its share loads) for
+//             all of them, in pairs of 560 ALU operations (282 per block); 900 for a round of record loads
+//   memory    3300 bytes a clock from HBM (6.8 TB/s), of which n warps per SM draw 400 n, twice that where
+//             the reads of one unit pass under another's lookups; 5000 from L2, where groups read a tile
+//             again; L2 holds the tiles in work up to 64 MB, none of them from 256 MB
+// Where every unit finds a warp at once, the block's warps share the walk and the cooperative levels if
+// it has more than four units (fused.cuh); else the port is busy throughout.
 inline double shape_clocks(const impir_config& c, uint64_t n_records, uint32_t words, uint32_t n_queries, int sms,
                            bool add = false) {
     const double slots = c.queries_per_warp, s = c.lane_bits, w = c.warps_per_cta;
