@@ -97,8 +97,8 @@ struct Db {
     bool owned = false;
     bool live = false;
     bool cfg_set = false;
-    bool cfg_tuned = false;  // cfg came from the autotuner, with warps_only
-    bool warps_only = false; // the tuner found the warp kernels alone faster
+    bool cfg_tuned = false;  // cfg came from the autotuner
+    uint32_t warps_only_n = 0;  // batch size for which it found the warp kernels alone faster (0: none)
     impir_config cfg{};
     uint64_t version = 0;  // bumped by every bulk update
     uint64_t row_lo = 0;   // a row shard: global index of its first row
@@ -269,7 +269,7 @@ struct BatchShape {
 
 BatchShape shape_for(const Db& db, uint32_t n_queries, int sms, int mode) {
     const bool free_shape = !db.cfg_set || db.cfg_tuned;
-    if (mode == 0) return {config_for(db, n_queries, sms), free_shape, db.warps_only};
+    if (mode == 0) return {config_for(db, n_queries, sms), free_shape, db.warps_only_n == n_queries};
     const uint32_t words = db.stride / 16;
     return {add_config(db.cfg_set ? db.cfg : default_add_config(db.n, words, n_queries, sms), words), free_shape, true};
 }
@@ -807,7 +807,8 @@ impir_status impir_get_config_add32(int32_t h, uint32_t n_queries, impir_config*
     return IMPIR_OK;
 }
 
-static impir_status set_config(int32_t h, const impir_config* cfg, bool tuned, bool warps_only = false) {
+// warps_only_n: see Db
+static impir_status set_config(int32_t h, const impir_config* cfg, bool tuned, uint32_t warps_only_n = 0) {
     if (!cfg) return fail(IMPIR_EINVAL, "NULL argument");
     std::lock_guard<std::mutex> lk(g_db_mu);
     if (h < 1 || size_t(h) > g_dbs.size() || !g_dbs[h - 1].live) return fail(IMPIR_EINVAL, "unknown database handle %d", h);
@@ -815,7 +816,7 @@ static impir_status set_config(int32_t h, const impir_config* cfg, bool tuned, b
     g_dbs[h - 1].cfg = *cfg;
     g_dbs[h - 1].cfg_set = true;
     g_dbs[h - 1].cfg_tuned = tuned;
-    g_dbs[h - 1].warps_only = warps_only;
+    g_dbs[h - 1].warps_only_n = warps_only_n;
     return IMPIR_OK;
 }
 
@@ -834,7 +835,7 @@ impir_status impir_autotune(int32_t h, const uint8_t* d_keys, const uint32_t* d_
         auto it = g_tune.find(key);
         if (it != g_tune.end()) {
             if (best) *best = it->second.c;
-            return set_config(h, &it->second.c, true, it->second.warps_only);
+            return set_config(h, &it->second.c, true, it->second.warps_only ? n : 0);
         }
     }
     const impir_config base = default_config(db.n, db.stride / 16, n, dev->sms);
@@ -897,7 +898,7 @@ impir_status impir_autotune(int32_t h, const uint8_t* d_keys, const uint32_t* d_
         g_tune[key] = found;
     }
     if (best) *best = found.c;
-    return set_config(h, &found.c, true, found.warps_only);
+    return set_config(h, &found.c, true, found.warps_only ? n : 0);
 }
 
 // ---- databases larger than HBM: streamed in chunks (§3.3) ----

@@ -44,9 +44,10 @@ class Batch:
     def tuned(self):
         return impir.impir_autotune(*self.args)
 
-    def answer(self):
+    def answer(self, n=None):
         """The answers, and the units of the tensor-core kernel (header bytes 48 to 55)."""
-        impir.impir_answer_async(*self.args)
+        args = self.args if n is None else self.args[:3] + (n,) + self.args[4:]
+        impir.impir_answer_async(*args)
         return self.out.cpu().numpy().copy(), int(self.ws[48:56].cpu().numpy().view("<u8")[0])
 
 
@@ -63,6 +64,7 @@ def test_tuned_batches_run_what_was_timed(tmp_path):
             assert b.tuned().as_dict() == dict(lane_bits=4, queries_per_warp=4, warps_per_cta=16, queries_per_launch=0)
             got, units = b.answer()
             assert units == expect and np.array_equal(got, want)
+            assert b.answer(Q - 1)[1] == N // 1024      # a batch size that was not timed: the default rule
         impir.impir_set_config(b.h, lane_bits=4, queries_per_warp=4)     # set, not tuned: as it is
         got, units = b.answer()
         assert units == 0 and np.array_equal(got, want)
