@@ -220,13 +220,13 @@ def peaks():
 # schedule 40, round 1 of both children 17, rounds 2-9 256, final rounds 32), a pair at the
 # leaf level 288 (key schedule 36, round 1 17, rounds 2-8 224, column 0 of round 9 8, the
 # three S-box lookups the selection bits need 3). A domain of 2^m leaves has 2^(m-1) leaf-level
-# pairs and 2^(m-1) - 1 internal ones: 158.25 lookups per AES block on average. These counts are the
-# roofline's fixed basis, the engine without sharing between the two blocks beyond round 1; the
-# kernels now execute 329 and 270 (round 2 and the first key step shared, the leaf's last key steps cut
-# down to the bytes its bit needs), 149.75 per block, so a fraction of this peak can exceed 1 by 5.7 %.
+# pairs and 2^(m-1) - 1 internal ones: 158.25 lookups per AES block on average. That is the engine with
+# nothing shared between the two blocks beyond round 1. The kernels execute 329 and 270 (round 2 and the
+# first key step shared, the leaf's last key steps cut down to the bytes its bit needs; additive leaf
+# pairs 305), 149.75 per block: the roofline is taken at these.
 LOOKUPS_INTERNAL_PAIR = 345
 LOOKUPS_LEAF_PAIR = 288
-LOOKUPS_EXECUTED_PAIR = 329   # what the isolated engine and the kernels execute per internal pair
+EXECUTED_INTERNAL_PAIR, EXECUTED_LEAF_PAIR, EXECUTED_LEAF_PAIR_ADD = 329, 270, 305
 # the additive answer's leaf-level pair: the low 32 bits of both leaves (key schedule 36, round 1
 # 17, rounds 2-9 256, column 0 of round 10 and its round-key word 12)
 LOOKUPS_LEAF_PAIR_ADD = 321
@@ -236,6 +236,11 @@ SMEM_LOOKUPS_PER_CLK_PER_SM = 32   # one 32-bit word per bank per clock, 32 bank
 def lookups_per_query(m: int, leaf_pair: int = LOOKUPS_LEAF_PAIR) -> int:
     half = 1 << (m - 1)
     return leaf_pair * half + LOOKUPS_INTERNAL_PAIR * (half - 1)
+
+
+def executed_lookups(m: int, leaf_pair: int = EXECUTED_LEAF_PAIR) -> int:
+    half = 1 << (m - 1)
+    return leaf_pair * half + EXECUTED_INTERNAL_PAIR * (half - 1)
 
 
 def smem_peak_gaes(sms: int, mhz: float, lookups_per_block: float) -> float:
@@ -472,9 +477,9 @@ def main():
     nq = sum(bt["n"] for bt in batches)
     stream = torch.cuda.Stream()
 
-    def run_step(server=0):
+    def run_step(server=0, handle=dbh):
         for bt in batches:
-            impir.impir_answer_async(dbh, bt["d_keys%d" % server], bt["d_off"], bt["n"], bt["d_out"], bt["d_ws"],
+            impir.impir_answer_async(handle, bt["d_keys%d" % server], bt["d_off"], bt["n"], bt["d_out"], bt["d_ws"],
                                      bt["wsb"], stream)
 
     # autotune on the largest batch (outside the timed region)
@@ -495,6 +500,11 @@ def main():
     run_step(0)
     stream.synchronize()
     ans0 = [bt["d_out"].cpu().numpy().copy() for bt in batches]
+    # which kernels had work in each batch, from the workspace headers (bytes 8 and 48: units)
+    kernels = []
+    for bt in batches:
+        hdr = bt["d_ws"][:56].cpu().numpy().view("<u8")
+        kernels.append([k for k, units in (("fused_tc_kernel", hdr[6]), ("fused_kernel", hdr[1])) if units])
     bad = 0
     for bt, a0, a1 in zip(batches, ans0, ans1):
         for i, (m, a) in enumerate(zip(bt["ms"], bt["alphas"])):
@@ -564,25 +574,26 @@ def main():
     # ---- plain form: one query per launch on the same queries ----
     plain = None
     if not args.no_plain:
-        impir.impir_set_config(dbh, cfg["lane_bits"], 1, cfg["warps_per_cta"], 1)
-        pc = impir.impir_get_config(dbh, 1).as_dict()
-        run_step()
+        ph = impir.impir_db_attach(impir.impir_db_info(dbh)["d_records"], N, B, stride)   # a handle of its own shape
+        impir.impir_set_config(ph, cfg["lane_bits"], 1, cfg["warps_per_cta"], 1)
+        pc = impir.impir_get_config(ph, 1).as_dict()
+        run_step(handle=ph)
         stream.synchronize()
         p0, p1 = torch.cuda.Event(enable_timing=True), torch.cuda.Event(enable_timing=True)
         p0.record(stream)
-        run_step()
+        run_step(handle=ph)
         p1.record(stream)
         p1.synchronize()
         pms = p0.elapsed_time(p1)
         same = all(np.array_equal(bt["d_out"].cpu().numpy(), a) for bt, a in zip(batches, ans0))
         plain = {"value": nq / (pms / 1e3), "unit": "queries/s", "config": pc, "bit_identical_to_batched": same}
-        impir.impir_set_config(dbh, cfg["lane_bits"], cfg["queries_per_warp"], cfg["warps_per_cta"], 0)
+        impir.impir_db_free(ph)
 
     # ---- roofline of the dominant kernel (fused EvalAll + dpXOR) ----
     pk, pk_kind = peaks()
     mhz = clocks.get("sm_mhz") or pk.get("sm_max_mhz", 2070.0)
     blocks_per_step = sum(aes_blocks(m) for bt in batches for m in bt["ms"])
-    lookups_per_step = sum(lookups_per_query(m) for bt in batches for m in bt["ms"])
+    lookups_per_step = sum(executed_lookups(m) for bt in batches for m in bt["ms"])
     lookups_per_block = lookups_per_step / blocks_per_step
     launch_ms = fused_ms / max(1, fused_launches)
     achieved = blocks_per_step * args.steps / (fused_ms / 1e3) / 1e9 if fused_ms else None
@@ -590,18 +601,26 @@ def main():
     scan_bytes = sum(min(N, 1 << m) * B for bt in batches for m in bt["ms"])
     # the integer-ALU form of the same bound: AES blocks x the engine's ALU-pipe instructions
     # per block (ncu, isolated engine, scaled from its internal-node pairs to the kernel's mix
-    # of internal and leaf pairs by lookups) + one 32-bit mask-and-XOR per record word and query
-    # of the scan, over the ALU pipe's lanes x SMs x clock
+    # of internal and leaf pairs by lookups) + the scan's operations per 32-bit record word: one
+    # mask-and-XOR per query in the warp kernels, nine per group of at most 128 queries on the
+    # tensor cores, over the ALU pipe's lanes x SMs x clock
     alu = None
     ac = alu_counts()
     if ac and fused_ms:
-        xor_ops = sum(min(N, 1 << m) * (stride // 4) for bt in batches for m in bt["ms"])
+        scan_ops = 0
+        for bt, ks in zip(batches, kernels):
+            lo = 0
+            for m in sorted(set(bt["ms"])):    # records that the domains from 2^m on reach beyond the smaller ones
+                hi, active = min(N, 1 << m), sum(x >= m for x in bt["ms"])
+                on_tc = "fused_tc_kernel" in ks and active >= 64
+                scan_ops += (hi - lo) * (stride // 4) * (9 * -(-active // 128) if on_tc else active)
+                lo = hi
         per_block = ac["engine_alu_thread_inst_per_block"] * lookups_per_block / ac["engine_lookups_per_block"]
-        ops = blocks_per_step * per_block + xor_ops
+        ops = blocks_per_step * per_block + scan_ops
         alu_peak = sms * ac["alu_lanes_per_sm_per_clk"] * mhz * 1e6
         alu = {"bound": "alu", "achieved": ops * args.steps / (fused_ms / 1e3) / 1e12, "peak": alu_peak / 1e12,
                "unit": "T int-ops/s", "frac": ops * args.steps / alu_peak / (fused_ms / 1e3),
-               "ops_per_step": ops, "aes_ops_per_block": per_block, "scan_xor_ops_per_step": xor_ops,
+               "ops_per_step": ops, "aes_ops_per_block": per_block, "scan_ops_per_step": scan_ops,
                "basis": f"{sms} SMs x {ac['alu_lanes_per_sm_per_clk']} ALU lanes/clk x {mhz:.0f} MHz; "
                         f"engine {ac['engine_alu_thread_inst_per_block']:.1f} ALU ops per block "
                         f"({ac['source']})"}
@@ -611,7 +630,7 @@ def main():
     cal = calibrate_engines(impir)
     engine_gaes = cal["ttable_keyed"]["gaes_per_s"]
     engine = {"gaes_per_s": engine_gaes,
-              "lookups_per_clk_per_sm": engine_gaes * 1e9 * LOOKUPS_EXECUTED_PAIR / 2 / (sms * mhz * 1e6),
+              "lookups_per_clk_per_sm": engine_gaes * 1e9 * EXECUTED_INTERNAL_PAIR / 2 / (sms * mhz * 1e6),
               "fused_over_engine": (achieved / engine_gaes) if achieved else None,
               "engines": {k: v["gaes_per_s"] for k, v in cal.items()},
               "note": "keyed T-table node expansions in registers, 164.5 table lookups per block (rounds 1 "
@@ -715,7 +734,7 @@ def main():
         rec = s32.astype("<u4").view(np.uint8).reshape(len(sub), B)
         ok = sum(int(np.array_equal(rec[i], db[a])) for i, a in enumerate(al))
         add_blocks = sum(aes_blocks(bt["ms"][i]) for bt, i in sub)
-        add_lookups = sum(lookups_per_query(bt["ms"][i], LOOKUPS_LEAF_PAIR_ADD) for bt, i in sub)
+        add_lookups = sum(executed_lookups(bt["ms"][i], EXECUTED_LEAF_PAIR_ADD) for bt, i in sub)
         add_peak = smem_peak_gaes(sms, mhz, add_lookups / add_blocks)
         additive = {"queries": len(sub), "add32_queries_per_s": len(sub) / t_add, "xor_queries_per_s": len(sub) / t_xor,
                     "reconstructed_ok": ok, "launch": impir.impir_get_config_add32(dbh, len(sub)).as_dict(),
@@ -723,7 +742,7 @@ def main():
                     "aes_gaes_per_s": add_blocks / t_add / 1e9,
                     "frac_of_peak": add_blocks / t_add / 1e9 / add_peak,
                     "peak_basis": f"{add_lookups / add_blocks:.2f} lookups per AES block (leaf-level pairs "
-                                  f"{LOOKUPS_LEAF_PAIR_ADD})"}
+                                  f"{EXECUTED_LEAF_PAIR_ADD})"}
 
     # the fixed-key PRF variant (Matyas-Meyer-Oseas with two fixed AES keys: no key schedule
     # per node, but no round shared between the two children) on the largest batch, against the
@@ -763,6 +782,9 @@ def main():
         try:
             for hh in hs:
                 impir.impir_set_config(hh, **{k: cfg[k] for k in ("lane_bits", "queries_per_warp", "warps_per_cta")})
+            wh = impir.impir_db_attach(impir.impir_db_info(dbh)["d_records"], N, B, stride)
+            hs.append(wh)      # the whole database in the shards' shape, warp kernels as there
+            impir.impir_set_config(wh, **{k: cfg[k] for k in ("lane_bits", "queries_per_warp", "warps_per_cta")})
             nb, d_keys, d_off, d_ws, wsb = big["n"], big["d_keys0"], big["d_off"], big["d_ws"], big["wsb"]
             parts = torch.zeros((2, nb, B), dtype=torch.uint8, device="cuda")
             whole = torch.zeros((nb, B), dtype=torch.uint8, device="cuda")
@@ -772,7 +794,7 @@ def main():
             with torch.cuda.stream(st):
                 for rep in range(3):
                     ev[0].record(st)
-                    impir.impir_answer_async(dbh, d_keys, d_off, nb, whole, d_ws, wsb, st)
+                    impir.impir_answer_async(wh, d_keys, d_off, nb, whole, d_ws, wsb, st)
                     ev[1].record(st)
                     impir.impir_answer_async(hs[0], d_keys, d_off, nb, parts[0], d_ws, wsb, st)
                     ev[2].record(st)
@@ -849,10 +871,11 @@ def main():
                          "frac": (achieved / peak) if achieved else None,
                          "traffic": traffic,
                          "peak_basis": f"{sms} SMs x {mhz:.0f} MHz x {SMEM_LOOKUPS_PER_CLK_PER_SM} table lookups/clk"
-                                       f" / {lookups_per_block:.2f} lookups per AES block (fixed basis: "
-                                       f"{LOOKUPS_INTERNAL_PAIR} per internal node pair, {LOOKUPS_LEAF_PAIR} per "
-                                       f"leaf-level pair; the kernels execute {LOOKUPS_EXECUTED_PAIR} and 270)",
-                         "kernel": "fused_kernel", "avg_launch_ms": launch_ms, "launches": fused_launches},
+                                       f" / {lookups_per_block:.2f} lookups per AES block as executed "
+                                       f"({EXECUTED_INTERNAL_PAIR} per internal node pair, {EXECUTED_LEAF_PAIR} per "
+                                       f"leaf-level pair)",
+                         "kernel": " + ".join(sorted({k for ks in kernels for k in ks}, reverse=True)),
+                         "kernels_per_batch": kernels, "avg_launch_ms": launch_ms, "launches": fused_launches},
             "roofline_alu": alu,
             "scan": {"logical_gbs": scan_bytes * args.steps / (ms / 1e3) / 1e9,
                      # DRAM bytes of one fused launch (ncu capture) over its live duration
