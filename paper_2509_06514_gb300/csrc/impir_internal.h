@@ -188,7 +188,7 @@ inline SmemSplit split_smem(uint32_t warps, size_t slice) {
 //             the port for 32 nodes (1.3 pairs' time each in the steady state); the fifth level 0.8 pairs
 //             per query and lane. The additive answer's lanes walk all five (0.65 each for the four more)
 //   scan      per 16-byte word 4.3 operations for each query and 4 (additive: 14, with its share loads) for
-//             all of them, in pairs of 560 ALU operations (282 per block); 900 for a round of record loads
+//             all of them, in pairs of 560 ALU operations; 900 for a round of record loads
 //   memory    3300 bytes a clock from HBM (6.8 TB/s), of which n warps per SM draw 400 n, twice that where
 //             the reads of one unit pass under another's lookups; 5000 from L2, where groups read a tile
 //             again; L2 holds the tiles in work up to 64 MB, none of them from 256 MB
