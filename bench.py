@@ -185,12 +185,12 @@ def kernel_source_hash() -> str:
     return h.hexdigest()
 
 
-def captured_traffic(cfg: dict, batches: list):
+def captured_traffic(cfg: dict, batches: list, kernels: list = None):
     """DRAM bytes per fused launch of this step, from the committed ncu capture of the same
     batches on a smaller database (1 GiB; the full-size workload is too large to capture with
     more than the launch-time metric): each batch's measured DRAM bytes per byte of the DB prefix
     its queries cover, times that prefix here, averaged over the step's launches. Valid only for
-    the kernel source and launch shape the capture was taken with; else None."""
+    the kernel source, launch shape and kernels the capture was taken with; else None."""
     try:
         with open(os.path.join(ROOT, "profiles", "fused_kernel_traffic.json")) as f:
             t = json.load(f)
@@ -199,6 +199,8 @@ def captured_traffic(cfg: dict, batches: list):
     if t.get("kernel_source_sha256") != kernel_source_hash() or t.get("launch") != cfg:
         return None
     per = t.get("per_batch", [])
+    if kernels is not None and [b.get("kernels") for b in per] != kernels:
+        return None
     if [b["queries"] for b in per] != [bt["n"] for bt in batches]:
         return None
     total = 0.0
@@ -862,7 +864,7 @@ def main():
         serving = run_serving(args, impir, workloads)
 
     if rank == 0:
-        traffic = captured_traffic(cfg, batches)
+        traffic = captured_traffic(cfg, batches, kernels)
         out = {
             "metric": "PIR queries/s (DPF eval+dpXOR) at 8 GiB DB", "value": value, "unit": "queries/s",
             "n_gpus": world, "steps": args.steps, "warmup": args.warmup, "ms_per_step": ms / args.steps,

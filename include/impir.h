@@ -230,7 +230,7 @@ impir_status impir_get_config_add32(int32_t db_handle, uint32_t n_queries, impir
  * this database, writes it to *best and records it in the process-wide tuning cache
  * keyed by (SM count, N, stride, batch size). Where the tensor-core kernel may take tiles of the
  * batch, the launch with it is timed too, and later batches of this size keep to the warp kernels
- * if they alone were faster (of other sizes, for which that was not timed, they follow the default
+ * if they alone were faster by more than 1 % (of other sizes, for which that was not timed, they follow the default
  * rule). Synchronizes the stream. */
 impir_status impir_autotune(int32_t db_handle, const uint8_t* d_keys, const uint32_t* d_key_offsets,
                             uint32_t n_queries, uint8_t* d_out, void* d_workspace, size_t workspace_bytes,

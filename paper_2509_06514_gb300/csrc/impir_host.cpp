@@ -879,17 +879,12 @@ impir_status impir_autotune(int32_t h, const uint8_t* d_keys, const uint32_t* d_
             found.c = c;
         }
     }
-    // Where the tensor-core kernel may take tiles of the batch it stays only if that is faster than the
-    // fastest warp shape; the shape beside it (the tiles that few queries reach) is that one or the default.
+    // Where the tensor-core kernel may take tiles of the batch it stays unless the fastest warp shape, which
+    // keeps the tiles that few queries reach, is faster without it by more than 1 % (more than one launch
+    // differs from the next).
     if (xor_shape(found.c, true, db.n, db.stride / 16, n, dev->sms).tc) {
-        found.warps_only = true;
-        for (const impir_config& c : {found.c, base}) {
-            if (impir_status s = time_ms(c, false, &ms)) return s;
-            if (ms < best_ms) {
-                best_ms = ms;
-                found = {c, false};
-            }
-        }
+        if (impir_status s = time_ms(found.c, false, &ms)) return s;
+        found.warps_only = ms > best_ms * 1.01f;
     }
     cudaEventDestroy(e0);
     cudaEventDestroy(e1);
