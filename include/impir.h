@@ -414,7 +414,9 @@ impir_status impir_aes_calibrate_bitsliced(uint32_t iters, uint32_t n_threads, u
  * clears the record. EINVAL in a library built without IMPIR_BOUNDS. For testing the checks
  * themselves, the debug library reads IMPIR_BOUNDS_TEST_WITHHOLD_RECORDS=k from the environment
  * and withholds the last k records of every database from the checked extent (their memory stays
- * valid), so that reads of them fail the check; the normal library ignores it. */
+ * valid), so that reads of them fail the check; IMPIR_BOUNDS_TEST_WAIT_NS=t, the limit of the tensor-core
+ * kernel's waits in nanoseconds; and IMPIR_BOUNDS_TEST_NO_TABLES, with which the fused kernels refuse to
+ * run. The normal library ignores all three. */
 impir_status impir_bounds_status(uint32_t* n_failed, uint32_t* first_site, uint64_t* first_index);
 
 /* Number of streaming multiprocessors of the current device (0 if none). */
